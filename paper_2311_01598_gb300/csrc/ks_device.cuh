@@ -6,6 +6,8 @@
 //     The NTT butterflies use an estimate of that quotient built from three
 //     of the four 32x32-bit partial products of a*w' (shoup_est), which
 //     widens the range to [0, 4q) and saves a full 64x64 high product.
+//     Prime sets just below a power of two take a cheaper product without a
+//     quotient (AR_PM below).
 //   * Lazy butterflies (after Harvey): the forward (Cooley-Tukey) butterfly
 //     lets values grow by at most 4q per stage and is reduced once at the
 //     end; the inverse (Gentleman-Sande) one keeps them in [0, 4q).
@@ -89,22 +91,133 @@ __device__ __forceinline__ u64 shoup_est_sp(u64 a, u64 w, u64 wp, u64 q)
     return ((((u64)hi) << 32) | (u32)lo) - e;
 }
 
-// Forward NTT outputs before the final reduction are below kFwdLazy * q:
-// inputs below 4q grow by less than 4q per stage, 4q + 17*4q = 72q for the
-// 17 stages of N = 2^17, and 76q < 2^63 for q < 2^56.
-constexpr u64 kFwdLazy = 72;
+// ------------------------------------------------------------------ butterfly arithmetic
+// The NTT kernels are instantiated for one of three forms of the butterfly's
+// product by a twiddle, chosen by the parameter set's primes (Tables::arith):
+//   AR_GEN  any prime: Shoup product with the estimated quotient (28 cycles
+//           of the 32-bit multiply pipe a warp: six 32x32->64 or high
+//           products and four low ones);
+//   AR_SP   every prime k*2^32 + 1: one low product fewer (shoup_est_sp);
+//   AR_PM   every prime just below a power of two, q = 2^b - c with c small
+//           (the default prime rule: the largest primes below 2^bits that
+//           are 1 mod 2N, so c is a few hundred times 2N): five 32x32->64
+//           products and no quotient at all.
+//
+// AR_PM product.  A twiddle w is stored with w2 = w*2^32 mod q, each cut at
+// bit k = b - 31 into a low and a high part (below 2^k and 2^31).  For any
+// 64-bit a = a1*2^32 + a0,
+//   a*w == a0*w + a1*w2 = M0 + M1*2^k (mod q),
+//   M0 = a0*wl + a1*w2l < 2^(b+2),  M1 = a0*wh + a1*w2h < 2^64,
+// and with M1 = h*2^32 + r the top part h*2^(k+32) = h*2^(b+1) == h*c2,
+// c2 = 2^(b+1) - 2q = 2c.  So t = M0 + r*2^k + h*c2 is congruent to a*w and
+// below 2^33 c + 6*2^b (2^60 at 54 bits and N = 2^16), without a comparison
+// or a quotient estimate; every word boundary falls on a register.  Values
+// are kept lazily below 2^64 and folded, x -> (x mod 2^(b+1)) +
+// (x >> (b+1)) c2, only where the next stages could carry past it (host
+// bounds per parameter set: pm_plan in ks_host.cpp).
+// Register-only loops of 16 values (4 stages, twiddles from shared memory)
+// on a GB300: 39 cycles of a scheduler per warp butterfly for AR_GEN, 29-30
+// for AR_PM.
+
+// The constants of one modulus that a transform keeps in registers.
+template <int AR> struct ModR {
+    u64 q;
+};
+template <> struct ModR<AR_PM> {
+    u64 off;  // a multiple of q at least as large as what is subtracted (forward: any product; inverse: any value)
+    u32 c2;   // 2^(b+1) - 2q
+    u32 k;    // b - 31
+};
+template <int AR> __device__ __forceinline__ ModR<AR> mod_fwd(const ModC &mc)
+{
+    if constexpr (AR == AR_PM)
+        return ModR<AR>{mc.pm_T, mc.pm_c2, mc.pm_k};
+    else
+        return ModR<AR>{mc.q};
+}
+template <int AR> __device__ __forceinline__ ModR<AR> mod_inv(const ModC &mc)
+{
+    if constexpr (AR == AR_PM)
+        return ModR<AR>{mc.pm_D, mc.pm_c2, mc.pm_k};
+    else
+        return ModR<AR>{mc.q};
+}
+// 32x32->64 products and multiply-adds, one instruction each (the C form of
+// a sum of them is not always compiled to the accumulating instruction).
+__device__ __forceinline__ u64 mul_wide(u32 a, u32 b)
+{
+    u64 r;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ u64 mad_wide(u32 a, u32 b, u64 c)
+{
+    u64 r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+// a * w mod q, lazily, W = (w2l | wl << 32, w2h | wh << 32).  WIDE: r*2^k is
+// accumulated by a sixth multiply-add instead of two shifts and an addition:
+// fewer instructions for one more on the multiply pipe, which suits the
+// inverse passes (their butterflies have more additions: 205 -> 192 and 220 ->
+// 214 us for 640 limbs of 2^16) and not the forward ones (494 -> 509 us for
+// 1920 limbs).
+template <bool WIDE = false>
+__device__ __forceinline__ u64 pm_mul(u64 a, const ulonglong2 &W, u32 c2, u32 k)
+{
+    const u32 a0 = (u32)a, a1 = (u32)(a >> 32);
+    const u64 M1 = mad_wide(a1, (u32)W.y, mul_wide(a0, (u32)(W.y >> 32)));
+    u64 M0;
+    if constexpr (WIDE)
+        M0 = mad_wide(a1, (u32)W.x, mad_wide(a0, (u32)(W.x >> 32), mul_wide((u32)M1, 1u << k)));
+    else
+        M0 = mad_wide(a1, (u32)W.x, mul_wide(a0, (u32)(W.x >> 32)));
+    const u64 t = mad_wide((u32)(M1 >> 32), c2, M0);
+    return WIDE ? t : t + ((u64)(u32)M1 << k);
+}
+// Any 64-bit x -> below 2^(b+1) + 2^(63-b) c2, the same residue.
+__device__ __forceinline__ u64 pm_fold(u64 x, u32 c2, u32 k)
+{
+    const u32 hi = (u32)(x >> 32);
+    return mad_wide(hi >> k, c2, ((u64)(hi & ((1u << k) - 1)) << 32) | (u32)x);
+}
+// Any 64-bit x -> [0, q): the fold at 2^b leaves it below 2q.
+__device__ __forceinline__ u64 pm_canon(u64 x, u64 q, u32 c2, u32 k)
+{
+    const u32 hi = (u32)(x >> 32);
+    const u64 r = mad_wide(hi >> (k - 1), c2 >> 1, ((u64)(hi & ((1u << (k - 1)) - 1)) << 32) | (u32)x);
+    return r >= q ? r - q : r;
+}
+template <int AR> __device__ __forceinline__ u64 fold(u64 x, const ModR<AR> &m)
+{
+    if constexpr (AR == AR_PM)
+        return pm_fold(x, m.c2, m.k);
+    else
+        return x;
+}
+// Forward NTT outputs of the AR_GEN and AR_SP forms before the final
+// reduction are below kFwdLazy * q: inputs below 4q grow by less than 4q per
+// stage, 4q + 17*4q = 72q for the 17 stages of N = 2^17, and 76q < 2^63 for
+// q < 2^56 (kFwdLazy = 72).  ModC::flz holds the bound of the set's own form (a
+// multiple of q; flz + q < 2^64).
 
 // Forward Cooley-Tukey butterfly without a per-stage correction of X: with
 // X, Y < B the outputs are below B + 4q (the estimated Shoup product is below
 // 4q for any 64-bit Y), so a transform of at most 17 stages fed with values
-// below 4q ends below kFwdLazy*q.  Consumers reduce with reduce_any.  SP:
-// the modulus has the special form (shoup_est_sp).
-template <bool SP = false>
-__device__ __forceinline__ void fwd_bfly(u64 &X, u64 &Y, u64 w, u64 wp, u64 q, u64 q2)
+// below 4q ends below kFwdLazy*q.  AR_PM adds less than off (pm_T) a stage.
+// Consumers reduce with reduce_any.
+template <int AR>
+__device__ __forceinline__ void fwd_bfly(u64 &X, u64 &Y, const ulonglong2 &W, const ModR<AR> &m)
 {
-    const u64 t = SP ? shoup_est_sp(Y, w, wp, q) : shoup_est(Y, w, wp, 0 - q);
-    Y = X + (q2 + q2) - t;
-    X = X + t;
+    if constexpr (AR == AR_PM) {
+        const u64 t = pm_mul(Y, W, m.c2, m.k);
+        Y = X + m.off - t;
+        X = X + t;
+    } else {
+        const u64 t = AR == AR_SP ? shoup_est_sp(Y, W.x, W.y, m.q) : shoup_est(Y, W.x, W.y, 0 - m.q);
+        Y = X + 4 * m.q - t;
+        X = X + t;
+    }
 }
 
 // Any 64-bit x -> [0, q): Shoup product by 1 (into [0, 2q)), one correction.
@@ -114,18 +227,37 @@ __device__ __forceinline__ u64 reduce_any(u64 x, u64 q, u64 one_sh)
     return r >= q ? r - q : r;
 }
 
-// Inverse Harvey butterfly on [0, 4q): X, Y in [0, 4q) -> [0, 4q) (the sum
-// below 8q takes one conditional subtraction of 4q; the difference plus 4q
-// is below 8q and its estimated Shoup product below 4q).
-template <bool SP = false>
-__device__ __forceinline__ void inv_bfly(u64 &X, u64 &Y, u64 w, u64 wp, u64 q, u64 q2)
+// Inverse butterfly.  AR_GEN, AR_SP: Harvey's on [0, 4q): X, Y in [0, 4q) ->
+// [0, 4q) (the sum below 8q takes one conditional subtraction of 4q; the
+// difference plus 4q is below 8q and its estimated Shoup product below 4q).
+// AR_PM: X, Y at most off; the sum is folded when FOLD (see inv_fold).
+template <int AR>
+__device__ __forceinline__ void inv_bfly(u64 &X, u64 &Y, const ulonglong2 &W, const ModR<AR> &m, bool fold_sum)
 {
-    const u64 q4 = q2 + q2;
-    u64 s = X + Y;
-    s = s >= q4 ? s - q4 : s;
-    const u64 d = X - Y + q4;
-    X = s;
-    Y = SP ? shoup_est_sp(d, w, wp, q) : shoup_est(d, w, wp, 0 - q);
+    if constexpr (AR == AR_PM) {
+        const u64 s = X + Y;
+        const u64 d = X - Y + m.off;
+        X = fold_sum ? pm_fold(s, m.c2, m.k) : s;
+        Y = pm_mul<true>(d, W, m.c2, m.k);
+    } else {
+        const u64 q4 = 4 * m.q;
+        u64 s = X + Y;
+        s = s >= q4 ? s - q4 : s;
+        const u64 d = X - Y + q4;
+        X = s;
+        Y = AR == AR_SP ? shoup_est_sp(d, W.x, W.y, m.q) : shoup_est(d, W.x, W.y, 0 - m.q);
+    }
+}
+// AR_PM inverse rounds.  Entry values are folded (small: they may double at
+// every stage of a round); a product is below T, its first sum with another
+// below 2T, and the second such sum (below 4T < 2^64) is folded back.  In a
+// round's stage pairing registers k and k + half, both values were last a
+// product at the stage of k's highest set bit (the earlier stages pair bits
+// below half), so the sum is the second one exactly when bit half/4 of k is
+// set and bit half/2 is not: known at compile time.
+__device__ __forceinline__ constexpr bool inv_fold(int k, int half)
+{
+    return half >= 4 && (k & (half >> 2)) != 0 && (k & (half >> 1)) == 0;
 }
 
 // 128-bit accumulator.
@@ -322,10 +454,20 @@ template <> struct ShapeOf<16> { typedef Shape<8, 8> T; };
 template <> struct ShapeOf<17> { typedef Shape<9, 8> T; };
 
 // ------------------------------------------------------------------ rounds
+// Folds of a whole register set (AR_PM; nothing for the other forms).
+template <int R, int AR>
+__device__ __forceinline__ void fold_all(u64 (&x)[R], const ModR<AR> &m)
+{
+    if constexpr (AR == AR_PM) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) x[k] = fold<AR>(x[k], m);
+    }
+}
+
 // Round 1 in registers: x[k], k = the high RR bits of the sub-transform index.
 // tw(s, i) returns the (w, w') pair of local stage s, local group i.
-template <int RR, bool SP = false, class TW>
-__device__ __forceinline__ void fwd_round1(u64 (&x)[1 << RR], const TW &tw, u64 q, u64 q2)
+template <int RR, int AR, class TW>
+__device__ __forceinline__ void fwd_round1(u64 (&x)[1 << RR], const TW &tw, const ModR<AR> &m)
 {
 #pragma unroll
     for (int s = 0; s < RR; ++s) {
@@ -334,15 +476,17 @@ __device__ __forceinline__ void fwd_round1(u64 (&x)[1 << RR], const TW &tw, u64 
         for (int g = 0; g < (1 << s); ++g) {
             const ulonglong2 W = tw(s, g);
 #pragma unroll
-            for (int k = 0; k < half; ++k) fwd_bfly<SP>(x[g * 2 * half + k], x[g * 2 * half + k + half], W.x, W.y, q, q2);
+            for (int k = 0; k < half; ++k) fwd_bfly<AR>(x[g * 2 * half + k], x[g * 2 * half + k + half], W, m);
         }
     }
 }
 
-// Round 2 in registers: NG groups of M = 2^(L-RR) values; group gg has
-// global group id gid0 + gg (the high RR bits of the index).
-template <int L, int RR, bool SP = false, class TW>
-__device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int gid0, const TW &tw, u64 q, u64 q2)
+// Round 2 in registers: NG groups of M = 2^(L-RR) values; group gg of thread
+// tau is group tau*NG + gg of the sub-transform (the high RR bits of the
+// index).  tw.r2(s, s2, tau, gg, g2) is the twiddle of stage s = RR + s2 and
+// sub-group g2 of that group.
+template <int L, int RR, int AR, class TW>
+__device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m)
 {
     constexpr int M = 1 << (L - RR);
     constexpr int NG = (1 << RR) / M;
@@ -353,18 +497,18 @@ __device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int gid0, const TW
         for (int gg = 0; gg < NG; ++gg) {
 #pragma unroll
             for (int g2 = 0; g2 < (1 << s2); ++g2) {
-                const ulonglong2 W = tw(RR + s2, ((gid0 + gg) << s2) + g2);
+                const ulonglong2 W = tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
 #pragma unroll
                 for (int k = 0; k < half; ++k)
-                    fwd_bfly<SP>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W.x, W.y, q, q2);
+                    fwd_bfly<AR>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W, m);
             }
         }
     }
 }
 
 // Inverse of fwd_round2: local stages L-1 .. RR on the low bits.
-template <int L, int RR, bool SP = false, class TW>
-__device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int gid0, const TW &tw, u64 q, u64 q2)
+template <int L, int RR, int AR, class TW>
+__device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m)
 {
     constexpr int M = 1 << (L - RR);
     constexpr int NG = (1 << RR) / M;
@@ -375,18 +519,19 @@ __device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int gid0, const TW
         for (int gg = 0; gg < NG; ++gg) {
 #pragma unroll
             for (int g2 = 0; g2 < (1 << s2); ++g2) {
-                const ulonglong2 W = tw(RR + s2, ((gid0 + gg) << s2) + g2);
+                const ulonglong2 W = tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
 #pragma unroll
                 for (int k = 0; k < half; ++k)
-                    inv_bfly<SP>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W.x, W.y, q, q2);
+                    inv_bfly<AR>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W, m,
+                                 inv_fold(k, half));
             }
         }
     }
 }
 
 // Inverse of fwd_round1: local stages RR-1 .. 0 on the high bits.
-template <int RR, bool SP = false, class TW>
-__device__ __forceinline__ void inv_round1(u64 (&x)[1 << RR], const TW &tw, u64 q, u64 q2)
+template <int RR, int AR, class TW>
+__device__ __forceinline__ void inv_round1(u64 (&x)[1 << RR], const TW &tw, const ModR<AR> &m)
 {
 #pragma unroll
     for (int s = RR - 1; s >= 0; --s) {
@@ -395,36 +540,38 @@ __device__ __forceinline__ void inv_round1(u64 (&x)[1 << RR], const TW &tw, u64 
         for (int g = 0; g < (1 << s); ++g) {
             const ulonglong2 W = tw(s, g);
 #pragma unroll
-            for (int k = 0; k < half; ++k) inv_bfly<SP>(x[g * 2 * half + k], x[g * 2 * half + k + half], W.x, W.y, q, q2);
+            for (int k = 0; k < half; ++k)
+                inv_bfly<AR>(x[g * 2 * half + k], x[g * 2 * half + k + half], W, m, inv_fold(k, half));
         }
     }
 }
 
 // Twiddle fetchers.  Column pass: the first 2^LA entries of the tower's table,
-// staged in shared memory (G = 1).  Row pass: the forward row kernel stages
-// its rows' first-round twiddles in shared memory (TwStaged,
-// ks_ntt_core.cuh); TwRow reads straight from the tower's global table
-// (G = 2^LA + row).
+// staged in shared memory (G = 1).  Row pass (G = 2^LA + row): the first
+// round's entries are common to a row; those of the second round differ per
+// thread, and the table holds each row's of a stage in the order its threads
+// read them, position (g2*NG + gg)*TB + tau instead of ((tau*NG + gg) << s2)
+// + g2 (tw_pos, ks_host.cpp), so that a warp's load of one (gg, g2) covers
+// whole 256-byte pieces.  In the plain order a stage with 2^s2 sub-groups
+// made each load touch lines 2^s2 * 16 bytes apart, and the L1 pipeline, 90%
+// busy, bounded the row passes (1920 forward limbs of 2^16: 569 -> 494 us; 640
+// inverse ones: 250 -> 205 us).
 struct TwSmem {
     const ulonglong2 *t;
     __device__ __forceinline__ ulonglong2 operator()(int s, int i) const { return t[(1 << s) + i]; }
+    template <int NG> __device__ __forceinline__ ulonglong2 r2(int s, int s2, int tau, int gg, int g2) const
+    {
+        return t[(1 << s) + ((tau * NG + gg) << s2) + g2];
+    }
 };
+template <class S>
 struct TwRow {
     const ulonglong2 *t;  // tower table
     int G;
     __device__ __forceinline__ ulonglong2 operator()(int s, int i) const { return __ldg(t + (G << s) + i); }
-};
-// Same table, fetched with a volatile load: kernels that run several row
-// transforms of one tower in a loop would otherwise keep every twiddle of the
-// row live in registers across iterations.
-struct TwRowV {
-    const ulonglong2 *t;
-    int G;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int i) const
+    template <int NG> __device__ __forceinline__ ulonglong2 r2(int s, int, int tau, int gg, int g2) const
     {
-        ulonglong2 r;
-        asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(r.x), "=l"(r.y) : "l"(t + (G << s) + i));
-        return r;
+        return __ldg(t + (G << s) + (g2 * NG + gg) * S::TB + tau);
     }
 };
 

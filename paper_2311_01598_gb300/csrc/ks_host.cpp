@@ -142,6 +142,103 @@ static int upload(T **dst, const std::vector<T> &src)
     return KS_OK;
 }
 
+// Plan of the AR_PM butterflies (ks_device.cuh) for the moduli prim: per tower
+// the bit length b, c = 2^b - q and the bounds T (a lazy product) and D (a
+// value of an inverse round), and the forward folds the set needs.  The
+// transforms are followed stage by stage with exact bounds; use is false when
+// some value could reach 2^64 even with every fold, or a prime is not just
+// below a power of two.
+struct PmTower {
+    u64 c2, T, D, flz;
+    u32 k;
+};
+struct PmPlan {
+    bool use = false;
+    int fold = 0;
+    std::vector<PmTower> t;
+};
+static PmPlan pm_plan(const std::vector<u64> &prim, int logN)
+{
+    const u128 lim = (u128)1 << 64;
+    const int LA = logN - logN / 2, LB = logN / 2;  // column and row stages (ShapeOf)
+    const int RA = (LA + 1) / 2, RB = (LB + 1) / 2;  // stages of a pass's first round
+    for (int fold : {0, (int)PM_FOLD_ROW, PM_FOLD_ROW | PM_FOLD_MID}) {
+        PmPlan P;
+        P.fold = fold;
+        bool ok = true;
+        for (u64 q : prim) {
+            int b = 64 - __builtin_clzll(q);
+            if (b < 40 || b > kMaxPrimeBits) return PmPlan();
+            const u64 c = ((u64)1 << b) - q;
+            if (2 * c >= ((u64)1 << 32)) return PmPlan();
+            PmTower t;
+            t.c2 = 2 * c;
+            t.k = (u32)(b - 31);
+            const u128 word = 0xffffffffu, two_b1 = (u128)1 << (b + 1);
+            const u128 tmax = word * t.c2 + 2 * word * (((u64)1 << t.k) - 1) + (word << t.k);
+            const u128 T = (tmax + q - 1) / q * q;                       // any product is at most T
+            const u128 E = two_b1 + ((lim - 1) >> (b + 1)) * t.c2;       // any folded value is below E
+            const u128 full = ((u128)1 << b) + ((lim - 1) >> b) * c;     // pm_canon before its subtraction
+            // forward: a stage adds at most T
+            u128 B = 4 * (u128)q;
+            auto stages = [&](int n) {
+                B += n * T;
+                ok = ok && B < lim;
+            };
+            stages(RA);
+            if (fold & PM_FOLD_MID) B = E;
+            stages(LA - RA);
+            if (fold & PM_FOLD_ROW) B = E;
+            stages(RB);
+            if (fold & PM_FOLD_MID) B = E;
+            stages(LB - RB);
+            const u128 flz = (B + q - 1) / q * q;
+            // inverse: entry values (4q, then folded ones) double at most every
+            // stage of a round; products reach 2T before their sum is folded
+            u128 D = 2 * T;
+            const u128 ents[] = {(4 * (u128)q) << (LB - RB), E << RB, E << (LA - RA), E << RA};
+            for (u128 e : ents) D = D > e ? D : e;
+            D = (D + q - 1) / q * q;
+            ok = ok && 4 * T < lim && 2 * D < lim && flz + q < lim && full < 2 * (u128)q;
+            if (!ok) break;
+            t.T = (u64)T;
+            t.D = (u64)D;
+            t.flz = (u64)flz;
+            P.t.push_back(t);
+        }
+        if (ok) {
+            P.use = true;
+            return P;
+        }
+    }
+    return PmPlan();
+}
+
+// A twiddle or factor w of modulus q in AR_PM form: w and w*2^32 mod q, each
+// cut at bit k, the low parts in one word and the high parts in the other.
+static ulonglong2 pm_pair(u64 w, u64 q, u32 k)
+{
+    const u64 w2 = (u64)(((u128)w << 32) % q), mask = ((u64)1 << k) - 1;
+    return make_ulonglong2((w2 & mask) | ((w & mask) << 32), (w2 >> k) | ((w >> k) << 32));
+}
+
+// Position in the twiddle tables of entry i (bit-reversed order: stage m's
+// entries are [2^m, 2^(m+1))).  Entries of the column pass's stages and of the
+// row pass's first round stay in place; those of the row pass's second round
+// are laid out per row and stage in the order the row's threads read them
+// (TwRow, ks_device.cuh).
+static u64 tw_pos(u64 i, int logN)
+{
+    const int LA = logN - logN / 2, LB = logN / 2, RB = (LB + 1) / 2;
+    if (i < 2) return i;
+    const int s = 63 - __builtin_clzll(i) - LA;  // row-pass stage
+    if (s < RB) return i;
+    const int s2 = s - RB, TB = 1 << (LB - RB), NG = (1 << RB) / TB;
+    const u64 j = i & (((u64)1 << s) - 1);
+    const u64 gid = j >> s2, g2 = j & (((u64)1 << s2) - 1), tau = gid / NG, gg = gid % NG;
+    return (i - j) + (g2 * NG + gg) * TB + tau;
+}
+
 int build_tables(ks_params *P)
 {
     const int nt = P->nq + P->kp;
@@ -154,6 +251,12 @@ int build_tables(ks_params *P)
         P->psi[t] = find_psi(prim[t], P->logN);
         if (!P->psi[t]) return fail(KS_EINVAL, "no primitive 2N-th root for a prime");
     }
+
+    // butterfly form the primes allow
+    bool sp = true;
+    for (u64 q : prim) sp = sp && (q & 0xFFFFFFFFull) == 1;
+    const PmPlan pm = sp ? PmPlan() : pm_plan(prim, P->logN);
+    auto pair = [&](int t, u64 w) { return pm.use ? pm_pair(w, prim[t], pm.t[t].k) : shoup_pair(w, prim[t]); };
 
     // per-tower constants
     std::vector<ModC> modc(nt);
@@ -170,10 +273,21 @@ int build_tables(ks_params *P)
         m.r28_sh = shoup_h(m.r28, q);
         m.r56 = ((u64)1 << 56) % q;
         m.r56_sh = shoup_h(m.r56, q);
-        m.ninv = invmod_h(N % q, q);
-        m.ninv_sh = shoup_h(m.ninv, q);
+        const ulonglong2 ninv = pair(t, invmod_h(N % q, q));
+        m.ninv = ninv.x;
+        m.ninv_sh = ninv.y;
         u64 r64 = (u64)((((u128)1) << 64) % q);
         m.r2 = mulmod_h(r64, r64, q);
+        m.flz = kFwdLazy * q;
+        m.pm_T = m.pm_D = 0;
+        m.pm_c2 = m.pm_k = 0;
+        if (pm.use) {
+            m.flz = pm.t[t].flz;
+            m.pm_T = pm.t[t].T;
+            m.pm_D = pm.t[t].D;
+            m.pm_c2 = (u32)pm.t[t].c2;
+            m.pm_k = pm.t[t].k;
+        }
         m.pad = 0;
     }
 
@@ -190,8 +304,9 @@ int build_tables(ks_params *P)
         }
         for (u64 i = 0; i < N; ++i) {
             u64 r = brv(i, P->logN);
-            tw[(size_t)t * N + i] = shoup_pair(pw[r], q);
-            itw[(size_t)t * N + i] = shoup_pair(ipw[r], q);
+            const u64 at = (size_t)t * N + tw_pos(i, P->logN);
+            tw[at] = pair(t, pw[r]);
+            itw[at] = pair(t, ipw[r]);
         }
     }
 
@@ -213,7 +328,7 @@ int build_tables(ks_params *P)
                 for (int k = 0; k < a; ++k)
                     if (k != i) hat = mulmod_h(hat, prim[lo + k] % qi, qi);
                 u64 s = mulmod_h(invmod_h(N % qi, qi), invmod_h(hat, qi), qi);
-                pre.push_back(shoup_pair(s, qi));
+                pre.push_back(pair(lo + i, s));
             }
             for (int i = 0; i < a; ++i)
                 for (int t = 0; t < nt; ++t) {
@@ -356,9 +471,8 @@ int build_tables(ks_params *P)
     T.tc_below54 = 1;
     for (u64 q : P->q) T.tc_below54 = T.tc_below54 && q < (1ull << 54);
     for (u64 p : P->p) T.tc_below54 = T.tc_below54 && p < (1ull << 54);
-    T.spq = 1;
-    for (u64 q : P->q) T.spq = T.spq && (q & 0xFFFFFFFFull) == 1;
-    for (u64 p : P->p) T.spq = T.spq && (p & 0xFFFFFFFFull) == 1;
+    T.arith = pm.use ? AR_PM : sp ? AR_SP : AR_GEN;
+    T.pm_fold = pm.fold;
     T.logN = P->logN;
     T.nq = P->nq;
     T.kp = P->kp;

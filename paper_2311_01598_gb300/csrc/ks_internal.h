@@ -2,7 +2,7 @@
 //
 // Layout of everything the library keeps on the device (one parameter set):
 //   modc[t]          per-tower constants, t over the full basis q_0..q_L, p_0..p_{K-1}
-//   tw[t][N]         forward twiddles (w, floor(w*2^64/q)) in bit-reversed order:
+//   tw[t][N]         forward twiddles (w, floor(w*2^64/q), or an AR_PM pair) in bit-reversed order:
 //                    tw[t][i] = psi^brv(i) for the Cooley-Tukey NTT
 //   itw[t][N]        inverse twiddles psi^-brv(i) for the Gentleman-Sande iNTT
 //   up_pre[...]      ModUp P1 scale N^-1 * (Q_j/q_i)^-1 mod q_i per (digit, active
@@ -39,6 +39,13 @@ constexpr int kMaxLogN = 17;
 constexpr int kMaxPrimeBits = 56;  // 28-bit split products in BConv; 4q < 2^58 in the NTT
 constexpr int kSplit = 28;
 
+// Butterfly form of a parameter set's primes (ks_device.cuh), and the folds
+// its AR_PM forward transforms need: at the start of the row pass, and between
+// the two rounds of each pass.
+enum { AR_GEN = 0, AR_SP = 1, AR_PM = 2 };
+enum { PM_FOLD_ROW = 1, PM_FOLD_MID = 2 };
+constexpr u64 kFwdLazy = 72;  // AR_GEN, AR_SP: forward outputs are below kFwdLazy * q
+
 // Per-tower constants.
 struct ModC {
     u64 q;       // modulus
@@ -49,6 +56,12 @@ struct ModC {
     u64 r56, r56_sh;  // 2^56 mod q and its Shoup companion
     u64 ninv, ninv_sh;  // N^-1 mod q and its Shoup companion
     u64 r2;             // 2^128 mod q (into Montgomery form)
+    u64 flz;            // multiple of q no forward NTT output (lazy) exceeds; flz + q < 2^64
+    // q = 2^b - c just below a power of two (arith AR_PM, ks_device.cuh)
+    u64 pm_T;     // multiple of q no lazy product exceeds
+    u64 pm_D;     // multiple of q no value of an inverse round exceeds
+    u32 pm_c2;    // 2^(b+1) - 2q
+    u32 pm_k;     // b - 31
     u64 pad;
 };
 
@@ -78,7 +91,9 @@ struct Tables {
     const uint4 *dn_tc;
     int ntt_cluster;  // host side: NTTs as one cluster launch where supported
     int row_stage;    // host side: forward row passes staged by bulk copies (k_fwd_row_st)
-    int spq;          // every modulus is q1*2^32 + 1: two-pass NTTs use shoup_est_sp
+    int arith;        // butterfly form the primes allow (AR_GEN, AR_SP, AR_PM: ks_device.cuh); AR_PM sets hold
+                      // tw, itw, the ModUp P1 factors and N^-1 as AR_PM pairs instead of Shoup pairs
+    int pm_fold;      // AR_PM: folds the forward transforms need (PM_FOLD_*)
     int tc_below54;   // every modulus is below 2^54: 9-bit constant slices (tensor-core BConv)
     int logN;
     int nq, kp, alpha, ndig;

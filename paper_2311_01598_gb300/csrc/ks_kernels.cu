@@ -9,9 +9,9 @@
 namespace ks {
 
 // ------------------------------------------------------------------ NTT passes
-// Forward column pass (stages 0..LA-1).  grid (2^LB/COLS, limbs).  SP: every
-// modulus has the special form q1*2^32 + 1 (cheaper butterfly product).
-template <class S, bool SP>
+// Forward column pass (stages 0..LA-1).  grid (2^LB/COLS, limbs).  AR: the
+// butterfly form the set's primes allow (ks_device.cuh).
+template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, LimbMaps ms)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
     if (lg >= ms.pre[ms.n]) return;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
-    const u64 q = T.modc[L.tf].q, q2 = 2 * q;
+    const ModR<AR> md = mod_fwd<AR>(T.modc[L.tf]);
     const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
     for (int i = threadIdx.x; i < (1 << S::LA); i += S::THREADS_A) tws[i] = twt[i];
     const int cc = threadIdx.x % S::COLS, tau = threadIdx.x / S::COLS;
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
 #pragma unroll
     for (int k = 0; k < S::REGA; ++k) x[k] = L.src[((size_t)(k * S::TA + tau) << S::LB) + c];
     __syncthreads();
-    fwd_round1<S::RA, SP>(x, TwSmem{tws}, q, q2);
+    fwd_round1<S::RA, AR>(x, TwSmem{tws}, md);
 #pragma unroll
     for (int k = 0; k < S::REGA; ++k) sm[(k * S::TA + tau) * S::COLS + cc] = x[k];
     __syncthreads();
@@ -39,7 +39,8 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = sm[((tau * NG + gg) * M + k2) * S::COLS + cc];
-    fwd_round2<S::LA, S::RA, SP>(x, tau * NG, TwSmem{tws}, q, q2);
+    if (AR == AR_PM && (T.pm_fold & PM_FOLD_MID)) fold_all<S::REGA, AR>(x, md);
+    fwd_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
 // second shared-memory exchange returns the values to the first-round
 // layout; measured faster than storing each thread's consecutive values
 // with strided vector stores).
-template <class S, bool CANON, bool SP>
+template <class S, bool CANON, int AR>
 __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, LimbMaps ms)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, L
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
-    const u64 q = mc.q, q2 = 2 * q;
+    const ModR<AR> md = mod_fwd<AR>(mc);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
     const int G = (1 << S::LA) + h;
@@ -78,10 +79,9 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, L
     stage_row_round1<S>(tsh, twt, G, tau);
     static_assert(S::TB <= 32, "a row's threads share one warp");
     __syncwarp();
-    row_fwd_core<S, SP>(x, TwStaged<S>{tsh, twt, G}, sm + rr * S::ROWPAD, tau, q, q2);
-    const u64 one_sh = CANON ? mc.one_sh : 0;
+    row_fwd_core<S, AR>(x, TwStaged<S>{tsh, twt, G}, sm + rr * S::ROWPAD, tau, md, T.pm_fold);
 #pragma unroll
-    for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? reduce_any(x[k], q, one_sh) : x[k];
+    for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? canon_any<AR>(x[k], mc) : x[k];
 }
 
 // ------------------------------------------------------------------ staged row pass
@@ -146,7 +146,7 @@ __device__ __forceinline__ void staged_issue(const Tables &T, const LimbMaps &ms
 
 // 12 resident CTAs per SM (18 KB of shared memory each at 2^16): at most 85
 // registers a thread.
-template <class S, bool CANON>
+template <class S, bool CANON, int AR>
 __global__ void __launch_bounds__(S::THREADS_B, 12) k_fwd_row_st(Tables T, LimbMaps ms)
 {
     typedef StagedRow<S> SR;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(S::THREADS_B, 12) k_fwd_row_st(Tables T, LimbM
         phase ^= 1u << cur;
         const LimbRef L = limb_ref(ms, b / nblk, T.nq, T.alpha, S::LOGN);
         const ModC &mc = T.modc[L.tf];
-        const u64 q = mc.q, q2 = 2 * q;
+        const ModR<AR> md = mod_fwd<AR>(mc);
         const int h = (b % nblk) * S::ROWS + rr;
         const int G = (1 << S::LA) + h;
         const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
@@ -193,11 +193,10 @@ __global__ void __launch_bounds__(S::THREADS_B, 12) k_fwd_row_st(Tables T, LimbM
         for (int k = 0; k < S::REGB; ++k) x[k] = sb[rr * (1 << S::LB) + k * S::TB + tau];
         stage_row_round1<S>(tsh, twt, G, tau);
         __syncthreads();  // every row is in registers before the buffer becomes the exchange buffer
-        row_fwd_core<S>(x, TwStaged<S>{tsh, twt, G}, sb + rr * S::ROWPAD, tau, q, q2);
+        row_fwd_core<S, AR>(x, TwStaged<S>{tsh, twt, G}, sb + rr * S::ROWPAD, tau, md, T.pm_fold);
         u64 *gout = L.dst + ((size_t)h << S::LB);
-        const u64 one_sh = CANON ? mc.one_sh : 0;
 #pragma unroll
-        for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? reduce_any(x[k], q, one_sh) : x[k];
+        for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? canon_any<AR>(x[k], mc) : x[k];
         b = nb;
         cur ^= 1;
     }
@@ -224,8 +223,8 @@ int ntt_error_flag(bool clear)
 }
 
 // Inverse row pass (stages logN-1..LA), first half of the iNTT.  Input below
-// 4q; output below 4q.
-template <class S, bool SP>
+// 4q; output below 4q (AR_PM: any 64-bit value, folded by the column pass).
+template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, LimbMaps ms)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -234,7 +233,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
     if (lg >= ms.pre[ms.n]) return;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
-    const u64 q = T.modc[L.tf].q, q2 = 2 * q;
+    const ModR<AR> md = mod_inv<AR>(T.modc[L.tf]);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
     const int G = (1 << S::LA) + h;
@@ -249,14 +248,15 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
     // as in the forward row pass; the block barriers of the first round
     // order them before their use
     stage_row_round1<S>(tsh, itwt, G, tau);
-    row_inv_core<S, SP>(x, TwStaged<S>{tsh, itwt, G}, sm + rr * S::ROWPAD, tau, q, q2);
+    row_inv_core<S, AR>(x, TwStaged<S>{tsh, itwt, G}, sm + rr * S::ROWPAD, tau, md);
 #pragma unroll
     for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = x[k];
 }
 
 // Inverse column pass (stages LA-1..0), second half of the iNTT, then the
-// scale (SC: 0 none, 1 the job's per-entry scale, 2 N^-1); output canonical.
-template <class S, int SC, bool SP>
+// scale (SC: the job's per-entry scale where its map has one, else N^-1);
+// output canonical.
+template <class S, bool SC, int AR>
 __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, LimbMaps ms)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
-    const u64 q = mc.q, q2 = 2 * q;
+    const ModR<AR> md = mod_inv<AR>(mc);
     const ulonglong2 *twt = T.itw + ((size_t)L.tf << S::LOGN);
     for (int i = threadIdx.x; i < (1 << S::LA); i += S::THREADS_A) tws[i] = twt[i];
     const int cc = threadIdx.x % S::COLS, tau = threadIdx.x / S::COLS;
@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = L.src[((size_t)((tau * NG + gg) * M + k2) << S::LB) + c];
     __syncthreads();
-    inv_round2<S::LA, S::RA, SP>(x, tau * NG, TwSmem{tws}, q, q2);
+    fold_all<S::REGA, AR>(x, md);
+    inv_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
@@ -289,34 +290,24 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < S::REGA; ++k) x[k] = sm[(k * S::TA + tau) * S::COLS + cc];
-    inv_round1<S::RA, SP>(x, TwSmem{tws}, q, q2);
-    u64 w = 0, wp = 0;
-    if (SC == 1) {
-        const ulonglong2 f = L.scale[L.b];
-        w = f.x;
-        wp = f.y;
-    } else if (SC == 2) {
-        w = mc.ninv;
-        wp = mc.ninv_sh;
-    }
+    fold_all<S::REGA, AR>(x, md);
+    inv_round1<S::RA, AR>(x, TwSmem{tws}, md);
+    ulonglong2 f = make_ulonglong2(0, 0);
+    if (SC) f = L.scale ? L.scale[L.b] : make_ulonglong2(mc.ninv, mc.ninv_sh);
 #pragma unroll
-    for (int k = 0; k < S::REGA; ++k) {
-        u64 v = x[k];
-        if (SC != 0) v = shoup_lazy(v, w, wp, q);
-        L.dst[((size_t)(k * S::TA + tau) << S::LB) + c] = reduce4(v, q, q2);
-    }
+    for (int k = 0; k < S::REGA; ++k)
+        L.dst[((size_t)(k * S::TA + tau) << S::LB) + c] = inv_finish<AR, SC>(x[k], f, mc);
 }
 
-template <class S, bool SP>
-static void set_smem_attrs_sp()
+template <class S, int AR>
+static void set_smem_attrs_ar()
 {
-    cudaFuncSetAttribute(k_fwd_col<S, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_inv_col<S, 0, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_inv_col<S, 1, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_inv_col<S, 2, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_fwd_row<S, true, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
-    cudaFuncSetAttribute(k_fwd_row<S, false, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
-    cudaFuncSetAttribute(k_inv_row<S, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
+    cudaFuncSetAttribute(k_fwd_col<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+    cudaFuncSetAttribute(k_inv_col<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+    cudaFuncSetAttribute(k_inv_col<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+    cudaFuncSetAttribute(k_fwd_row<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
+    cudaFuncSetAttribute(k_fwd_row<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
+    cudaFuncSetAttribute(k_inv_row<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
 }
 
 template <class S>
@@ -324,8 +315,9 @@ static void set_smem_attrs()
 {
     static std::atomic<uint64_t> done{0};  // per instantiation, per device
     once_per_device(done, [] {
-        set_smem_attrs_sp<S, false>();
-        set_smem_attrs_sp<S, true>();
+        set_smem_attrs_ar<S, AR_GEN>();
+        set_smem_attrs_ar<S, AR_SP>();
+        set_smem_attrs_ar<S, AR_PM>();
     });
 }
 
@@ -356,15 +348,12 @@ static void fwd_col_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    if (T.spq)
-        KS_LAUNCH(st, "ntt_fwd_col", k_fwd_col<S, true><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-    else
-        KS_LAUNCH(st, "ntt_fwd_col", k_fwd_col<S, false><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (k_fwd_col<S, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))));
 }
 
 // Persistent grid of the staged row pass: resident CTAs per SM x SMs, at
 // most one CTA per item.
-template <class S, bool CANON>
+template <class S, bool CANON, int AR>
 static int staged_grid(int items)
 {
     static std::atomic<uint64_t> done{0};
@@ -375,9 +364,10 @@ static int staged_grid(int items)
         dev = 0;
     }
     once_per_device(done, [dev] {
-        cudaFuncSetAttribute(k_fwd_row_st<S, CANON>, cudaFuncAttributeMaxDynamicSharedMemorySize, StagedRow<S>::SMEM);
+        cudaFuncSetAttribute(k_fwd_row_st<S, CANON, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             StagedRow<S>::SMEM);
         int n = 0, c = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fwd_row_st<S, CANON>, S::THREADS_B,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fwd_row_st<S, CANON, AR>, S::THREADS_B,
                                                           StagedRow<S>::SMEM) != cudaSuccess ||
             cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
@@ -398,26 +388,22 @@ static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, cudaSt
     // limb are); maps over caller buffers that are not run the plain pass
     bool aligned = true;
     for (int j = 0; j < m.n; ++j) aligned = aligned && (((uintptr_t)m.m[j].src & 15) == 0);
+    const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
     if (T.row_stage && aligned) {
         const int items = m.pre[m.n] * ((1 << S::LA) / S::ROWS);
+        constexpr int TH = S::THREADS_B, SM = StagedRow<S>::SMEM;
         if (canonical)
-            KS_LAUNCH(st, "ntt_fwd_row",
-                      k_fwd_row_st<S, true><<<staged_grid<S, true>(items), S::THREADS_B, StagedRow<S>::SMEM, st>>>(T, m));
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row_st<S, true, AR><<<staged_grid<S, true, AR>(items),
+                                                                                        TH, SM, st>>>(T, m))))
         else
-            KS_LAUNCH(st, "ntt_fwd_row",
-                      k_fwd_row_st<S, false><<<staged_grid<S, false>(items), S::THREADS_B, StagedRow<S>::SMEM, st>>>(T,
-                                                                                                                   m));
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row_st<S, false, AR><<<staged_grid<S, false, AR>(items),
+                                                                                         TH, SM, st>>>(T, m))))
         return;
     }
-    const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
-    if (canonical && T.spq)
-        KS_LAUNCH(st, "ntt_fwd_row", k_fwd_row<S, true, true><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
-    else if (canonical)
-        KS_LAUNCH(st, "ntt_fwd_row", k_fwd_row<S, true, false><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
-    else if (T.spq)
-        KS_LAUNCH(st, "ntt_fwd_row", k_fwd_row<S, false, true><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
+    if (canonical)
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row<S, true, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
     else
-        KS_LAUNCH(st, "ntt_fwd_row", k_fwd_row<S, false, false><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row<S, false, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
 }
 
 template <class S>
@@ -425,33 +411,19 @@ static void inv_row_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
-    if (T.spq)
-        KS_LAUNCH(st, "ntt_inv_row", k_inv_row<S, true><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
-    else
-        KS_LAUNCH(st, "ntt_inv_row", k_inv_row<S, false><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m));
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row", (k_inv_row<S, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
 }
 
+// scaled: multiply by the maps' per-entry scale, or by N^-1 where a map has none.
 template <class S>
-static void inv_col_S(const Tables &T, const LimbMaps &m, bool ninv, cudaStream_t st)
+static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    const int sc = any_scale(m) ? 1 : ninv ? 2 : 0;
-    if (T.spq) {
-        if (sc == 1)
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 1, true><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-        else if (sc == 2)
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 2, true><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-        else
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 0, true><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-    } else {
-        if (sc == 1)
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 1, false><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-        else if (sc == 2)
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 2, false><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-        else
-            KS_LAUNCH(st, "ntt_inv_col", k_inv_col<S, 0, false><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m));
-    }
+    if (scaled)
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (k_inv_col<S, true, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))))
+    else
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (k_inv_col<S, false, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))))
 }
 
 #define KS_DISPATCH_LOGN(logN, FN, ...)                                                                   \
@@ -494,7 +466,7 @@ int launch_fwd_col(const Tables &T, const LimbMaps &m, cudaStream_t st)
 int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st)
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
-    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m, scale_by_ninv, st);
+    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m, scale_by_ninv || any_scale(m), st);
     return launch_status("inverse column pass launch");
 }
 
@@ -516,13 +488,13 @@ int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaS
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     if (T.ntt_cluster) {
-        const int rc = launch_ntt_inv_cluster(T, m, any_scale(m) ? 1 : scale_by_ninv ? 2 : 0, st);
+        const int rc = launch_ntt_inv_cluster(T, m, scale_by_ninv || any_scale(m), st);
         if (rc != KS_EUNSUPPORTED) return rc;
     }
     KS_DISPATCH_LOGN(T.logN, inv_row_S, T, m, st);
     LimbMaps m2 = m;
     for (int j = 0; j < m2.n; ++j) m2.m[j].src = m2.m[j].dst;
-    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m2, scale_by_ninv, st);
+    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m2, scale_by_ninv || any_scale(m), st);
     return launch_status("inverse NTT launch");
 }
 
@@ -740,7 +712,8 @@ __global__ void __launch_bounds__(256) k_apply_key(Tables T, int nact, int j0, i
         mac128(sb, dv, key_b<CK>(key, j, tf, n, nfull, T.logN));
         mac128(sa, dv, key_a<CK>(key, j, tf, n, nfull, T.logN, mc.q));
     }
-    // D below kFwdLazy*q: the REDC result is below q + kFwdLazy*nd*q^2/2^64, reduced fully.
+    // D any 64-bit words: each product is below 2^64 q, the sum of at most 64
+    // below 2^126 and its REDC below 65 q, reduced fully.
     u64 rb = reduce_any(redc(sb, mc.q, mc.mont), mc.q, mc.one_sh);
     u64 ra = key_a_finish<CK>(key, sa, mc, T.key_sc, tf);
     u64 *cb = cp + (size_t)t * N + n;
@@ -785,7 +758,7 @@ struct OutPtrs {
     u64 *p[2];
 };
 
-// ModDown P4: out = cp - v mod q (cp canonical, v lazy below kFwdLazy*q).
+// ModDown P4: out = cp - v mod q (cp canonical, v lazy, at most flz).
 __global__ void __launch_bounds__(256) k_down_final(Tables T, const u64 *cp, size_t cp_stride, const u64 *v,
                                                     size_t v_stride, OutPtrs outs)
 {
@@ -793,7 +766,7 @@ __global__ void __launch_bounds__(256) k_down_final(Tables T, const u64 *cp, siz
     const size_t N = (size_t)1 << T.logN;
     const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const ModC &mc = T.modc[i];
-    const u64 r = cp[x * cp_stride + (size_t)i * N + n] + kFwdLazy * mc.q - v[x * v_stride + (size_t)i * N + n];
+    const u64 r = cp[x * cp_stride + (size_t)i * N + n] + mc.flz - v[x * v_stride + (size_t)i * N + n];
     outs.p[x][(size_t)i * N + n] = reduce_any(r, mc.q, mc.one_sh);
 }
 

@@ -60,7 +60,7 @@ LimbMaps one_map(const LimbMap &m, int nlimbs);
 void add_map(LimbMaps &ms, const LimbMap &m, int nlimbs);
 
 // Forward NTT (column pass src->dst, row pass in place on dst).  Input below
-// 4q.  canonical: output in [0, q); otherwise lazy, below kFwdLazy*q = 72q (every
+// 4q.  canonical: output in [0, q); otherwise lazy, at most ModC::flz (every
 // consumer of lazy output reduces it).
 int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st);
 // Inverse NTT without the N^-1 factor (row pass src->dst, column pass in
@@ -68,13 +68,13 @@ int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStrea
 // map has one, or by N^-1 when scale_by_ninv; output canonical.  Input below 4q.
 int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st);
 // One-launch forms over thread-block clusters (ks_ntt_cluster.cu): the same
-// contracts and bit-identical outputs; sc of the inverse: 0 none, 1 the
-// job's per-entry scale, 2 N^-1.  They return KS_EUNSUPPORTED, launching
+// contracts and bit-identical outputs; scaled (inverse): by the maps'
+// per-entry scale, or by N^-1 where a map has none.  They return KS_EUNSUPPORTED, launching
 // nothing, when the ring degree's shape or the device has no cluster form;
 // launch_ntt_fwd/inv use them when T.ntt_cluster is set and fall back.
 bool ntt_cluster_shape(int logN);
 int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st);
-int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, int sc, cudaStream_t st);
+int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st);
 // Single passes.
 int launch_fwd_col(const Tables &T, const LimbMaps &m, cudaStream_t st);
 int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st);

@@ -21,10 +21,10 @@ namespace ks {
 
 namespace {
 
-// Forward NTT (input below 4q; output canonical with CANON, else below kFwdLazy*q).
+// Forward NTT (input below 4q; output canonical with CANON, else lazy, at most flz).
 // grid (C, limbs), cluster (C, 1, 1): every CTA of a cluster has the same
 // limb, so the early exits below are uniform over the cluster.
-template <class S, int MUL, bool CANON>
+template <class S, int MUL, bool CANON, int AR>
 __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_cl(Tables T, LimbMaps ms)
 {
     typedef Cl<S, MUL> G_;
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
-    const u64 q = mc.q, q2 = 2 * q;
+    const ModR<AR> md = mod_fwd<AR>(mc);
     const int r = cluster_rank();
     const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
     {
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
 #pragma unroll
         for (int k = 0; k < S::REGA; ++k) x[k] = L.src[((size_t)(k * S::TA + tau) << S::LB) + c];
         __syncthreads();
-        fwd_round1<S::RA>(x, TwSmem{tws}, q, q2);
+        fwd_round1<S::RA, AR>(x, TwSmem{tws}, md);
 #pragma unroll
         for (int k = 0; k < S::REGA; ++k) buf[(k * S::TA + tau) * COLS + cc] = x[k];
         __syncthreads();
@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
         for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
             for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = buf[((tau * NG + gg) * M + k2) * COLS + cc];
-        fwd_round2<S::LA, S::RA>(x, tau * NG, TwSmem{tws}, q, q2);
+        if (AR == AR_PM && (T.pm_fold & PM_FOLD_MID)) fold_all<S::REGA, AR>(x, md);
+        fwd_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
         __syncthreads();  // every read of the transpose precedes the block's writes
 #pragma unroll
         for (int gg = 0; gg < NG; ++gg)
@@ -82,16 +83,15 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
     ulonglong2 *tsh = tsh_all + rr * S::REGB;
     stage_row_round1<S>(tsh, twt, G, tau);
     cluster_barrier();  // no CTA reads another's block after this point
-    row_fwd_core<S>(x, TwStaged<S>{tsh, twt, G}, buf + rr * S::ROWPAD, tau, q, q2);
+    row_fwd_core<S, AR>(x, TwStaged<S>{tsh, twt, G}, buf + rr * S::ROWPAD, tau, md, T.pm_fold);
     u64 *gout = L.dst + ((size_t)h << S::LB);
-    const u64 one_sh = CANON ? mc.one_sh : 0;
 #pragma unroll
-    for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? reduce_any(x[k], q, one_sh) : x[k];
+    for (int k = 0; k < S::REGB; ++k) gout[k * S::TB + tau] = CANON ? canon_any<AR>(x[k], mc) : x[k];
 }
 
-// Inverse NTT (input below 4q), then the scale (SC: 0 none, 1 the job's
-// per-entry scale, 2 N^-1); output canonical.
-template <class S, int MUL, int SC>
+// Inverse NTT (input below 4q), then the scale (SC: the job's per-entry scale
+// where its map has one, else N^-1); output canonical.
+template <class S, int MUL, bool SC, int AR>
 __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_cl(Tables T, LimbMaps ms)
 {
     typedef Cl<S, MUL> G_;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
     if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
-    const u64 q = mc.q, q2 = 2 * q;
+    const ModR<AR> md = mod_inv<AR>(mc);
     const int r = cluster_rank();
     const ulonglong2 *itw = T.itw + ((size_t)L.tf << S::LOGN);
     for (int i = threadIdx.x; i < (1 << S::LA); i += G_::THREADS) tws[i] = itw[i];
@@ -113,12 +113,12 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
         // buf[(h - r*ROWS) * 2^LB + c]
         const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
         const int h = r * ROWS + rr;
-        const TwRow tw{itw, (1 << S::LA) + h};
+        const TwRow<S> tw{itw, (1 << S::LA) + h};
         const u64 *gin = L.src + ((size_t)h << S::LB);
         u64 x[S::REGB];
 #pragma unroll
         for (int k = 0; k < S::REGB; ++k) x[k] = gin[k * S::TB + tau];
-        row_inv_core<S>(x, tw, buf + rr * S::ROWPAD, tau, q, q2);  // ends with buf free
+        row_inv_core<S, AR>(x, tw, buf + rr * S::ROWPAD, tau, md);  // ends with buf free
 #pragma unroll
         for (int k = 0; k < S::REGB; ++k) buf[rr * (1 << S::LB) + k * S::TB + tau] = x[k];
     }
@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
             x[gg * M + k2] = ld_dsmem(dsmem_addr(buf + (h % ROWS) * (1 << S::LB) + c, h / ROWS));
         }
     cluster_barrier();  // no CTA reads another's block after this point
-    inv_round2<S::LA, S::RA>(x, tau * NG, TwSmem{tws}, q, q2);
+    fold_all<S::REGA, AR>(x, md);
+    inv_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
@@ -144,38 +145,31 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < S::REGA; ++k) x[k] = buf[(k * S::TA + tau) * COLS + cc];
-    inv_round1<S::RA>(x, TwSmem{tws}, q, q2);
-    u64 w = 0, wp = 0;
-    if (SC == 1) {
-        const ulonglong2 f = L.scale[L.b];
-        w = f.x;
-        wp = f.y;
-    } else if (SC == 2) {
-        w = mc.ninv;
-        wp = mc.ninv_sh;
-    }
+    fold_all<S::REGA, AR>(x, md);
+    inv_round1<S::RA, AR>(x, TwSmem{tws}, md);
+    ulonglong2 f = make_ulonglong2(0, 0);
+    if (SC) f = L.scale ? L.scale[L.b] : make_ulonglong2(mc.ninv, mc.ninv_sh);
 #pragma unroll
-    for (int k = 0; k < S::REGA; ++k) {
-        u64 v = x[k];
-        if (SC != 0) v = shoup_lazy(v, w, wp, q);
-        L.dst[((size_t)(k * S::TA + tau) << S::LB) + c] = reduce4(v, q, q2);
-    }
+    for (int k = 0; k < S::REGA; ++k)
+        L.dst[((size_t)(k * S::TA + tau) << S::LB) + c] = inv_finish<AR, SC>(x[k], f, mc);
 }
 
 template <class S, int MUL>
 struct ClKernels {
     typedef Cl<S, MUL> G;
+    template <int AR> static bool prepare()
+    {
+        return cluster_prepare(k_fwd_cl<S, MUL, false, AR>, G::C, G::THREADS, G::SMEM) &&
+               cluster_prepare(k_fwd_cl<S, MUL, true, AR>, G::C, G::THREADS, G::SMEM) &&
+               cluster_prepare(k_inv_cl<S, MUL, false, AR>, G::C, G::THREADS, G::SMEM) &&
+               cluster_prepare(k_inv_cl<S, MUL, true, AR>, G::C, G::THREADS, G::SMEM);
+    }
     // per device: attributes set and the cluster shape accepted
     static bool ready()
     {
         static std::atomic<uint64_t> done{0}, ok{0};
         once_per_device(done, [] {
-            bool r = true;
-            r = r && cluster_prepare(k_fwd_cl<S, MUL, false>, G::C, G::THREADS, G::SMEM);
-            r = r && cluster_prepare(k_fwd_cl<S, MUL, true>, G::C, G::THREADS, G::SMEM);
-            r = r && cluster_prepare(k_inv_cl<S, MUL, 0>, G::C, G::THREADS, G::SMEM);
-            r = r && cluster_prepare(k_inv_cl<S, MUL, 1>, G::C, G::THREADS, G::SMEM);
-            r = r && cluster_prepare(k_inv_cl<S, MUL, 2>, G::C, G::THREADS, G::SMEM);
+            const bool r = prepare<AR_GEN>() && prepare<AR_PM>();
             int dev = 0;
             if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
             if (r) ok.fetch_or(1ull << (dev & 63));
@@ -218,19 +212,20 @@ static int fwd_cl_SM(const Tables &T, const LimbMaps &m, bool canonical, cudaStr
         if (!ClKernels<S, MUL>::ready()) return KS_EUNSUPPORTED;
         cudaError_t e;
         const int limbs = m.pre[m.n];
+        constexpr int C = G::C, TH = G::THREADS, SM = G::SMEM;
         if (canonical)
-            KS_LAUNCH(st, "ntt_fwd_cl",
-                      e = launch_cluster(k_fwd_cl<S, MUL, true>, G::C, G::THREADS, G::SMEM, limbs, T, m, st));
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_cl", (e = launch_cluster(k_fwd_cl<S, MUL, true, AR>, C, TH, SM, limbs,
+                                                                               T, m, st))))
         else
-            KS_LAUNCH(st, "ntt_fwd_cl",
-                      e = launch_cluster(k_fwd_cl<S, MUL, false>, G::C, G::THREADS, G::SMEM, limbs, T, m, st));
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_cl", (e = launch_cluster(k_fwd_cl<S, MUL, false, AR>, C, TH, SM, limbs,
+                                                                               T, m, st))))
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("cluster NTT launch: ") + cudaGetErrorString(e));
         return KS_OK;
     }
 }
 
 template <class S, int MUL>
-static int inv_cl_SM(const Tables &T, const LimbMaps &m, int sc, cudaStream_t st)
+static int inv_cl_SM(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
 {
     typedef Cl<S, MUL> G;
     if constexpr (!G::OK) {
@@ -240,12 +235,12 @@ static int inv_cl_SM(const Tables &T, const LimbMaps &m, int sc, cudaStream_t st
         cudaError_t e;
         const int limbs = m.pre[m.n];
         constexpr int C = G::C, TH = G::THREADS, SM = G::SMEM;
-        if (sc == 1)
-            KS_LAUNCH(st, "ntt_inv_cl", e = launch_cluster(k_inv_cl<S, MUL, 1>, C, TH, SM, limbs, T, m, st));
-        else if (sc == 2)
-            KS_LAUNCH(st, "ntt_inv_cl", e = launch_cluster(k_inv_cl<S, MUL, 2>, C, TH, SM, limbs, T, m, st));
+        if (scaled)
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_inv_cl", (e = launch_cluster(k_inv_cl<S, MUL, true, AR>, C, TH, SM, limbs,
+                                                                               T, m, st))))
         else
-            KS_LAUNCH(st, "ntt_inv_cl", e = launch_cluster(k_inv_cl<S, MUL, 0>, C, TH, SM, limbs, T, m, st));
+            KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_inv_cl", (e = launch_cluster(k_inv_cl<S, MUL, false, AR>, C, TH, SM, limbs,
+                                                                               T, m, st))))
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("cluster NTT launch: ") + cudaGetErrorString(e));
         return KS_OK;
     }
@@ -258,9 +253,9 @@ static int fwd_cl_S(const Tables &T, const LimbMaps &m, bool canonical, cudaStre
     return T.ntt_cluster == 2 ? fwd_cl_SM<S, 2>(T, m, canonical, st) : fwd_cl_SM<S, 1>(T, m, canonical, st);
 }
 template <class S>
-static int inv_cl_S(const Tables &T, const LimbMaps &m, int sc, cudaStream_t st)
+static int inv_cl_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
 {
-    return T.ntt_cluster == 2 ? inv_cl_SM<S, 2>(T, m, sc, st) : inv_cl_SM<S, 1>(T, m, sc, st);
+    return T.ntt_cluster == 2 ? inv_cl_SM<S, 2>(T, m, scaled, st) : inv_cl_SM<S, 1>(T, m, scaled, st);
 }
 
 #define KS_CL_DISPATCH(logN, FN, ...)                         \
@@ -298,9 +293,9 @@ int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, c
     KS_CL_DISPATCH(T.logN, fwd_cl_S, T, m, canonical, st);
 }
 
-int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, int sc, cudaStream_t st)
+int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
 {
-    KS_CL_DISPATCH(T.logN, inv_cl_S, T, m, sc, st);
+    KS_CL_DISPATCH(T.logN, inv_cl_S, T, m, scaled, st);
 }
 
 }  // namespace ks

@@ -64,10 +64,10 @@ struct TwStaged {
     const ulonglong2 *sh;
     const ulonglong2 *t;
     int G;
-    __device__ __forceinline__ ulonglong2 operator()(int s, int i) const
+    __device__ __forceinline__ ulonglong2 operator()(int s, int i) const { return sh[(1 << s) - 1 + i]; }
+    template <int NG> __device__ __forceinline__ ulonglong2 r2(int s, int, int tau, int gg, int g2) const
     {
-        if (s < S::RB) return sh[(1 << s) - 1 + i];
-        return __ldg(t + (G << s) + i);
+        return __ldg(t + (G << s) + (g2 * NG + gg) * S::TB + tau);
     }
 };
 
@@ -75,11 +75,14 @@ struct TwStaged {
 // leaves in the first-round layout (x[k] is element k*TB + tau of the row),
 // srow is the row's padded shared-memory buffer.  Contains block barriers:
 // every thread of the block must call it.
-template <class S, bool SP = false, class TW>
-__device__ __forceinline__ void row_fwd_core(u64 (&x)[S::REGB], const TW &tw, u64 *srow, int tau, u64 q, u64 q2)
+// pf: the folds this set's transforms need (Tables::pm_fold, uniform).
+template <class S, int AR, class TW>
+__device__ __forceinline__ void row_fwd_core(u64 (&x)[S::REGB], const TW &tw, u64 *srow, int tau, const ModR<AR> &m,
+                                             int pf)
 {
     constexpr int M = S::MB, NG = S::REGB / S::MB;
-    fwd_round1<S::RB, SP>(x, tw, q, q2);
+    if (AR == AR_PM && (pf & PM_FOLD_ROW)) fold_all<S::REGB, AR>(x, m);
+    fwd_round1<S::RB, AR>(x, tw, m);
 #pragma unroll
     for (int k = 0; k < S::REGB; ++k) srow[rpad<S>(k * S::TB + tau)] = x[k];
     __syncthreads();
@@ -87,7 +90,8 @@ __device__ __forceinline__ void row_fwd_core(u64 (&x)[S::REGB], const TW &tw, u6
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = srow[rpad<S>((tau * NG + gg) * M + k2)];
-    fwd_round2<S::LB, S::RB, SP>(x, tau * NG, tw, q, q2);
+    if (AR == AR_PM && (pf & PM_FOLD_MID)) fold_all<S::REGB, AR>(x, m);
+    fwd_round2<S::LB, S::RB, AR>(x, tau, tw, m);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
@@ -100,8 +104,8 @@ __device__ __forceinline__ void row_fwd_core(u64 (&x)[S::REGB], const TW &tw, u6
 }
 
 // Row pass of the inverse NTT (stages logN-1 .. LA), same layout contract.
-template <class S, bool SP = false, class TW>
-__device__ __forceinline__ void row_inv_core(u64 (&x)[S::REGB], const TW &tw, u64 *srow, int tau, u64 q, u64 q2)
+template <class S, int AR, class TW>
+__device__ __forceinline__ void row_inv_core(u64 (&x)[S::REGB], const TW &tw, u64 *srow, int tau, const ModR<AR> &m)
 {
     constexpr int M = S::MB, NG = S::REGB / S::MB;
 #pragma unroll
@@ -111,7 +115,7 @@ __device__ __forceinline__ void row_inv_core(u64 (&x)[S::REGB], const TW &tw, u6
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = srow[rpad<S>((tau * NG + gg) * M + k2)];
-    inv_round2<S::LB, S::RB, SP>(x, tau * NG, tw, q, q2);
+    inv_round2<S::LB, S::RB, AR>(x, tau, tw, m);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
@@ -121,7 +125,52 @@ __device__ __forceinline__ void row_inv_core(u64 (&x)[S::REGB], const TW &tw, u6
 #pragma unroll
     for (int k = 0; k < S::REGB; ++k) x[k] = srow[rpad<S>(k * S::TB + tau)];
     __syncthreads();
-    inv_round1<S::RB, SP>(x, tw, q, q2);
+    fold_all<S::REGB, AR>(x, m);
+    inv_round1<S::RB, AR>(x, tw, m);
 }
+
+// A forward output as the key product takes it: canonical or lazy in the
+// other forms (below kFwdLazy*q), folded below 2^(b+1) plus a little here.
+template <int AR>
+__device__ __forceinline__ u64 key_input(u64 x, const ModR<AR> &m)
+{
+    return fold<AR>(x, m);
+}
+// Any 64-bit value -> [0, q).
+template <int AR>
+__device__ __forceinline__ u64 canon_any(u64 x, const ModC &mc)
+{
+    if constexpr (AR == AR_PM)
+        return pm_canon(x, mc.q, mc.pm_c2, mc.pm_k);
+    else
+        return reduce_any(x, mc.q, mc.one_sh);
+}
+// End of an inverse transform: the scale (W a twiddle-form pair when SC) and
+// the reduction to [0, q).  x below 4q (AR_GEN, AR_SP) or any (AR_PM).
+template <int AR, bool SC>
+__device__ __forceinline__ u64 inv_finish(u64 x, const ulonglong2 &W, const ModC &mc)
+{
+    if constexpr (AR == AR_PM) {
+        if (SC) x = pm_mul(x, W, mc.pm_c2, mc.pm_k);
+        return pm_canon(x, mc.q, mc.pm_c2, mc.pm_k);
+    } else {
+        if (SC) x = shoup_lazy(x, W.x, W.y, mc.q);
+        return reduce4(x, mc.q, 2 * mc.q);
+    }
+}
+
+// Runs FN<AR>(...) for the parameter set's butterfly form.
+#define KS_DISPATCH_AR(T, CALL)                \
+    switch ((T).arith) {                       \
+    case AR_PM: { constexpr int AR = AR_PM; CALL; break; } \
+    case AR_SP: { constexpr int AR = AR_SP; CALL; break; } \
+    default: { constexpr int AR = AR_GEN; CALL; break; }   \
+    }
+// The same for kernels without a special-form instance (AR_SP sets use AR_GEN).
+#define KS_DISPATCH_AR2(T, CALL)               \
+    switch ((T).arith) {                       \
+    case AR_PM: { constexpr int AR = AR_PM; CALL; break; } \
+    default: { constexpr int AR = AR_GEN; CALL; break; }   \
+    }
 
 }  // namespace ks

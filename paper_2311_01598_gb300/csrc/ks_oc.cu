@@ -24,7 +24,8 @@
 namespace ks {
 
 // x * e with the stored key word e: REDC of the 128-bit product; x below
-// kFwdLazy*q, so the result is below q + 72q^2/2^64 < 2q before the correction.
+// kFwdLazy*q or folded (key_input), so the result is below q + 72q^2/2^64 <
+// 2q before the correction.
 __device__ __forceinline__ u64 key_mul(u64 x, u64 e, u64 q, u64 mont)
 {
     U128 t = {0, 0};
@@ -48,56 +49,58 @@ struct RowSmem {
 // One digit's share of the key product for the block's rows: the row pass of
 // the limb at gin (skipped for the bypassed digit, whose input is already in
 // evaluation form), then x * evk_b and x * evk_a added into the accumulators.
-template <class S>
+template <class S, int AR>
 __device__ __noinline__ void oc_digit(const u64 *gin, int transform, const ulonglong2 *twt, int G, u64 *srow, int tau,
-                                      const u64 *eb, const u64 *ea, u64 *ab, u64 *aa, int first, u64 q, u64 mont)
+                                      const u64 *eb, const u64 *ea, u64 *ab, u64 *aa, int first, ModR<AR> md, int pf,
+                                      u64 q, u64 mont)
 {
     u64 x[S::REGB];
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) x[i] = gin[i * S::TB + tau];
-    if (transform) row_fwd_core<S>(x, TwRow{twt, G}, srow, tau, q, 2 * q);
+    if (transform) row_fwd_core<S, AR>(x, TwRow<S>{twt, G}, srow, tau, md, pf);
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) {
         const int c = i * S::TB + tau;
-        const u64 pb = key_mul(x[i], __ldg(eb + c), q, mont);
-        const u64 pa = key_mul(x[i], __ldg(ea + c), q, mont);
+        const u64 v = key_input<AR>(x[i], md);
+        const u64 pb = key_mul(v, __ldg(eb + c), q, mont);
+        const u64 pa = key_mul(v, __ldg(ea + c), q, mont);
         ab[c] = first ? pb : reduce2(ab[c] + pb, q);
         aa[c] = first ? pa : reduce2(aa[c] + pa, q);
     }
 }
 
 // Row pass of the inverse NTT of an accumulator row, stored to out.
-template <class S>
+template <class S, int AR>
 __device__ __noinline__ void oc_inv_store(const u64 *acc, const ulonglong2 *itwt, int G, u64 *srow, int tau, u64 *out,
-                                          u64 q)
+                                          ModR<AR> md)
 {
     u64 x[S::REGB];
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) x[i] = acc[i * S::TB + tau];
-    row_inv_core<S>(x, TwRow{itwt, G}, srow, tau, q, 2 * q);
+    row_inv_core<S, AR>(x, TwRow<S>{itwt, G}, srow, tau, md);
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) out[i * S::TB + tau] = x[i];
 }
 
 // Row pass of a ModDown limb, then out = acc - NTT(v) mod q.
-template <class S>
+template <class S, int AR>
 __device__ __noinline__ void oc_down_store(const u64 *gin, const ulonglong2 *twt, int G, u64 *srow, int tau,
-                                           const u64 *acc, u64 *out, u64 q, u64 one_sh)
+                                           const u64 *acc, u64 *out, ModR<AR> md, int pf, const ModC &mc)
 {
     u64 v[S::REGB];
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) v[i] = gin[i * S::TB + tau];
-    row_fwd_core<S>(v, TwRow{twt, G}, srow, tau, q, 2 * q);
-    const u64 qlz = kFwdLazy * q;
+    row_fwd_core<S, AR>(v, TwRow<S>{twt, G}, srow, tau, md, pf);
+    const u64 qlz = mc.flz;
 #pragma unroll
     for (int i = 0; i < S::REGB; ++i) {
         const int c = i * S::TB + tau;
-        out[c] = reduce_any(acc[c] + qlz - v[i], q, one_sh);
+        out[c] = reduce_any(acc[c] + qlz - v[i], mc.q, mc.one_sh);
     }
 }
 
 // P section, fused row kernel.  grid (2^LA/ROWS, jobs*K).
-template <class S>
+template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowP(Tables T, OcJobs oj)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowP(Tables T, OcJobs oj)
     const int nt = nact + K;
     const int nfull = T.nq + K;
     const ModC &mc = T.modc[tf];
+    const ModR<AR> mdf = mod_fwd<AR>(mc);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
     u64 *srow = sm + rr * S::ROWPAD;
@@ -130,20 +134,21 @@ __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowP(Tables T, OcJobs oj)
     if (threadIdx.x == 0) prefetch_digit(0);
     for (int j = 0; j < J.nd; ++j) {
         if (threadIdx.x == 0 && j + 1 < J.nd) prefetch_digit(j + 1);
-        oc_digit<S>(J.tmp + ((size_t)(j * K + k) << S::LOGN) + rowoff, 1, twt, G, srow, tau,
+        oc_digit<S, AR>(J.tmp + ((size_t)(j * K + k) << S::LOGN) + rowoff, 1, twt, G, srow, tau,
                     J.key.evk + ((size_t)((j * 2 + 0) * nfull + tf) << S::LOGN) + rowoff,
-                    J.key.evk + ((size_t)((j * 2 + 1) * nfull + tf) << S::LOGN) + rowoff, ab, aa, j == 0, mc.q, mc.mont);
+                    J.key.evk + ((size_t)((j * 2 + 1) * nfull + tf) << S::LOGN) + rowoff, ab, aa, j == 0, mdf, T.pm_fold,
+                        mc.q, mc.mont);
     }
     const ulonglong2 *itwt = T.itw + ((size_t)tf << S::LOGN);
-    oc_inv_store<S>(ab, itwt, G, srow, tau, J.cp + ((size_t)t << S::LOGN) + rowoff, mc.q);
-    oc_inv_store<S>(aa, itwt, G, srow, tau, J.cp + ((size_t)(nt + t) << S::LOGN) + rowoff, mc.q);
+    oc_inv_store<S, AR>(ab, itwt, G, srow, tau, J.cp + ((size_t)t << S::LOGN) + rowoff, mod_inv<AR>(mc));
+    oc_inv_store<S, AR>(aa, itwt, G, srow, tau, J.cp + ((size_t)(nt + t) << S::LOGN) + rowoff, mod_inv<AR>(mc));
 }
 
 // Q section, fused row kernel.  grid (2^LA/ROWS, sum of nact over jobs).
 // tmp holds [nd + 2][nact] limbs: rows j < nd the ModUp limbs of digit j
 // (the slot of the tower's own digit unused), rows nd and nd+1 the ModDown
 // limbs of the two polynomials.
-template <class S>
+template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowQ(Tables T, OcJobs oj)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -155,6 +160,7 @@ __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowQ(Tables T, OcJobs oj)
     const int j0 = t / T.alpha;
     const int nfull = T.nq + T.kp;
     const ModC &mc = T.modc[t];
+    const ModR<AR> mdf = mod_fwd<AR>(mc);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
     u64 *srow = sm + rr * S::ROWPAD;
@@ -183,31 +189,37 @@ __global__ void __launch_bounds__(S::THREADS_B) k_oc_rowQ(Tables T, OcJobs oj)
         }
         const u64 *gin = j == j0 ? J.d + ((size_t)t << S::LOGN) + rowoff
                                  : J.tmp + ((size_t)(j * nact + t) << S::LOGN) + rowoff;
-        oc_digit<S>(gin, j != j0, twt, G, srow, tau, J.key.evk + ((size_t)((j * 2 + 0) * nfull + t) << S::LOGN) + rowoff,
-                    J.key.evk + ((size_t)((j * 2 + 1) * nfull + t) << S::LOGN) + rowoff, ab, aa, j == 0, mc.q, mc.mont);
+        oc_digit<S, AR>(gin, j != j0, twt, G, srow, tau, J.key.evk + ((size_t)((j * 2 + 0) * nfull + t) << S::LOGN) + rowoff,
+                    J.key.evk + ((size_t)((j * 2 + 1) * nfull + t) << S::LOGN) + rowoff, ab, aa, j == 0, mdf, T.pm_fold,
+                        mc.q, mc.mont);
     }
     for (int xp = 0; xp < 2; ++xp)
-        oc_down_store<S>(J.tmp + ((size_t)((J.nd + xp) * nact + t) << S::LOGN) + rowoff, twt, G, srow, tau,
-                         xp == 0 ? ab : aa, (xp == 0 ? J.out0 : J.out1) + ((size_t)t << S::LOGN) + rowoff, mc.q,
-                         mc.one_sh);
+        oc_down_store<S, AR>(J.tmp + ((size_t)((J.nd + xp) * nact + t) << S::LOGN) + rowoff, twt, G, srow, tau,
+                         xp == 0 ? ab : aa, (xp == 0 ? J.out0 : J.out1) + ((size_t)t << S::LOGN) + rowoff, mdf, T.pm_fold, mc);
+}
+
+template <class S, int AR>
+static void oc_rows_SA(const Tables &T, const OcJobs &oj, bool p_section, cudaStream_t st)
+{
+    static std::atomic<uint64_t> attr{0};
+    once_per_device(attr, [] {
+        cudaFuncSetAttribute(k_oc_rowP<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowSmem<S>::BYTES);
+        cudaFuncSetAttribute(k_oc_rowQ<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowSmem<S>::BYTES);
+    });
+    if (p_section)
+        KS_LAUNCH(st, "oc_row_p",
+                  (k_oc_rowP<S, AR><<<dim3((1 << S::LA) / S::ROWS, oj.n * T.kp), S::THREADS_B, RowSmem<S>::BYTES, st>>>(
+                      T, oj)));
+    else
+        KS_LAUNCH(st, "oc_row_q",
+                  (k_oc_rowQ<S, AR><<<dim3((1 << S::LA) / S::ROWS, oj.pre[oj.n]), S::THREADS_B, RowSmem<S>::BYTES, st>>>(
+                      T, oj)));
 }
 
 template <class S>
 static void oc_rows_S(const Tables &T, const OcJobs &oj, bool p_section, cudaStream_t st)
 {
-    static std::atomic<uint64_t> attr{0};
-    once_per_device(attr, [] {
-        cudaFuncSetAttribute(k_oc_rowP<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowSmem<S>::BYTES);
-        cudaFuncSetAttribute(k_oc_rowQ<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, RowSmem<S>::BYTES);
-    });
-    if (p_section)
-        KS_LAUNCH(st, "oc_row_p",
-                  k_oc_rowP<S><<<dim3((1 << S::LA) / S::ROWS, oj.n * T.kp), S::THREADS_B, RowSmem<S>::BYTES, st>>>(
-                      T, oj));
-    else
-        KS_LAUNCH(st, "oc_row_q",
-                  k_oc_rowQ<S><<<dim3((1 << S::LA) / S::ROWS, oj.pre[oj.n]), S::THREADS_B, RowSmem<S>::BYTES, st>>>(
-                      T, oj));
+    KS_DISPATCH_AR2(T, (oc_rows_SA<S, AR>(T, oj, p_section, st)))
 }
 
 static int oc_rows(const Tables &T, const OcJobs &oj, bool p_section, cudaStream_t st)
@@ -364,7 +376,7 @@ __global__ void __launch_bounds__(256) k_oc_comb_q(Tables T, OcJobs oj)
     u64 vb[V], va[V], o0[V], o1[V];
     ldv<V>(J.tmp + (size_t)(J.nd * nact + t) * N + n, vb);
     ldv<V>(J.tmp + (size_t)((J.nd + 1) * nact + t) * N + n, va);
-    const u64 qlz = kFwdLazy * mc.q;
+    const u64 qlz = mc.flz;
 #pragma unroll
     for (int c = 0; c < V; ++c) {
         const u64 cb = reduce_any(redc(sb[c], mc.q, mc.mont), mc.q, mc.one_sh);
@@ -512,7 +524,7 @@ __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGrou
                 }
             }
     }
-    const u64 qlz = kFwdLazy * mc.q;
+    const u64 qlz = mc.flz;
 #pragma unroll
     for (int i = 0; i < kGroupJobs; ++i)
         if (i < cnt) {
@@ -692,7 +704,7 @@ __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
     u64 vb[V], va[V], o0[V], o1[V];
     ldv<V>(v + (size_t)t * N + n, vb);
     ldv<V>(v + (size_t)(nact + t) * N + n, va);
-    const u64 qlz = kFwdLazy * mc.q;
+    const u64 qlz = mc.flz;
 #pragma unroll
     for (int c = 0; c < V; ++c) {
         const u64 cb = reduce_any(redc(sb[c], mc.q, mc.mont), mc.q, mc.one_sh);

@@ -44,7 +44,8 @@ struct TowerShape {
 };
 
 // x * e (e a stored key word, Montgomery form with the tower's fold factor):
-// REDC of the 128-bit product; x below kFwdLazy*q gives a result below 2q.
+// REDC of the 128-bit product; x below kFwdLazy*q or folded (key_input) gives
+// a result below 2q.
 __device__ __forceinline__ u64 key_prod(u64 x, u64 e, u64 q, u64 mont)
 {
     U128 t = {0, 0};
@@ -54,17 +55,17 @@ __device__ __forceinline__ u64 key_prod(u64 x, u64 e, u64 q, u64 mont)
 
 // Forward NTT of one limb of tower t spread over the cluster.  Enters with
 // xc[k] = element (row k*TA + tauc, column c) of the CTA's column block
-// (below 4q) and leaves with xr[k] = element k*TB + tau of row h (below
-// kFwdLazy*q).  Contains block and cluster barriers: every thread of every CTA of
+// (below 4q) and leaves with xr[k] = element k*TB + tau of row h (at most
+// flz).  Contains block and cluster barriers: every thread of every CTA of
 // the cluster calls it.
-template <class S>
+template <class S, int AR>
 __device__ __forceinline__ void tower_ntt(u64 (&xc)[S::REGA], u64 (&xr)[S::REGB], u64 *buf,
                                           const ulonglong2 *tws, const ulonglong2 *tsh, const ulonglong2 *twt,
-                                          int G, int cc, int tauc, int rr, int tau, int h, u64 q, u64 q2)
+                                          int G, int cc, int tauc, int rr, int tau, int h, const ModR<AR> &md, int pf)
 {
     typedef Cl<S, 1> G_;
     constexpr int COLS = G_::COLS;
-    fwd_round1<S::RA>(xc, TwSmem{tws}, q, q2);
+    fwd_round1<S::RA, AR>(xc, TwSmem{tws}, md);
 #pragma unroll
     for (int k = 0; k < S::REGA; ++k) buf[(k * S::TA + tauc) * COLS + cc] = xc[k];
     __syncthreads();
@@ -73,7 +74,8 @@ __device__ __forceinline__ void tower_ntt(u64 (&xc)[S::REGA], u64 (&xr)[S::REGB]
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) xc[gg * M + k2] = buf[((tauc * NG + gg) * M + k2) * COLS + cc];
-    fwd_round2<S::LA, S::RA>(xc, tauc * NG, TwSmem{tws}, q, q2);
+    if (AR == AR_PM && (pf & PM_FOLD_MID)) fold_all<S::REGA, AR>(xc, md);
+    fwd_round2<S::LA, S::RA, AR>(xc, tauc, TwSmem{tws}, md);
     __syncthreads();  // every read of the transpose precedes the block's writes
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
@@ -86,7 +88,7 @@ __device__ __forceinline__ void tower_ntt(u64 (&xc)[S::REGA], u64 (&xr)[S::REGB]
         xr[k] = ld_dsmem(dsmem_addr(buf + h * COLS + c % COLS, c / COLS));
     }
     cluster_barrier();  // no CTA reads another's block after this point
-    row_fwd_core<S>(xr, TwStaged<S>{tsh, twt, G}, buf + rr * S::ROWPAD, tau, q, q2);
+    row_fwd_core<S, AR>(xr, TwStaged<S>{tsh, twt, G}, buf + rr * S::ROWPAD, tau, md, pf);
 }
 
 // Base conversion at the CTA's column positions: xc[k] = sum_i src_i[n] *
@@ -121,7 +123,7 @@ __device__ __forceinline__ void tower_bconv(u64 (&xc)[S::REGA], const u64 *src, 
 // grid (C, sum of nact over jobs), cluster (C, 1, 1): every CTA of a
 // cluster has the same (job, tower), so all control flow below is uniform
 // over the cluster.  Full keys only (the launcher checks).
-template <class S>
+template <class S, int AR>
 __global__ void __launch_bounds__(Cl<S, 1>::THREADS, 2) k_oc_tower(Tables T, OcJobs oj)
 {
     typedef Cl<S, 1> G_;
@@ -143,7 +145,8 @@ __global__ void __launch_bounds__(Cl<S, 1>::THREADS, 2) k_oc_tower(Tables T, OcJ
     const int nt = nact + K, nfull = T.nq + K;
     const int alpha = T.alpha, j0 = t / alpha;
     const ModC &mc = T.modc[t];
-    const u64 q = mc.q, q2 = 2 * q;
+    const u64 q = mc.q;
+    const ModR<AR> md = mod_fwd<AR>(mc);
     const size_t N = (size_t)1 << S::LOGN;
     const int r = cluster_rank();
     const ulonglong2 *twt = T.tw + ((size_t)t << S::LOGN);
@@ -195,7 +198,7 @@ __global__ void __launch_bounds__(Cl<S, 1>::THREADS, 2) k_oc_tower(Tables T, OcJ
     // instruction fetch).
     u64 xc[S::REGA], xr[S::REGB];
     const int nup = J.nd - 1;
-    const u64 qlz = kFwdLazy * q;
+    const u64 qlz = mc.flz;
     for (int p = 0; p < nup + 2; ++p) {
         const bool down = p >= nup;
         const int j = down ? 0 : (p < j0 ? p : p + 1);
@@ -217,7 +220,7 @@ __global__ void __launch_bounds__(Cl<S, 1>::THREADS, 2) k_oc_tower(Tables T, OcJ
         __syncthreads();
         // base conversion to t at the CTA's column positions, then the NTT
         tower_bconv<S>(xc, src, nsrc, cst, c, tauc, mc);
-        tower_ntt<S>(xc, xr, buf, tws, tsh, twt, G, cc, tauc, rr, tau, h, q, q2);
+        tower_ntt<S, AR>(xc, xr, buf, tws, tsh, twt, G, cc, tauc, rr, tau, h, md, T.pm_fold);
         if (!down) {
             // key product of digit j added into the accumulators
             const u64 *eb = J.key.evk + ((size_t)((2 * j) * nfull + t) << S::LOGN) + rowoff;
@@ -225,8 +228,9 @@ __global__ void __launch_bounds__(Cl<S, 1>::THREADS, 2) k_oc_tower(Tables T, OcJ
 #pragma unroll
             for (int k = 0; k < S::REGB; ++k) {
                 const int e = k * S::TB + tau;
-                ab[e] = reduce2(ab[e] + key_prod(xr[k], __ldg(eb + e), q, mc.mont), q);
-                aa[e] = reduce2(aa[e] + key_prod(xr[k], __ldg(ea + e), q, mc.mont), q);
+                const u64 v = key_input<AR>(xr[k], md);
+                ab[e] = reduce2(ab[e] + key_prod(v, __ldg(eb + e), q, mc.mont), q);
+                aa[e] = reduce2(aa[e] + key_prod(v, __ldg(ea + e), q, mc.mont), q);
             }
         } else {
             // ModDown P4: out_x = c'_x - NTT(v_x)
@@ -251,7 +255,9 @@ struct TowerKernel {
         } else {
             static std::atomic<uint64_t> done{0}, ok{0};
             once_per_device(done, [] {
-                const bool r = cluster_prepare(k_oc_tower<S>, Cl<S, 1>::C, Cl<S, 1>::THREADS, TowerShape<S>::SMEM);
+                const bool r =
+                    cluster_prepare(k_oc_tower<S, AR_GEN>, Cl<S, 1>::C, Cl<S, 1>::THREADS, TowerShape<S>::SMEM) &&
+                    cluster_prepare(k_oc_tower<S, AR_PM>, Cl<S, 1>::C, Cl<S, 1>::THREADS, TowerShape<S>::SMEM);
                 int dev = 0;
                 if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
                 if (r) ok.fetch_or(1ull << (dev & 63));
@@ -286,7 +292,7 @@ int tower_S(const Tables &T, const OcJobs &oj, cudaStream_t st)
         cfg.attrs = at;
         cfg.numAttrs = 1;
         cudaError_t e;
-        KS_LAUNCH(st, "oc_tower", e = cudaLaunchKernelEx(&cfg, k_oc_tower<S>, T, oj));
+        KS_DISPATCH_AR2(T, KS_LAUNCH(st, "oc_tower", (e = cudaLaunchKernelEx(&cfg, k_oc_tower<S, AR>, T, oj))))
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC tower launch: ") + cudaGetErrorString(e));
         return KS_OK;
     }

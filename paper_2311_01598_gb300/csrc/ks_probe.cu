@@ -1,6 +1,6 @@
 // ks_probe.cu -- arithmetic ceilings of this GPU for the two inner loops of
 // key switching, measured with the same device functions the kernels use:
-//   * the forward NTT butterfly (Shoup product by a twiddle, lazy sums),
+//   * the forward NTT butterfly (AR_PM product by a twiddle, lazy sums),
 //   * the base-conversion multiply-accumulate (three 32x32->64 multiply-adds
 //     into three 64-bit column sums, Karatsuba form).
 // Each probe runs a register-only loop on every SM (no memory traffic inside
@@ -14,19 +14,25 @@ namespace ks {
 constexpr int kProbeBlocks = 152 * 8;
 constexpr int kProbeThreads = 256;
 
+// A prime just below 2^54 (the default rule's form) and its AR_PM constants.
+constexpr u64 kProbePrime = (1ull << 54) - (1ull << 26);  // the rate does not depend on primality
+__device__ __forceinline__ ModR<AR_PM> probe_mod() { return ModR<AR_PM>{kProbePrime * 80, 1u << 27, 23}; }
+// Twiddles vary with i so that no product is shared between butterflies.
+__device__ __forceinline__ ulonglong2 probe_tw(u64 w, u64 wp, int i) { return make_ulonglong2(w + i, wp + i); }
+
 __global__ void __launch_bounds__(kProbeThreads) k_probe_bfly(u64 *out, u64 q, u64 w, u64 wp, int iters)
 {
     u64 x[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) x[i] = (threadIdx.x * 16 + i + blockIdx.x) % q;
-    const u64 q2 = 2 * q;
+    const ModR<AR_PM> md = probe_mod();
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) fwd_bfly(x[i], x[i + 8], w + i, wp + i, q, q2);
+        for (int i = 0; i < 8; ++i) fwd_bfly<AR_PM>(x[i], x[i + 8], probe_tw(w, wp, i), md);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            fwd_bfly(x[i], x[i + 4], w, wp, q, q2);
-            fwd_bfly(x[i + 8], x[i + 12], w + 1, wp + 1, q, q2);
+            fwd_bfly<AR_PM>(x[i], x[i + 4], probe_tw(w, wp, 0), md);
+            fwd_bfly<AR_PM>(x[i + 8], x[i + 12], probe_tw(w, wp, 1), md);
         }
     }
     u64 s = 0;
@@ -35,20 +41,20 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_bfly(u64 *out, u64 q, u
     out[blockIdx.x * blockDim.x + threadIdx.x] = s;  // keeps the loop alive
 }
 
-// The inverse (Harvey) butterfly in the same pattern.
+// The inverse butterfly in the same pattern.
 __global__ void __launch_bounds__(kProbeThreads) k_probe_ibfly(u64 *out, u64 q, u64 w, u64 wp, int iters)
 {
     u64 x[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) x[i] = (threadIdx.x * 16 + i + blockIdx.x) % q;
-    const u64 q2 = 2 * q;
+    const ModR<AR_PM> md = probe_mod();
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) inv_bfly(x[i], x[i + 8], w + i, wp + i, q, q2);
+        for (int i = 0; i < 8; ++i) inv_bfly<AR_PM>(x[i], x[i + 8], probe_tw(w, wp, i), md, false);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            inv_bfly(x[i], x[i + 4], w, wp, q, q2);
-            inv_bfly(x[i + 8], x[i + 12], w + 1, wp + 1, q, q2);
+            inv_bfly<AR_PM>(x[i], x[i + 4], probe_tw(w, wp, 0), md, false);
+            inv_bfly<AR_PM>(x[i + 8], x[i + 12], probe_tw(w, wp, 1), md, false);
         }
     }
     u64 s = 0;
