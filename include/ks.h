@@ -105,8 +105,9 @@ int ks_params_info(const ks_params *params, uint64_t *h_q, uint64_t *h_p,
 /* Implementation options of a parameter set (none changes any result).
  *   KS_OPT_BCONV_TENSOR (default 1): run the fast base conversions (ModUp P2,
  *     ModDown P2) on the tensor cores (tcgen05, exact f16 slices)
- *     wherever at most 18 source towers meet N >= 2^7; 0 selects the CUDA-core
- *     kernels everywhere.
+ *     wherever at most 18 source towers meet (36 for primes just below a power
+ *     of two, as the default rule gives); 0 selects the CUDA-core kernels
+ *     everywhere.
  *   KS_OPT_BATCH_LANES (default 2, 1..4): an Output-Centric batch of at least
  *     4 jobs per lane is split over that many library streams, forked from
  *     and joined back to the caller's stream (the memory-bound combine

@@ -15,19 +15,22 @@
 // 511 with W = 9, below 2^23) is an exact integer in the fp32 accumulator.  One MMA of M=128 coefficients,
 // K = 7*(sources) padded to 64 (up to 9 sources) or 128 (up to 18: two K
 // blocks), N = 8 per target (7 byte rows used) computes
-// all P_{t,b} of up to 32 targets: the A tile holds the byte slices of y
+// all P_{t,b} of up to 32 targets.  19 to 36 sources take two such A tiles with
+// an accumulator each, added in the epilogue (16 targets at a time).  The A
+// tile holds the byte slices of y
 // (built by the CTA from the source limbs), the B tile the per-target slabs
 // B[b][7i+a] = c'_{i,a,t,b} (precomputed on the host, 1 KB a K block).  The
 // epilogue reads the 6 or 7 sums from tensor memory and recombines them into
-// S = sum_{i,a} y_{i,a} c'_{i,a,t} exactly; S <= 126*255*r < 2^15 r, so one
-// Montgomery step by 2^32 (constants carry 2^32) leaves (S + m r)/2^32 below
-// 2r: a lazy [0, 2r) output like the CUDA-core kernels (the same residue; the
-// representative may differ).
+// S = sum_{i,a} y_{i,a} c'_{i,a,t} exactly; S <= 126*255*r < 2^15 r.  For moduli
+// just below a power of two (AR_PM, ks_device.cuh) the top bits of S are folded
+// by r = 2^b - c (tc_reduce_pm), an output below 4r; otherwise one Montgomery
+// step by 2^32 (constants carry 2^32) leaves (S + m r)/2^32 below 2r.  Either
+// is the same residue as the CUDA-core kernels' lazy output.
 //
 // Operand layout: the canonical K-major layout without swizzle: 8x16-byte
 // core matrices, K-adjacent core matrices 128 bytes apart (LBO), 8-row
 // groups 1024 bytes a K block apart (SBO); B slabs of 8 rows concatenate.
-#include <cstdio>
+#include <algorithm>
 
 #include "ks_device.cuh"
 #include "ks_launch.h"
@@ -45,7 +48,13 @@ template <int KB> struct TcK {
     static constexpr int K = 64 * KB;
     static constexpr uint32_t SBO = (K / 8) * 128;
     static constexpr int SLAB = 8 * K * 2;  // bytes of one target slab
-    static constexpr int NSV = KB == 1 ? 5 : 10;  // source words of one producer (half a row)
+    static constexpr int SRC = 9 * KB;            // sources of one A tile
+    static constexpr int ATILE = TC_M * K * 2;    // bytes of an A tile
+};
+// Targets of one item: both accumulator buffers hold NS accumulators of 8
+// columns a target in 512 columns of tensor memory.
+template <int NS> struct TcTargets {
+    static constexpr int N = TC_TB / NS;
 };
 static_assert(TcK<1>::SLAB == 2 * kTcSlabHalves && TcK<2>::SLAB == 4 * kTcSlabHalves, "slab size");
 constexpr int TC_WAIT_LIMIT = 1 << 24;  // mbarrier polls before giving up
@@ -114,6 +123,36 @@ __device__ __forceinline__ u64 tc_reduce(const uint32_t *v, u64 q, uint32_t qinv
     const uint32_t m = l0 * qinv;
     const u64 w = (u64)m * (uint32_t)q + l0;
     return (u64)m * (uint32_t)(q >> 32) + (w >> 32) + l1 + ((u64)hi << 32);
+}
+
+// The same recombination for moduli r = 2^b - c.  Neighbouring sums pair up in
+// 32 bits, a_{2i} = P_{2i} + P_{2i+1} 2^W (W = 9: at most 9*7*255*511*513 <
+// 2^32; W = 8 and up to 36 sources in NS accumulators: 36*7*255*255*257 < 2^32;
+// the shifted accumulator's bias, NS * 75 * 2^24 << W, vanishes modulo 2^32, so
+// one constant per pair takes the bias out), and the bits of S from b up are
+// multiplied by c:
+//   W = 9: S = a01 + a23 2^18 + a45 2^36,
+//   W = 8: S = a01 + a23 2^16 + (a45 + P_6 2^16) 2^32.
+// Outputs are below 4r (tc_pm_ok, checked for the set on the host).  15-17
+// instructions an output against 35 for the Montgomery form (ModUp conversion of
+// 16 key switches, N = 2^16, 24 + 8 primes, 3 digits: 235 -> 219 us).
+template <int W, int NS>
+__device__ __forceinline__ u64 tc_reduce_pm(const uint32_t *v, uint32_t c, int b)
+{
+    constexpr uint32_t B = NS * 0x4B000000u;
+    const uint32_t a01 = v[0] - B + (v[1] << W);
+    const uint32_t a23 = v[2] - B + (v[3] << W);
+    const uint32_t a45 = v[4] - B + (v[5] << W);
+    if constexpr (W == 9) {
+        const u64 x = mul_wide(a23, 1u << 18);
+        const uint32_t hi = (uint32_t)(x >> 32) + ((a45 & ((1u << (b - 36)) - 1)) << 4);
+        return mad_wide(a45 >> (b - 36), c, ((u64)hi << 32) | (uint32_t)x) + a01;
+    } else {
+        const u64 u = mul_wide(v[6] - B, 1u << 16) + a45;
+        const u64 x = mul_wide(a23, 1u << 16);
+        const uint32_t hi = (uint32_t)(x >> 32) + ((uint32_t)u & ((1u << (b - 32)) - 1));
+        return mad_wide((uint32_t)(u >> (b - 32)), c, ((u64)hi << 32) | (uint32_t)x) + a01;
+    }
 }
 
 // 16 consecutive accumulator columns of this warp's 32 lanes (no wait).
@@ -219,116 +258,120 @@ __device__ __forceinline__ void mbar_arrive(uint32_t a)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
 }
-__device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-// OR of a flag over the 256 producer threads (named barrier 1 with reduction).
-__device__ __forceinline__ bool producers_or(bool f)
+// OR of a flag over the threads of a named barrier.
+template <int ID, int COUNT>
+__device__ __forceinline__ bool bar_or(bool f)
 {
     uint32_t r;
     asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}"
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
         : "=r"(r)
-        : "r"((uint32_t)f)
+        : "r"((uint32_t)f), "n"(ID), "n"(COUNT)
         : "memory");
     return r != 0;
 }
 
-constexpr int TC_PROD = 256;                  // producer threads (warps 0-7): two per tile row
+constexpr int TC_PROD = 256;                  // producer threads (warps 0-7): two groups, one thread per tile row
 constexpr int TC_CONS_WARPS = 16;             // consumer warps: 4 lane quarters x 4 target groups
 constexpr int TC_PIPE_THREADS = TC_PROD + 32 * TC_CONS_WARPS;
+constexpr int TC_TILE_COST = 18;              // work of an A tile in epilogues of one target (TcSplit)
 constexpr uint32_t TC_PIPE_COLS = 512;        // two accumulators of 256 columns
 
-// Half H of A-tile row m: K chunks CH*H..CH*H+CH-1 (CH = 4*KB chunks of 8
-// columns) from the sources they touch, y[u] = source SB + u with SB =
-// 8*CH*H/7 (zero past the item's sources).  Column K-1 is the bias.
-template <int KB, int H>
-struct TcHalf {
-    static constexpr int SB = 8 * 4 * KB * H / 7;                          // first source
-    static constexpr int LAST = H == 1 ? 64 * KB - 2 : 8 * 4 * KB * (H + 1) - 1;  // last slice column
-    static_assert(LAST / 7 - SB < TcK<KB>::NSV, "source words of a half row");
-};
-template <int KB, int H>
-__device__ __forceinline__ void tc_build_half(unsigned char *sa, int m, const u64 (&y)[TcK<KB>::NSV])
+// Row m of an A tile from its sources' words (zero past the item's sources):
+// column 7i + a = byte a of source i, the last column the bias.
+template <int KB>
+__device__ __forceinline__ void tc_build_row(unsigned char *sa, int m, const u64 (&y)[TcK<KB>::SRC])
 {
-    constexpr int CH = 4 * KB, SB = TcHalf<KB, H>::SB, NSV = TcK<KB>::NSV, K = TcK<KB>::K;
-    uint32_t wd[2 * NSV];
+    constexpr int K = TcK<KB>::K;
+    constexpr int SRC = TcK<KB>::SRC;  // with two K blocks column 126 is spare (0)
 #pragma unroll
-    for (int u = 0; u < NSV; ++u) {
-        wd[2 * u] = (uint32_t)y[u];
-        wd[2 * u + 1] = (uint32_t)(y[u] >> 32);
-    }
-#pragma unroll
-    for (int c = CH * H; c < CH * H + CH; ++c) {
+    for (int c = 0; c < K / 8; ++c) {
         uint32_t w[4];
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
             const int k0 = 8 * c + e, k1 = k0 + 1;
-            const int u0 = k0 / 7 - SB, a0 = k0 % 7, u1 = k1 / 7 - SB, a1 = k1 % 7;
-            if (k1 == K - 1)  // the last slice byte, then the bias 2048 (f16 0x6800)
-                w[e / 2] = (f16x2_bytes(wd[2 * u0 + a0 / 4], 0u, (uint32_t)(a0 % 4), 0u) & 0xFFFFu) | 0x68000000u;
-            else
-                w[e / 2] = f16x2_bytes(wd[2 * u0 + a0 / 4], wd[2 * u1 + a1 / 4], (uint32_t)(a0 % 4), (uint32_t)(a1 % 4));
+            const int a0 = k0 % 7, a1 = k1 % 7;
+            const uint32_t x0 = k0 / 7 < SRC ? (uint32_t)(y[k0 / 7 < SRC ? k0 / 7 : 0] >> (32 * (a0 / 4))) : 0u;
+            if (k1 == K - 1) {  // the last slice byte, then the bias 2048 (f16 0x6800)
+                w[e / 2] = (f16x2_bytes(x0, 0u, (uint32_t)(a0 % 4), 0u) & 0xFFFFu) | 0x68000000u;
+            } else {
+                const uint32_t x1 = (uint32_t)(y[k1 / 7] >> (32 * (a1 / 4)));  // k1 < K - 1: a source's byte
+                w[e / 2] = f16x2_bytes(x0, x1, (uint32_t)(a0 % 4), (uint32_t)(a1 % 4));
+            }
         }
         *reinterpret_cast<uint4 *>(sa + tc_off<KB>(m, 8 * c)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
-// Walks a CTA's contiguous run of items: (xt, r) advance without divisions and
-// the item is decoded again only when its (job block, target block) changes.
-template <int MODE>
-struct TcCursor {
-    int xt, r, XT, TBN, TB;
-    TcItem it;
-    __device__ __forceinline__ void start(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, int item, int XT_,
-                                          int TBN_, int TB_)
-    {
-        XT = XT_;
-        TBN = TBN_;
-        TB = TB_;
-        xt = item % XT;
-        r = item / XT;
-        it = tc_item<MODE>(T, bu, bd, item, XT, TBN, TB);
-    }
-    __device__ __forceinline__ void next(const Tables &T, const BUpJobs &bu, const BDnJobs &bd)
-    {
-        if (++xt == XT) {
-            xt = 0;
-            ++r;
-            it = tc_item<MODE>(T, bu, bd, r * XT, XT, TBN, TB);
-        } else {
-            it.src += TC_M;
-            it.dst0 += TC_M;
-        }
-    }
+// Runs of items per CTA with about equal work: items of job j cost w[j] (their
+// targets plus the cost of building an A tile); cpre are the costs of the jobs
+// before, ipre their items.  Equal counts instead left the CTAs that drew the
+// top-level jobs of a mixed batch working alone at the end.
+struct TcSplit {
+    int n;
+    uint32_t cpre[kMaxBatch + 1];
+    int ipre[kMaxBatch + 1];
+    uint16_t w[kMaxBatch];
 };
+__device__ __forceinline__ int tc_run_start(const TcSplit &sp, int cta, int ctas)
+{
+    if (cta >= ctas) return sp.ipre[sp.n];
+    const uint32_t at = (uint32_t)((u64)sp.cpre[sp.n] * (uint32_t)cta / (uint32_t)ctas);
+    int lo = 0, hi = sp.n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (sp.cpre[mid] <= at)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return sp.ipre[lo] + (int)((at - sp.cpre[lo]) / sp.w[lo]);
+}
 
 // Persistent pipelined base conversion: each CTA (one per SM) takes a
-// contiguous run of items.  Producer warps load the next item's sources into
-// registers while they build the current A tile, then one thread issues the
-// MMAs into the accumulator buffer of the item (two buffers alternate) and
-// commits them to acc_full; consumer warps wait on acc_full, run the
-// epilogue and release the buffer through acc_empty.  Every wait is bounded:
-// on timeout the kernel sets g_tc_error and its threads leave their loops.
-template <int MODE, int KB, int W>
+// contiguous run of items.  For every stretch of items that differ only in
+// their coefficients, the producer warps stage the B slabs and the targets'
+// outputs and constants once.  Two producer groups of 128 threads, a thread per
+// tile row, take the stretch's items in turn, each with its own A tiles and
+// accumulator buffer: build the A tile from the sources in registers, issue the
+// loads of the group's next item, then one thread issues the MMAs and commits
+// them to acc_full.  Consumer warps wait on acc_full, run the epilogue and
+// release the buffer through acc_empty; an item of no targets ends them.  Every
+// wait is bounded: on timeout the kernel sets g_tc_error and its threads leave
+// their loops.
+// What bounds it: the consumers' integer work at 24 targets an item (some 50
+// cycles of a scheduler an output, six warps each), the producers' chain (source
+// loads, tile, fence, barrier, issue) at few.  Measured for the ModUp conversion
+// of 16 key switches at N = 2^16 (24576 items of 24 targets): one group of 256
+// threads that fetched the targets' constants for every item 219 us (the load's
+// 700 cycles in its serial chain), targets staged once a stretch 193, two groups
+// 169.  More overlap only added instructions: consumers split between the
+// buffers 180, four half-item buffers 176, a warp of its own for the issue 182,
+// sources copied three items ahead 173.
+// KB: K blocks of an A tile; NS: A tiles (and accumulators) an item; PM: the
+// set's moduli are 2^b - c, b = T.tc_pm_b (tc_reduce_pm).
+template <int MODE, int KB, int NS, int W, bool PM>
 __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJobs bu, BDnJobs bd, const uint4 *slabs,
-                                                                int XT, int TBN, int TB, int items)
+                                                                int XT, int TBN, int TB, TcSplit split)
 {
-    constexpr int K = TcK<KB>::K, NSV = TcK<KB>::NSV;
+    constexpr int K = TcK<KB>::K, ATILE = TcK<KB>::ATILE, SLAB = TcK<KB>::SLAB;
+    constexpr int TBM = TcTargets<NS>::N;
     extern __shared__ unsigned char tc_dyn[];
-    unsigned char *sa0 = tc_dyn + ((128 - (smem_u32(tc_dyn) & 127)) & 127);
-    unsigned char *sb = sa0 + 2 * TC_M * K * 2;
+    unsigned char *sa0 = tc_dyn + ((128 - (smem_u32(tc_dyn) & 127)) & 127);  // [2 buffers][NS] A tiles
+    unsigned char *sb = sa0 + 2 * NS * ATILE;                               // [NS][TBM] B slabs
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
     __shared__ uint32_t tbase_s;
-    __shared__ u64 *s_dst[2][TC_TB];
-    __shared__ u64 s_q[2][TC_TB], s_mont[2][TC_TB];
-    __shared__ int s_G[2];
-    const int per = (items + gridDim.x - 1) / gridDim.x;
-    const int i0 = blockIdx.x * per, i1 = min(items, i0 + per);
+    __shared__ u64 *s_dst[TBM];       // output of each target at the stretch's first coefficient
+    __shared__ u64 s_q[TBM];
+    __shared__ uint32_t s_red[TBM];   // -q^-1 mod 2^32, or c (PM)
+    __shared__ int s_G[2], s_off[2];  // of the item in each buffer: targets, coefficients past the stretch's first
+    const int i0 = tc_run_start(split, blockIdx.x, gridDim.x), i1 = tc_run_start(split, blockIdx.x + 1, gridDim.x);
     if (i0 >= i1) return;
     const size_t N = (size_t)1 << T.logN;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     if (tid == 0) {
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&acc_full[b]), 2);              // MMA commit + producer release of the targets
+            mbar_init(smem_u32(&acc_full[b]), 2);              // MMA commit + producer release of the item
             mbar_init(smem_u32(&acc_empty[b]), TC_CONS_WARPS);  // one arrival per consumer warp
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -345,110 +388,138 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
 
     if (tid < TC_PROD) {
         // ------------------------------------------------------------ producers
-        const int m = tid % TC_M, h = tid / TC_M;  // row m, half h of its K columns
-        const int sb0 = h == 0 ? TcHalf<KB, 0>::SB : TcHalf<KB, 1>::SB;  // first source of the half
-        int k = 0, cur_r = -1;
-        TcCursor<MODE> cur, nxt;
-        nxt.start(T, bu, bd, i0, XT, TBN, TB);
-        u64 y[NSV];
-#pragma unroll
-        for (int u = 0; u < NSV; ++u)
-            y[u] = (nxt.it.G > 0 && sb0 + u < nxt.it.nsrc) ? nxt.it.src[(size_t)(sb0 + u) * N + m] : 0;
+        const int m = tid % TC_M, grp = tid / TC_M;  // tile row, group (items and buffer of this parity)
+        const uint32_t full = smem_u32(&acc_full[grp]), empty = smem_u32(&acc_empty[grp]);
+        unsigned char *sa = sa0 + grp * (NS * ATILE);
+        int k0 = 0;  // items before the stretch
         bool ok = true;
-        for (int item = i0; item < i1; ++item) {
-            cur = nxt;
-            u64 yc[NSV];
-#pragma unroll
-            for (int u = 0; u < NSV; ++u) yc[u] = y[u];
-            if (item + 1 < i1) {  // the next item's sources are in flight while this one is built
-                nxt.next(T, bu, bd);
-#pragma unroll
-                for (int u = 0; u < NSV; ++u)
-                    y[u] = (nxt.it.G > 0 && sb0 + u < nxt.it.nsrc) ? nxt.it.src[(size_t)(sb0 + u) * N + m] : 0;
-            }
-            const TcItem &it = cur.it;
+        for (int item = i0; item < i1;) {
+            const TcItem it = tc_item<MODE>(T, bu, bd, item, XT, TBN, TB);
+            const int n = min(i1 - item, XT - item % XT);
+            item += n;
             if (it.G == 0) continue;
-            const int buf = k & 1;
-            const bool restage = cur.r != cur_r;
-            bool bad = false;
-            // the accumulator and A tile of this buffer were last used by item k-2
-            if (k >= 2) bad = !tc_wait(smem_u32(&acc_empty[buf]), (uint32_t)(((k >> 1) - 1) & 1));
-            // new targets: every earlier MMA must be done with the B slabs
-            if (!bad && restage && k >= 1) bad = !tc_wait(smem_u32(&acc_empty[buf ^ 1]), (uint32_t)(((k - 1) >> 1) & 1));
-            if (producers_or(bad)) {
+            // new targets: every earlier item must be done with the slabs and tables
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int used = (k0 + 1 - b) >> 1;  // items that took buffer b
+                ok = ok && (used == 0 || tc_wait(smem_u32(&acc_empty[b]), (uint32_t)((used - 1) & 1)));
+            }
+            if (bar_or<3, TC_PROD>(!ok)) {
                 ok = false;
                 break;
             }
-            if (restage) {
+            {
                 // G slabs, and a zero slab after an odd G (the MMA's N is a
                 // multiple of 16 columns: two targets)
-                constexpr int W = TcK<KB>::SLAB / 16;
+                constexpr int WS = SLAB / 16;
                 const int Gp = (it.G + 1) & ~1;
-                for (int idx = tid; idx < Gp * W; idx += TC_PROD) {
-                    const int g = idx / W, w = idx % W;
+                for (int idx = tid; idx < Gp * NS * WS; idx += TC_PROD) {
+                    const int g = idx / (NS * WS), w = idx % (NS * WS);
                     uint4 val = make_uint4(0u, 0u, 0u, 0u);
                     if (g < it.G) {
                         int t, tf, slab;
                         tc_target<MODE>(T, it, g, t, tf, slab);
-                        val = slabs[(size_t)slab * W + w];
+                        val = slabs[(size_t)slab * (NS * WS) + w];
                     }
-                    reinterpret_cast<uint4 *>(sb)[idx] = val;
+                    reinterpret_cast<uint4 *>(sb + ((w / WS) * TBM + g) * SLAB)[w % WS] = val;
                 }
-                cur_r = cur.r;
             }
-            unsigned char *sa = sa0 + buf * (TC_M * K * 2);
-            // A tile: row m, columns 7i+a = byte a of source i (f16); column 63 =
-            // 2048, the bias with the slabs' 4096 there.  Sources past nsrc are 0.
-            if (h == 0)
-                tc_build_half<KB, 0>(sa, m, yc);
-            else
-                tc_build_half<KB, 1>(sa, m, yc);
-            if (h == 0 && m < it.G) {
+            if (tid < it.G) {
                 int t, tf, slab;
-                tc_target<MODE>(T, it, m, t, tf, slab);
-                s_dst[buf][m] = it.dst0 + (size_t)(t - it.t_base) * N;
-                s_q[buf][m] = T.modc[tf].q;
-                s_mont[buf][m] = T.modc[tf].mont;
+                tc_target<MODE>(T, it, tid, t, tf, slab);
+                s_dst[tid] = it.dst0 + (size_t)(t - it.t_base) * N;
+                if (!PM) s_q[tid] = T.modc[tf].q;
+                s_red[tid] = PM ? T.modc[tf].pm_c2 >> 1 : (uint32_t)T.modc[tf].mont;
             }
-            if (tid == 0) s_G[buf] = it.G;
+            // the slabs' writes ordered before the other group's MMAs too
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            producers_sync();
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t idesc = tc_idesc(8 * ((it.G + 1) & ~1));
-                const uint32_t dcol = tbase + (uint32_t)(buf * 256);
+            bar_or<3, TC_PROD>(false);
+            int k = k0 + ((k0 ^ grp) & 1);  // the group's first item of the stretch
+            const u64 *src = it.src + (size_t)(k - k0) * TC_M + m;
+            u64 y[TcK<KB>::SRC];
+            auto load = [&](int s) {
 #pragma unroll
-                for (int kk = 0; kk < K / 16; ++kk) {
-                    const uint64_t ad = tc_desc<KB>(smem_u32(sa) + kk * 2 * TC_LBO);
-                    const uint64_t bdsc = tc_desc<KB>(smem_u32(sb) + kk * 2 * TC_LBO);
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dcol),
-                        "l"(ad), "l"(bdsc), "r"(idesc), "r"((uint32_t)kk));
+                for (int u = 0; u < TcK<KB>::SRC; ++u) {
+                    const int i = s * TcK<KB>::SRC + u;
+                    y[u] = i < it.nsrc ? src[(size_t)i * N] : 0;
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&acc_full[buf]))
-                             : "memory");
-                mbar_arrive(smem_u32(&acc_full[buf]));  // releases s_dst/s_q/s_mont/s_G of this buffer
+            };
+            if (k < k0 + n) load(0);
+            for (; k < k0 + n; k += 2) {
+                // the accumulators and A tiles of this buffer were last used by item k-2
+                const int used = k >> 1;
+                ok = used == 0 || tc_wait(empty, (uint32_t)((used - 1) & 1));
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    tc_build_row<KB>(sa + s * ATILE, m, y);
+                    if (s + 1 < NS) load(s + 1);
+                }
+                if (k + 2 < k0 + n) {  // in flight while this item is issued and the buffer awaited
+                    src += 2 * TC_M;
+                    load(0);
+                }
+                if (m == 0) {
+                    s_G[grp] = it.G;
+                    s_off[grp] = (k - k0) * TC_M;
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (grp == 0 ? bar_or<1, TC_M>(!ok) : bar_or<2, TC_M>(!ok)) {
+                    ok = false;
+                    break;
+                }
+                if (m == 0) {
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t idesc = tc_idesc(8 * ((it.G + 1) & ~1));
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        const uint32_t dcol = tbase + (uint32_t)(grp * 256 + s * 8 * TBM);
+#pragma unroll
+                        for (int kk = 0; kk < K / 16; ++kk) {
+                            const uint64_t ad = tc_desc<KB>(smem_u32(sa + s * ATILE) + kk * 2 * TC_LBO);
+                            const uint64_t bdsc = tc_desc<KB>(smem_u32(sb + s * TBM * SLAB) + kk * 2 * TC_LBO);
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dcol),
+                                "l"(ad), "l"(bdsc), "r"(idesc), "r"((uint32_t)kk));
+                        }
+                    }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(full)
+                                 : "memory");
+                    mbar_arrive(full);  // releases the targets' tables and the item's G and offset
+                }
             }
-            ++k;
+            k0 += n;
         }
-        if (!ok && tid == 0) {
-            atomicExch(&g_tc_error, 1);
-            // once more, bounded, for the last MMAs still in flight before the memory is freed
-            if (k >= 1) tc_wait(smem_u32(&acc_full[(k - 1) & 1]), (uint32_t)(((k - 1) >> 1) & 1));
+        const bool mine = (k0 & 1) == grp;  // the group whose buffer comes next
+        const int used = (k0 + 1 - grp) >> 1;
+        if (m == 0) {
+            // the consumers' end: an item of no targets, once its buffer is free
+            if (ok && mine && used > 0) ok = tc_wait(empty, (uint32_t)((used - 1) & 1));
+            if (ok && mine) {
+                s_G[grp] = 0;
+                mbar_arrive(full);
+                mbar_arrive(full);
+            }
+            if (!ok) {
+                atomicExch(&g_tc_error, 1);
+                // bounded waits for MMAs still in flight before the memory is freed
+                tc_wait(full, 0);
+                tc_wait(full, 1);
+            }
         }
     } else {
         // ------------------------------------------------------------ consumers
         const int cw = warp - TC_PROD / 32, quarter = cw % 4, part = cw / 4;
         const int row = quarter * 32 + lane;
-        int k = 0;
+        const uint32_t tq = tbase + ((uint32_t)(quarter * 32) << 16);
         bool ok = true;
-        TcCursor<MODE> cur;
-        cur.start(T, bu, bd, i0, XT, TBN, TB);
-        for (int item = i0; item < i1; ++item) {
-            if (item > i0) cur.next(T, bu, bd);
-            if (cur.it.G == 0) continue;
+        auto reduce = [&](const uint32_t *v, int g) {
+            if constexpr (PM)
+                return tc_reduce_pm<W, NS>(v, s_red[g], T.tc_pm_b);
+            else
+                return tc_reduce<W>(v, s_q[g], s_red[g]);
+        };
+        for (int k = 0;; ++k) {
             const int buf = k & 1;
             const bool got = tc_wait(smem_u32(&acc_full[buf]), (uint32_t)((k >> 1) & 1));
             if (__any_sync(0xffffffffu, !got)) {  // the warp's lanes agree (tcgen05.ld is warp-collective)
@@ -457,28 +528,35 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
             }
             asm volatile("tcgen05.fence::after_thread_sync;");
             const int G = s_G[buf], NP = (G + 1) / 2;
+            if (G == 0) break;
+            const int at = s_off[buf] + row;
             // target pairs (2p, 2p+1: 16 columns) strided over the four warps
             // of a lane quarter, two tensor-memory loads in flight per wait
-            for (int p = part; p < NP; p += 8) {
-                const bool two = p + 4 < NP;
+            for (int p = part; p < NP; p += NS == 1 ? 8 : 4) {
                 uint32_t v[16], w[16];
-                const uint32_t taddr = tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + 16 * p);
+                const uint32_t taddr = tq + (uint32_t)(buf * 256 + 16 * p);
+                const bool two = NS == 1 && p + 4 < NP;
                 tmem_ld16(taddr, v);
-                if (two) tmem_ld16(taddr + 64, w);
+                if (NS == 2)
+                    tmem_ld16(taddr + 8 * TBM, w);
+                else if (two)
+                    tmem_ld16(taddr + 64, w);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (NS == 2) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] += w[i];
+                }
                 const int g = 2 * p;
-                s_dst[buf][g][row] = tc_reduce<W>(v, s_q[buf][g], (uint32_t)s_mont[buf][g]);
-                if (g + 1 < G) s_dst[buf][g + 1][row] = tc_reduce<W>(v + 8, s_q[buf][g + 1], (uint32_t)s_mont[buf][g + 1]);
+                s_dst[g][at] = reduce(v, g);
+                if (g + 1 < G) s_dst[g + 1][at] = reduce(v + 8, g + 1);
                 if (two) {
-                    s_dst[buf][g + 8][row] = tc_reduce<W>(w, s_q[buf][g + 8], (uint32_t)s_mont[buf][g + 8]);
-                    if (g + 9 < G)
-                        s_dst[buf][g + 9][row] = tc_reduce<W>(w + 8, s_q[buf][g + 9], (uint32_t)s_mont[buf][g + 9]);
+                    s_dst[g + 8][at] = reduce(w, g + 8);
+                    if (g + 9 < G) s_dst[g + 9][at] = reduce(w + 8, g + 9);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&acc_empty[buf]));
-            ++k;
         }
         if (!ok && lane == 0) atomicExch(&g_tc_error, 1);
     }
@@ -487,19 +565,20 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(TC_PIPE_COLS));
 }
 
-// Dynamic shared memory: two A tiles (16 KB each) and up to 16 B slabs
-// (32 KB), padded so that one CTA holds an SM (it takes all 512 columns of
-// tensor memory).
-// With two K blocks: two 32 KB A tiles and up to 32 slabs of 2 KB.
-template <int KB> constexpr int tc_pipe_smem() { return KB == 1 ? 120 * 1024 : 132 * 1024; }
-static_assert(tc_pipe_smem<1>() >= 2 * TC_M * TcK<1>::K * 2 + TC_TB * TcK<1>::SLAB + 128, "tile space");
-static_assert(tc_pipe_smem<2>() >= 2 * TC_M * TcK<2>::K * 2 + TC_TB * TcK<2>::SLAB + 128, "tile space");
+// Dynamic shared memory: two buffers of NS A tiles (16 KB, or 32 KB with two K
+// blocks) and the B slabs (1 or 2 KB a target and tile), padded so that one CTA
+// holds an SM (it takes all 512 columns of tensor memory).
+template <int KB, int NS> constexpr int tc_pipe_smem()
+{
+    return std::max(120 * 1024, 2 * NS * TcK<KB>::ATILE + NS * TcTargets<NS>::N * TcK<KB>::SLAB + 128);
+}
+static_assert(tc_pipe_smem<2, 2>() <= 200 * 1024, "shared memory of an SM");
 
 }  // namespace
 
 bool bconv_tc_supported(const Tables &T, int nsrc)
 {
-    return nsrc <= 18 && (((size_t)1 << T.logN) % (size_t)TC_M) == 0;
+    return nsrc <= tc_max_sources(T.tc_pm_b) && (((size_t)1 << T.logN) % (size_t)TC_M) == 0;
 }
 
 static int sm_count()
@@ -513,25 +592,60 @@ static int sm_count()
     return n;
 }
 
-template <int MODE, int KB, int W>
-static int launch_tc(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, int span, int Z, const uint4 *slabs,
-                     cudaStream_t st, const char *name)
+template <int MODE, int KB, int NS, int W, bool PM>
+static int launch_tc(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, int span, const uint4 *slabs, cudaStream_t st,
+                     const char *name)
 {
-    // target blocks of equal size (at most 32): 38 targets run as 19 + 19
-    const int TBN = (span + TC_TB - 1) / TC_TB;
+    // target blocks of equal size (at most 32, or 16 with two tiles): 38 targets run as 19 + 19
+    constexpr int TBM = TcTargets<NS>::N;
+    const int TBN = (span + TBM - 1) / TBM;
     const int TB = (span + TBN - 1) / TBN;
     static std::atomic<uint64_t> attr{0};
     once_per_device(attr, [] {
-        cudaFuncSetAttribute(k_bconv_tc<MODE, KB, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_pipe_smem<KB>());
+        cudaFuncSetAttribute(k_bconv_tc<MODE, KB, NS, W, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc_pipe_smem<KB, NS>());
     });
     const int XT = (int)(((size_t)1 << T.logN) / TC_M);
-    const long long items = (long long)XT * TBN * Z;
-    if (items <= 0) return KS_OK;
-    const int grid = (int)std::min<long long>(items, sm_count());
-    KS_LAUNCH(st, name, (k_bconv_tc<MODE, KB, W><<<grid, TC_PIPE_THREADS, tc_pipe_smem<KB>(), st>>>(T, bu, bd, slabs, XT,
-                                                                                                 TBN, TB, (int)items)));
+    // Cost of an item: its targets' epilogues plus the A tile, averaged over the
+    // job's target blocks (measured 0.46 us + 0.0245 us a target: 18 targets' worth).
+    TcSplit sp;
+    sp.n = MODE == 0 ? bu.n : bd.n;
+    u64 cost = 0, items = 0;  // at most 64 jobs x 64 digits x 1024 tiles x 6 blocks of cost 50: below 2^31
+    for (int j = 0; j < sp.n; ++j) {
+        const int z = MODE == 0 ? bu.zpre[j + 1] - bu.zpre[j] : bd.zpre[j + 1] - bd.zpre[j];
+        const int targets = MODE == 0 ? bu.job[j].t_end - bu.job[j].t_begin : bd.job[j].nact;
+        sp.w[j] = (uint16_t)(std::min(targets / TBN, TB) + TC_TILE_COST);
+        sp.cpre[j] = (uint32_t)cost;
+        sp.ipre[j] = (int)items;
+        items += (u64)XT * TBN * z;
+        cost += (u64)XT * TBN * z * sp.w[j];
+    }
+    if (items == 0) return KS_OK;
+    sp.cpre[sp.n] = (uint32_t)cost;
+    sp.ipre[sp.n] = (int)items;
+    const int grid = (int)std::min<u64>(items, (u64)sm_count());
+    constexpr int SM = tc_pipe_smem<KB, NS>();
+    KS_LAUNCH(st, name,
+              (k_bconv_tc<MODE, KB, NS, W, PM><<<grid, TC_PIPE_THREADS, SM, st>>>(T, bu, bd, slabs, XT, TBN, TB, sp)));
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? KS_OK : fail(KS_ECUDA, std::string(name) + " (tensor cores) launch: " + cudaGetErrorString(e));
+}
+
+// The kernel of a conversion with nsrc sources.
+template <int MODE>
+static int launch_tc_for(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, int nsrc, int span, const uint4 *slabs,
+                         cudaStream_t st, const char *name)
+{
+    const int kb = tc_kblocks(nsrc), bits = tc_slice_bits(kb, T.tc_below54);
+    if (MODE == 0 ? T.tc_pm_up : T.tc_pm_dn) {
+        if (kb == 4) return launch_tc<MODE, 2, 2, 8, true>(T, bu, bd, span, slabs, st, name);
+        if (kb == 2) return launch_tc<MODE, 2, 1, 8, true>(T, bu, bd, span, slabs, st, name);
+        return bits == 9 ? launch_tc<MODE, 1, 1, 9, true>(T, bu, bd, span, slabs, st, name)
+                         : launch_tc<MODE, 1, 1, 8, true>(T, bu, bd, span, slabs, st, name);
+    }
+    if (kb == 2) return launch_tc<MODE, 2, 1, 8, false>(T, bu, bd, span, slabs, st, name);
+    return bits == 9 ? launch_tc<MODE, 1, 1, 9, false>(T, bu, bd, span, slabs, st, name)
+                     : launch_tc<MODE, 1, 1, 8, false>(T, bu, bd, span, slabs, st, name);
 }
 
 int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, const int *, cudaStream_t st)
@@ -551,9 +665,7 @@ int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, co
     none.n = 0;
     Tables Tt = T;
     Tt.up_tc = slabs;
-    if (tc_kblocks(T.alpha) == 2) return launch_tc<0, 2, 8>(Tt, b, none, span, b.zpre[b.n], slabs, st, "bconv_up");
-    return tc_slice_bits(1, T.tc_below54) == 9 ? launch_tc<0, 1, 9>(Tt, b, none, span, b.zpre[b.n], slabs, st, "bconv_up")
-                                               : launch_tc<0, 1, 8>(Tt, b, none, span, b.zpre[b.n], slabs, st, "bconv_up");
+    return launch_tc_for<0>(Tt, b, none, T.alpha, span, slabs, st, "bconv_up");
 }
 
 int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, const uint4 *slabs, cudaStream_t st)
@@ -563,9 +675,7 @@ int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, const uint4 *slabs, 
     if (span <= 0) return KS_OK;
     BUpJobs none;
     none.n = 0;
-    if (tc_kblocks(T.kp) == 2) return launch_tc<1, 2, 8>(T, none, b, span, b.zpre[b.n], slabs, st, "bconv_down");
-    return tc_slice_bits(1, T.tc_below54) == 9 ? launch_tc<1, 1, 9>(T, none, b, span, b.zpre[b.n], slabs, st, "bconv_down")
-                                               : launch_tc<1, 1, 8>(T, none, b, span, b.zpre[b.n], slabs, st, "bconv_down");
+    return launch_tc_for<1>(T, none, b, T.kp, span, slabs, st, "bconv_down");
 }
 
 int tc_error_flag(bool clear)
@@ -584,18 +694,19 @@ int tc_error_flag(bool clear)
 
 // Host: the B slab of one target of modulus r: rows b (slice b of the
 // folded constant, W bits; rows past the slices zero), columns k = 7i + a
-// (source i, byte a of y): slice b of c_i * 2^(8a) * 2^-32 mod r (c_i carries
-// 2^64, the epilogue's reduction takes 2^32 off); the last column holds the bias.
+// (source i, byte a of y): slice b of c_i * 2^(8a) mod r, times 2^32 for the
+// Montgomery epilogue; the last column holds the bias.
 template <int KB>
-static void tc_slab_kb(const std::vector<u64> &c, u64 r, int W, uint16_t *slab)
+static void tc_slab_kb(const u64 *c, int n, u64 r, int W, bool pm, uint16_t *slab)
 {
     constexpr int K = TcK<KB>::K;
     const int NSL = W == 8 ? 7 : 6;
-    const u64 inv32 = invmod_h((u64)(((unsigned __int128)1 << 32) % r), r);
+    const u64 f = pm ? 1 : (u64)(((unsigned __int128)1 << 32) % r);
+    u64 sh[7];  // 2^(8a), with the epilogue's factor
+    for (int a = 0; a < 7; ++a) sh[a] = mulmod_h(f, powmod_h(2, 8 * (u64)a, r), r);
     for (int k = 0; k < K; ++k) {
         const int i = k / 7, a = k % 7;
-        const u64 cf = (k < K - 1 && i < (int)c.size())
-                           ? mulmod_h(mulmod_h(c[i] % r, inv32, r), powmod_h(2, 8 * (u64)a, r), r) : 0;
+        const u64 cf = (k < K - 1 && i < n) ? mulmod_h(c[i], sh[a], r) : 0;
         for (int b = 0; b < 8; ++b) {
             const uint32_t sl = b < NSL ? (uint32_t)((cf >> (W * b)) & ((1u << W) - 1)) : 0u;
             // f16 of an integer below 2048
@@ -615,12 +726,27 @@ static void tc_slab_kb(const std::vector<u64> &c, u64 r, int W, uint16_t *slab)
     for (int b = 0; b < NSL; ++b) slab[tc_off<KB>(b, K - 1) / 2] = (uint16_t)((15 + 12) << 10);
 }
 
-void tc_slab(const std::vector<u64> &c, u64 r, int kblocks, int bits, uint16_t *slab)
+void tc_slab(const std::vector<u64> &c, u64 r, int kblocks, int bits, bool pm, uint16_t *slab)
 {
-    if (kblocks == 1)
-        tc_slab_kb<1>(c, r, bits, slab);
-    else
-        tc_slab_kb<2>(c, r, 8, slab);
+    const int n = (int)c.size();
+    if (kblocks == 1) {
+        tc_slab_kb<1>(c.data(), n, r, bits, pm, slab);
+    } else {
+        const int s0 = std::min(n, TcK<2>::SRC);  // sources of the first tile
+        tc_slab_kb<2>(c.data(), s0, r, 8, pm, slab);
+        if (kblocks == 4) tc_slab_kb<2>(c.data() + s0, n - s0, r, 8, pm, slab + TcK<2>::SLAB / 2);
+    }
+}
+
+// Whether tc_reduce_pm's output stays below 4q (the NTT's input bound) for
+// moduli q = 2^b - c, c at most cmax.
+bool tc_pm_ok(int bits, int b, u64 cmax)
+{
+    typedef unsigned __int128 u128;
+    const u128 q4 = 4 * (((u128)1 << b) - cmax), word = (u128)1 << 32;
+    if (bits == 9)
+        return b >= 40 && b <= 54 && word + (word << 18) + ((u128)1 << b) + (((word - 1) >> (b - 36)) * cmax) < q4;
+    return b >= 40 && b <= 56 && word + (word << 16) + ((u128)1 << b) + (((word << 8) + word) >> (b - 32)) * cmax < q4;
 }
 
 }  // namespace ks

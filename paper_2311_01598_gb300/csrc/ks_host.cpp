@@ -365,8 +365,8 @@ int build_tables(ks_params *P)
             dn[(size_t)k * P->nq + i] = split28(to_mont(invmod_h(P->p[k] % P->q[i], P->q[i]), P->q[i]));
 
     // tensor-core base conversion: one B slab per (digit j, active towers a,
-    // full tower t) for ModUp and per Q tower for ModDown (<= 18 sources; one
-    // K block of 64 slice columns up to 9, two up to 18)
+    // full tower t) for ModUp and per Q tower for ModDown (tc_max_sources,
+    // tc_kblocks)
     std::vector<uint16_t> up_tc, dn_tc;
     std::vector<int> up_tc_lvl((size_t)P->nq * P->ndig, 0);
     const int kb_up = tc_kblocks(A), kb_dn = tc_kblocks(P->kp);
@@ -374,8 +374,17 @@ int build_tables(ks_params *P)
     for (u64 q : P->q) below54 = below54 && q < (1ull << 54);
     for (u64 p : P->p) below54 = below54 && p < (1ull << 54);
     const int bits_up = tc_slice_bits(kb_up, below54), bits_dn = tc_slice_bits(kb_dn, below54);
+    // folding epilogue: AR_PM moduli of one bit length, within its bounds
+    int pm_b = pm.use ? 31 + (int)pm.t[0].k : 0;
+    u64 cmax = 0;
+    for (int t = 0; t < nt && pm_b; ++t) {
+        if (31 + (int)pm.t[t].k != pm_b) pm_b = 0;
+        cmax = std::max(cmax, pm.t[t].c2 / 2);
+    }
+    const bool pm_up = pm_b && tc_pm_ok(bits_up, pm_b, cmax), pm_dn = pm_b && tc_pm_ok(bits_dn, pm_b, cmax);
     const size_t SLAB = (size_t)kTcSlabHalves * kb_up, DSLAB = (size_t)kTcSlabHalves * kb_dn;
-    if (A <= 18) {
+    const int max_up = pm_up ? 36 : 18, max_dn = pm_dn ? 36 : 18;
+    if (A <= max_up) {
         std::vector<int> off((size_t)P->ndig * (A + 1), -1);
         for (int j = 0; j < P->ndig; ++j) {
             int lo = j * A;
@@ -389,10 +398,10 @@ int build_tables(ks_params *P)
                         u64 hat = 1;
                         for (int k = 0; k < a; ++k)
                             if (k != i) hat = mulmod_h(hat, prim[lo + k] % r, r);
-                        c[i] = to_mont(hat, r);
+                        c[i] = hat;
                     }
                     up_tc.resize(up_tc.size() + SLAB);
-                    tc_slab(c, r, kb_up, bits_up, up_tc.data() + up_tc.size() - SLAB);
+                    tc_slab(c, r, kb_up, bits_up, pm_up, up_tc.data() + up_tc.size() - SLAB);
                 }
             }
         }
@@ -400,12 +409,12 @@ int build_tables(ks_params *P)
             for (int j = 0; j * A < nact; ++j)
                 up_tc_lvl[(size_t)(nact - 1) * P->ndig + j] = off[j * (A + 1) + std::min(A, nact - j * A)];
     }
-    if (P->kp <= 18) {
+    if (P->kp <= max_dn) {
         dn_tc.resize((size_t)P->nq * DSLAB);
         for (int i = 0; i < P->nq; ++i) {
             std::vector<u64> c(P->kp);
-            for (int k = 0; k < P->kp; ++k) c[k] = to_mont(invmod_h(P->p[k] % P->q[i], P->q[i]), P->q[i]);
-            tc_slab(c, P->q[i], kb_dn, bits_dn, dn_tc.data() + (size_t)i * DSLAB);
+            for (int k = 0; k < P->kp; ++k) c[k] = invmod_h(P->p[k] % P->q[i], P->q[i]);
+            tc_slab(c, P->q[i], kb_dn, bits_dn, pm_dn, dn_tc.data() + (size_t)i * DSLAB);
         }
     }
 
@@ -468,9 +477,10 @@ int build_tables(ks_params *P)
     T.dn_tc = P->bconv_tensor ? P->d_dn_tc : nullptr;
     T.ntt_cluster = P->ntt_cluster;
     T.row_stage = P->row_stage;
-    T.tc_below54 = 1;
-    for (u64 q : P->q) T.tc_below54 = T.tc_below54 && q < (1ull << 54);
-    for (u64 p : P->p) T.tc_below54 = T.tc_below54 && p < (1ull << 54);
+    T.tc_below54 = below54;
+    T.tc_pm_b = pm_up || pm_dn ? pm_b : 0;
+    T.tc_pm_up = pm_up;
+    T.tc_pm_dn = pm_dn;
     T.arith = pm.use ? AR_PM : sp ? AR_SP : AR_GEN;
     T.pm_fold = pm.fold;
     T.logN = P->logN;

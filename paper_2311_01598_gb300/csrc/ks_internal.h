@@ -94,6 +94,8 @@ struct Tables {
     int arith;        // butterfly form the primes allow (AR_GEN, AR_SP, AR_PM: ks_device.cuh); AR_PM sets hold
                       // tw, itw, the ModUp P1 factors and N^-1 as AR_PM pairs instead of Shoup pairs
     int pm_fold;      // AR_PM: folds the forward transforms need (PM_FOLD_*)
+    int tc_pm_b;      // tensor-core base conversion: the moduli's common bit length where its folding epilogue
+    int tc_pm_up, tc_pm_dn;  // serves the set (ModUp, ModDown; tc_reduce_pm), else 0
     int tc_below54;   // every modulus is below 2^54: 9-bit constant slices (tensor-core BConv)
     int logN;
     int nq, kp, alpha, ndig;

@@ -123,21 +123,25 @@ int launch_bconv_down(const Tables &T, const BDnJobs &b, cudaStream_t st);
 
 // Tensor-core base conversion (ks_bconv_tc.cu): same jobs and outputs as the
 // CUDA-core kernels; used by launch_bconv_up/down when the tables are present
-// and the shape is supported (at most 18 sources, N a multiple of 128).
+// and the shape is supported (at most 18 or 36 sources, N a multiple of 128).
 bool bconv_tc_supported(const Tables &T, int nsrc);
 int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, const int *slab_lvl, cudaStream_t st);
 int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, const uint4 *slabs, cudaStream_t st);
-// K blocks of 64 slice columns for nsrc sources: one up to 9, two up to 18.
-inline int tc_kblocks(int nsrc) { return nsrc <= 9 ? 1 : 2; }
+// K blocks of 64 slice columns for nsrc sources: one up to 9, two up to 18, two
+// tiles of two blocks up to 36 (with the folding epilogue only: tc_pm_b != 0).
+inline int tc_kblocks(int nsrc) { return nsrc <= 9 ? 1 : nsrc <= 18 ? 2 : 4; }
+inline int tc_max_sources(int tc_pm_b) { return tc_pm_b ? 36 : 18; }
 // Bits of the constants' slices: 9 (6 slices, partial sums below 9*7*255*511
 // < 2^23) with one K block when every modulus is below 2^54, else 8 (7).
 inline int tc_slice_bits(int kblocks, int below54) { return kblocks == 1 && below54 ? 9 : 8; }
 // Host: one B slab of kblocks KB (8 slice rows x 64*kblocks slice columns,
-// f16, canonical layout) for the constants c[0..nsrc) (carrying 2^64) of one
-// target of modulus r: row b, column 7i + a holds bit slice b (of `bits`
-// bits) of c_i * 2^(8a) * 2^-32 mod r.
+// f16, canonical layout) for the constants c[0..nsrc) of one target of modulus
+// r: row b, column 7i + a holds bit slice b (of `bits` bits) of c_i * 2^(8a)
+// mod r (pm: the folding epilogue), or of that times 2^32 (the Montgomery one).
 constexpr int kTcSlabHalves = 8 * 64;  // f16 words of a slab per K block
-void tc_slab(const std::vector<u64> &c, u64 r, int kblocks, int bits, uint16_t *slab);
+void tc_slab(const std::vector<u64> &c, u64 r, int kblocks, int bits, bool pm, uint16_t *slab);
+// Whether the folding epilogue serves moduli 2^b - c, c <= cmax, at this slice width.
+bool tc_pm_ok(int bits, int b, u64 cmax);
 // Device flag set by a tensor-core kernel whose MMA wait gave up (-1: unreadable).
 int tc_error_flag(bool clear);
 // Device flag set by a staged row pass whose bulk-copy wait gave up (-1: unreadable).
