@@ -158,7 +158,7 @@ int ks_keygen_upload(const ks_params *params, const int8_t *h_s, const int64_t *
  * Only b_j is stored (half the device memory of a full key); the kernels
  * regenerate a_j while they form the key product.  A compressed key works
  * with every entry point; Output-Centric schedules asking for the fused
- * variant run the split variant for batches that contain one. */
+ * variant run the whole-basis variant for batches that contain one. */
 int ks_keygen_upload_compressed(const ks_params *params, const int8_t *h_s, const int64_t *h_s_prime,
                                 uint64_t seed, ks_stream_t stream, ks_key **out);
 
@@ -302,14 +302,15 @@ typedef struct {
     int32_t dataflow;    /* KS_MP, KS_DC or KS_OC                                  */
     int32_t oc_variant;  /* KS_OC: 0 = fused row kernels (row pass, key product,
                             ModDown step in one kernel per row block), 1 = split
-                            (plain row pass, then a streaming combine kernel),
-                            2 = whole basis (one base conversion and one NTT
-                            launch over every raised limb, then the combines),
+                            (run as 2, which was faster in every measured
+                            shape), 2 = whole basis (one base conversion and
+                            one NTT launch over every raised limb, then
+                            streaming combine kernels),
                             3 = one thread-block-cluster kernel per output
                             tower (ModUp base conversion, NTTs, key product,
                             ModDown, subtraction with the tower's limbs on
                             chip; ring degrees with a cluster geometry and
-                            full keys, else run as 1)                          */
+                            full keys, else run as 2)                          */
     int32_t chunk;       /* KS_OC: jobs per batched launch group, 1..64           */
     int32_t order;       /* 0 = jobs in the given order, 1 = grouped by level
                             (descending), 2 = grouped by key (KS_OC: jobs of a

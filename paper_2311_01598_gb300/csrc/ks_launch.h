@@ -208,13 +208,12 @@ int check_job(const ks_params *P, const ks_key *K, uint32_t nact, const uint64_t
 // (base-conversion engine, NTT form) applied (ks_api.cu).
 Tables call_tables(const ks_params *P, const ks_schedule &sc);
 // Output-Centric variants: FUSED runs each section's row pass, key product
-// and ModDown step in one kernel per row block; SPLIT runs the row passes
-// with the plain row-pass kernel and the key product / subtraction in a
-// streaming combine kernel; WHOLE raises every digit to every tower in one
-// base-conversion launch and one NTT launch, then runs the same per-tower
-// combine kernels (special towers, ModDown, Q towers).
+// and ModDown step in one kernel per row block; WHOLE raises every digit to
+// every tower in one base-conversion launch and one NTT launch, then runs
+// streaming per-tower combine kernels (special towers, ModDown, Q towers);
+// SPLIT runs as WHOLE.
 enum { KS_OC_FUSED = 0, KS_OC_SPLIT = 1, KS_OC_WHOLE = 2, KS_OC_TOWER = 3 };
-// TOWER: the split variant's prep and special-tower section, then one
+// TOWER: prep and the special-tower section, then one
 // thread-block-cluster kernel per (job, Q output tower) that keeps the
 // tower's limbs on chip from ModUp base conversion to the ModDown
 // subtraction (ks_oc_tower.cu).  KS_EUNSUPPORTED (nothing launched) where

@@ -240,11 +240,10 @@ static int oc_rows(const Tables &T, const OcJobs &oj, bool p_section, cudaStream
     return KS_OK;
 }
 
-// ------------------------------------------------------------------ split variant
-// The same schedule with the row passes run by the plain row-pass kernel and
-// the key product / ModDown subtraction by streaming combine kernels: more
-// resident warps per SM than the fused row kernels, at the price of one more
-// round trip of the section's limbs through L2/HBM.
+// ------------------------------------------------------------------ combine kernels
+// The key product and the ModDown subtraction as streaming kernels beside the
+// plain row passes: more resident warps per SM than the fused row kernels, at
+// the price of one more round trip of the limbs through L2/HBM.
 
 // V consecutive coefficients per thread (V = 2: 16-byte loads and stores;
 // limb bases and even coefficient indices keep them aligned).
@@ -317,9 +316,8 @@ static bool any_compressed(const OcJobs &oj)
     return false;
 }
 
-// P section combine: c'_{x,p_k} = sum_j NTT(z_{j,p_k}) * evk_{j,x,p_k} for
-// every coefficient, written canonical to cp.  grid (N/(256V), jobs*K).
-template <bool CK, int V>
+// P section combine of the per-tower variant (D [nd][K], full keys): c'_{x,p_k} =
+// sum_j NTT(z_{j,p_k}) * evk_{j,x,p_k}, canonical.  grid (N/256, jobs*K).
 __global__ void __launch_bounds__(256) k_oc_comb_p(Tables T, OcJobs oj)
 {
     const int K = T.kp;
@@ -330,62 +328,15 @@ __global__ void __launch_bounds__(256) k_oc_comb_p(Tables T, OcJobs oj)
     const int nt = J.nact + K;
     const int nfull = T.nq + K;
     const size_t N = (size_t)1 << T.logN;
-    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const ModC &mc = T.modc[tf];
-    U128 sb[V], sa[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
+    U128 sb[1] = {{0, 0}}, sa[1] = {{0, 0}};
     for (int j = 0; j < J.nd; ++j) {
-        u64 x[V];
-        ldv<V>(J.tmp + (size_t)(j * K + k) * N + n, x);
-        key_macv<CK, V>(J.key, j, tf, n, nfull, T.logN, mc.q, x, sb, sa);
+        const u64 x[1] = {J.tmp[(size_t)(j * K + k) * N + n]};
+        key_macv<false, 1>(J.key, j, tf, n, nfull, T.logN, mc.q, x, sb, sa);
     }
-    u64 ob[V], oa[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        ob[c] = reduce_any(redc(sb[c], mc.q, mc.mont), mc.q, mc.one_sh);
-        oa[c] = key_a_finish<CK>(J.key, sa[c], mc, T.key_sc, tf);
-    }
-    stv<V>(J.cp + (size_t)t * N + n, ob);
-    stv<V>(J.cp + (size_t)(nt + t) * N + n, oa);
-}
-
-// Q section combine: out_x = sum_j D_j * evk_{j,x} - NTT(v_x), D_j the
-// transformed ModUp limb or the input tower for the own digit.
-// grid (N/(256V), sum of nact over jobs).
-template <bool CK, int V>
-__global__ void __launch_bounds__(256) k_oc_comb_q(Tables T, OcJobs oj)
-{
-    const int jb = find_slot(oj.pre, oj.n, blockIdx.y);
-    const OcJob &J = oj.job[jb];
-    const int t = blockIdx.y - oj.pre[jb];
-    const int nact = J.nact;
-    const int j0 = t / T.alpha;
-    const int nfull = T.nq + T.kp;
-    const size_t N = (size_t)1 << T.logN;
-    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
-    const ModC &mc = T.modc[t];
-    U128 sb[V], sa[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
-    for (int j = 0; j < J.nd; ++j) {
-        u64 x[V];
-        ldv<V>(j == j0 ? J.d + (size_t)t * N + n : J.tmp + (size_t)(j * nact + t) * N + n, x);
-        key_macv<CK, V>(J.key, j, t, n, nfull, T.logN, mc.q, x, sb, sa);
-    }
-    u64 vb[V], va[V], o0[V], o1[V];
-    ldv<V>(J.tmp + (size_t)(J.nd * nact + t) * N + n, vb);
-    ldv<V>(J.tmp + (size_t)((J.nd + 1) * nact + t) * N + n, va);
-    const u64 qlz = mc.flz;
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        const u64 cb = reduce_any(redc(sb[c], mc.q, mc.mont), mc.q, mc.one_sh);
-        const u64 ca = key_a_finish<CK>(J.key, sa[c], mc, T.key_sc, t);
-        o0[c] = reduce_any(cb + qlz - vb[c], mc.q, mc.one_sh);
-        o1[c] = reduce_any(ca + qlz - va[c], mc.q, mc.one_sh);
-    }
-    stv<V>(J.out0 + (size_t)t * N + n, o0);
-    stv<V>(J.out1 + (size_t)t * N + n, o1);
+    J.cp[(size_t)t * N + n] = reduce_any(redc(sb[0], mc.q, mc.mont), mc.q, mc.one_sh);
+    J.cp[(size_t)(nt + t) * N + n] = reduce_any(redc(sa[0], mc.q, mc.mont), mc.q, mc.one_sh);
 }
 
 // ------------------------------------------------------------------ shared keys
@@ -407,29 +358,23 @@ struct KeyGroups {
     int mem[kMaxBatch];        // job indices into the launch's OcJobs
 };
 
-// Row n of the section's limbs: WHOLE = the whole-basis layout (D
-// [nd][nact+K], then v [2][nact]); otherwise the split layout (P section D
-// [nd][K]; Q section D [nd][nact], then v [2][nact]).
-template <bool WHOLE>
+// Limbs of the whole-basis layout: D [nd][nact+K], then v [2][nact].
 __device__ __forceinline__ const u64 *p_limb(const OcJob &J, int j, int k, int K, size_t N)
 {
-    return WHOLE ? J.tmp + ((size_t)j * (J.nact + K) + J.nact + k) * N : J.tmp + ((size_t)j * K + k) * N;
+    return J.tmp + ((size_t)j * (J.nact + K) + J.nact + k) * N;
 }
-template <bool WHOLE>
 __device__ __forceinline__ const u64 *q_limb(const OcJob &J, int j, int t, int j0, int K, size_t N)
 {
     if (j == j0) return J.d + (size_t)t * N;
-    return J.tmp + ((size_t)j * (WHOLE ? J.nact + K : J.nact) + t) * N;
+    return J.tmp + ((size_t)j * (J.nact + K) + t) * N;
 }
-template <bool WHOLE>
 __device__ __forceinline__ const u64 *v_limb(const OcJob &J, int x, int t, int K, size_t N)
 {
-    const size_t base = WHOLE ? (size_t)J.nd * (J.nact + K) : (size_t)J.nd * J.nact;
-    return J.tmp + (base + (size_t)x * J.nact + t) * N;
+    return J.tmp + ((size_t)J.nd * (J.nact + K) + (size_t)x * J.nact + t) * N;
 }
 
 // P towers.  grid (N/(256V), groups*K).
-template <bool CK, bool WHOLE, int V>
+template <bool CK, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_pg(Tables T, OcJobs oj, KeyGroups kg)
 {
     const int K = T.kp;
@@ -457,7 +402,7 @@ __global__ void __launch_bounds__(256) k_oc_comb_pg(Tables T, OcJobs oj, KeyGrou
                 const OcJob &J = oj.job[kg.mem[m0 + i]];
                 if (j < J.nd) {
                     u64 x[V];
-                    ldv<V>(p_limb<WHOLE>(J, j, k, K, N) + n, x);
+                    ldv<V>(p_limb(J, j, k, K, N) + n, x);
 #pragma unroll
                     for (int c = 0; c < V; ++c) {
                         mac128(sb[i][c], x[c], kb[c]);
@@ -483,7 +428,7 @@ __global__ void __launch_bounds__(256) k_oc_comb_pg(Tables T, OcJobs oj, KeyGrou
 }
 
 // Q towers and the ModDown subtraction.  grid (N/(256V), kg.pre[kg.n]).
-template <bool CK, bool WHOLE, int V>
+template <bool CK, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGroups kg)
 {
     const int K = T.kp;
@@ -515,7 +460,7 @@ __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGrou
                 const OcJob &J = oj.job[kg.mem[m0 + i]];
                 if (J.nact > t && j < J.nd) {
                     u64 x[V];
-                    ldv<V>(q_limb<WHOLE>(J, j, t, j0, K, N) + n, x);
+                    ldv<V>(q_limb(J, j, t, j0, K, N) + n, x);
 #pragma unroll
                     for (int c = 0; c < V; ++c) {
                         mac128(sb[i][c], x[c], kb[c]);
@@ -531,8 +476,8 @@ __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGrou
             const OcJob &J = oj.job[kg.mem[m0 + i]];
             if (J.nact > t) {
                 u64 vb[V], va[V], o0[V], o1[V];
-                ldv<V>(v_limb<WHOLE>(J, 0, t, K, N) + n, vb);
-                ldv<V>(v_limb<WHOLE>(J, 1, t, K, N) + n, va);
+                ldv<V>(v_limb(J, 0, t, K, N) + n, vb);
+                ldv<V>(v_limb(J, 1, t, K, N) + n, va);
 #pragma unroll
                 for (int c = 0; c < V; ++c) {
                     const u64 cb = reduce_any(redc(sb[i][c], mc.q, mc.mont), mc.q, mc.one_sh);
@@ -586,7 +531,6 @@ static bool key_groups(const OcJobs &oj, KeyGroups &kg)
     return true;
 }
 
-template <bool WHOLE>
 static void comb_grouped(const Tables &T, const OcJobs &oj, const KeyGroups &kg, bool p_section, cudaStream_t st)
 {
     const size_t N = (size_t)1 << T.logN;
@@ -595,42 +539,16 @@ static void comb_grouped(const Tables &T, const OcJobs &oj, const KeyGroups &kg,
     if (p_section) {
         const dim3 g((unsigned)(N / (256 * V)), kg.n * T.kp);
         if (ck)
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<true, WHOLE, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<true, V><<<g, 256, 0, st>>>(T, oj, kg)));
         else
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<false, WHOLE, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<false, V><<<g, 256, 0, st>>>(T, oj, kg)));
     } else {
         const dim3 g((unsigned)(N / (256 * V)), kg.pre[kg.n]);
         if (ck)
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<true, WHOLE, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<true, V><<<g, 256, 0, st>>>(T, oj, kg)));
         else
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<false, WHOLE, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<false, V><<<g, 256, 0, st>>>(T, oj, kg)));
     }
-}
-
-static int oc_combine(const Tables &T, const OcJobs &oj, bool p_section, bool share_keys, cudaStream_t st)
-{
-    const size_t N = (size_t)1 << T.logN;
-    // Q towers: four coefficients a thread (two 16-byte accesses per
-    // stream: 0.42 ms against 0.47 ms with two at the benchmark step); the
-    // P-tower combine has few rows and keeps one (two measured slower)
-    const dim3 gp((unsigned)(N / 256), oj.n * T.kp), gq((unsigned)(N / 1024), oj.pre[oj.n]);
-    KeyGroups kg;
-    if (share_keys && key_groups(oj, kg)) {
-        comb_grouped<false>(T, oj, kg, p_section, st);
-    } else if (p_section) {
-        if (any_compressed(oj))
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_p<true, 1><<<gp, 256, 0, st>>>(T, oj)));
-        else
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_p<false, 1><<<gp, 256, 0, st>>>(T, oj)));
-    } else {
-        if (any_compressed(oj))
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_q<true, 4><<<gq, 256, 0, st>>>(T, oj)));
-        else
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_q<false, 4><<<gq, 256, 0, st>>>(T, oj)));
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC combine launch: ") + cudaGetErrorString(e));
-    return KS_OK;
 }
 
 size_t oc_scratch_words(const Tables &T, int nact)
@@ -749,10 +667,11 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     const bool ck = any_compressed(oj);
     KeyGroups kg;
     const bool grouped = share_keys && key_groups(oj, kg);
-    // Q towers four coefficients a thread, P towers one (as in oc_combine)
+    // Q towers four coefficients a thread (two 16-byte accesses per stream); the
+    // P-tower combine has few rows and keeps one (two measured slower)
     const dim3 gp((unsigned)(N / 256), n * K), gq((unsigned)(N / 1024), oj.pre[n]);
     if (grouped)  // P4+P5, P towers
-        comb_grouped<true>(T, oj, kg, true, st);
+        comb_grouped(T, oj, kg, true, st);
     else if (ck)
         KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pw<true, 1><<<gp, 256, 0, st>>>(T, oj)));
     else
@@ -761,7 +680,7 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;        // ModDown P2
     if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;    // ModDown P3
     if (grouped)  // P4+P5 Q, ModDown P4
-        comb_grouped<true>(T, oj, kg, false, st);
+        comb_grouped(T, oj, kg, false, st);
     else if (ck)
         KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qw<true, 4><<<gq, 256, 0, st>>>(T, oj)));
     else
@@ -771,9 +690,9 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     return KS_OK;
 }
 
-static int launch_oc_chunk(const Tables &T, int n, const OcJob *jobs, int variant, bool share_keys, cudaStream_t st)
+// Fused-row and per-tower variants: prep, the P section, then the Q section.
+static int launch_oc_sections(const Tables &T, int n, const OcJob *jobs, int variant, cudaStream_t st)
 {
-    if (variant == KS_OC_WHOLE) return launch_oc_whole(T, n, jobs, share_keys, st);
     const size_t N = (size_t)1 << T.logN;
     const int K = T.kp;
     int rc;
@@ -804,21 +723,19 @@ static int launch_oc_chunk(const Tables &T, int n, const OcJob *jobs, int varian
         oj.pre[i + 1] = oj.pre[i] + J.nact;
     }
     if ((rc = launch_bconv_up(T, bp, st)) != KS_OK) return rc;
-    if (variant == KS_OC_FUSED) {
-        if ((rc = launch_fwd_col(T, mp, st)) != KS_OK) return rc;
-        if ((rc = oc_rows(T, oj, true, st)) != KS_OK) return rc;
-        if ((rc = launch_inv_col(T, mw, false, st)) != KS_OK) return rc;
-    } else {
-        if ((rc = launch_ntt_fwd(T, mp, false, st)) != KS_OK) return rc;
-        if ((rc = oc_combine(T, oj, true, share_keys, st)) != KS_OK) return rc;
-        if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;
-    }
-    // 3. Q section: one cluster kernel per output tower (TOWER), else the
-    // split or fused form below
     if (variant == KS_OC_TOWER) {
-        rc = launch_oc_tower(T, oj, st);
-        if (rc != KS_EUNSUPPORTED) return rc;
+        if ((rc = launch_ntt_fwd(T, mp, false, st)) != KS_OK) return rc;
+        KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_p<<<dim3((unsigned)(N / 256), n * K), 256, 0, st>>>(T, oj)));
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC combine launch: ") + cudaGetErrorString(e));
+        if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;
+        // 3. Q section: one cluster kernel per output tower
+        return launch_oc_tower(T, oj, st);
     }
+    if ((rc = launch_fwd_col(T, mp, st)) != KS_OK) return rc;
+    if ((rc = oc_rows(T, oj, true, st)) != KS_OK) return rc;
+    if ((rc = launch_inv_col(T, mw, false, st)) != KS_OK) return rc;
+    // 3. Q section
     BUpJobs bq;
     bq.n = 0;
     BDnJobs bd;
@@ -834,33 +751,26 @@ static int launch_oc_chunk(const Tables &T, int n, const OcJob *jobs, int varian
     }
     if ((rc = launch_bconv_up(T, bq, st)) != KS_OK) return rc;
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;
-    if (variant == KS_OC_FUSED) {
-        if ((rc = launch_fwd_col(T, mq, st)) != KS_OK) return rc;
-        return oc_rows(T, oj, false, st);
-    }
-    if ((rc = launch_ntt_fwd(T, mq, false, st)) != KS_OK) return rc;
-    return oc_combine(T, oj, false, share_keys, st);
+    if ((rc = launch_fwd_col(T, mq, st)) != KS_OK) return rc;
+    return oc_rows(T, oj, false, st);
 }
 
 int launch_oc(const Tables &T, int njobs, const OcJob *jobs, int variant, cudaStream_t st, bool share_keys)
 {
-    // The tower kernel needs a ring degree with a cluster geometry and full
-    // keys; otherwise its launch group runs the split variant (same result).
-    if (variant == KS_OC_TOWER) {
-        bool ok = oc_tower_supported(T);
-        for (int i = 0; i < njobs && ok; ++i) ok = !jobs[i].key.comp;
-        if (!ok) variant = KS_OC_SPLIT;
-    }
-    // The fused row kernels read the key's a half from memory: batches with
-    // a compressed key run the split variant instead.
-    if (variant == KS_OC_FUSED)
-        for (int i = 0; i < njobs; ++i)
-            if (jobs[i].key.comp) {
-                variant = KS_OC_SPLIT;
-                break;
-            }
+    // The tower kernel needs a ring degree with a cluster geometry, and it and
+    // the fused row kernels read the key's a half from memory; other launch
+    // groups, and the split variant, run the whole-basis launches (same
+    // result).  The split variant's own form converted and transformed the
+    // digits for each section apart: one launch more, the source tiles built
+    // twice; slower in all 16 measured shapes (N = 2^11..2^17, 1 to 64 jobs), by
+    // 0.4% (N = 2^17, 4 jobs) to 17% (N = 2^13, 16 jobs).
+    bool full = true;
+    for (int i = 0; i < njobs; ++i) full = full && !jobs[i].key.comp;
+    if (variant == KS_OC_SPLIT || !full || (variant == KS_OC_TOWER && !oc_tower_supported(T))) variant = KS_OC_WHOLE;
     for (int i0 = 0; i0 < njobs; i0 += kMaxBatch) {
-        int rc = launch_oc_chunk(T, std::min(kMaxBatch, njobs - i0), jobs + i0, variant, share_keys, st);
+        const int n = std::min(kMaxBatch, njobs - i0);
+        const int rc = variant == KS_OC_WHOLE ? launch_oc_whole(T, n, jobs + i0, share_keys, st)
+                                              : launch_oc_sections(T, n, jobs + i0, variant, st);
         if (rc != KS_OK) return rc;
     }
     return KS_OK;
