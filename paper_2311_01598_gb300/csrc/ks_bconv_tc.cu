@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
     __shared__ u64 s_q[TBM];
     __shared__ uint32_t s_red[TBM];   // -q^-1 mod 2^32, or c (PM)
     __shared__ int s_G[2], s_off[2];  // of the item in each buffer: targets, coefficients past the stretch's first
+    pdl_start();
     const int i0 = tc_run_start(split, blockIdx.x, gridDim.x), i1 = tc_run_start(split, blockIdx.x + 1, gridDim.x);
     if (i0 >= i1) return;
     const size_t N = (size_t)1 << T.logN;
@@ -385,6 +386,7 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tbase = tbase_s;
+    pdl_wait();
 
     if (tid < TC_PROD) {
         // ------------------------------------------------------------ producers
@@ -626,7 +628,7 @@ static int launch_tc(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, int 
     const int grid = (int)std::min<u64>(items, (u64)sm_count());
     constexpr int SM = tc_pipe_smem<KB, NS>();
     KS_LAUNCH(st, name,
-              (k_bconv_tc<MODE, KB, NS, W, PM><<<grid, TC_PIPE_THREADS, SM, st>>>(T, bu, bd, slabs, XT, TBN, TB, sp)));
+              (launch_dep(st, k_bconv_tc<MODE, KB, NS, W, PM>, grid, TC_PIPE_THREADS, SM, T, bu, bd, slabs, XT, TBN, TB, sp)));
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? KS_OK : fail(KS_ECUDA, std::string(name) + " (tensor cores) launch: " + cudaGetErrorString(e));
 }

@@ -39,6 +39,15 @@
 
 namespace ks {
 
+// ------------------------------------------------------------------ dependent launches
+// Kernels launched with launch_dep: pdl_start lets the next kernel of the stream
+// begin its own prologue once every block of this one has started; pdl_wait
+// holds a block until the stream's previous kernel is complete.  Before pdl_wait
+// a kernel reads only its parameters and the parameter set's tables.  Blocks
+// with nothing to do may leave without waiting: every launch has others.
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ scalar
 __device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 wp, u64 q)
 {

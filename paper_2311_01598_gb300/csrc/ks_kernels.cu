@@ -14,6 +14,7 @@ namespace ks {
 template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, LimbMaps ms)
 {
+    pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
@@ -23,6 +24,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
     if (L.skip) return;
     const ModR<AR> md = mod_fwd<AR>(T.modc[L.tf]);
     const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
+    pdl_wait();
     for (int i = threadIdx.x; i < (1 << S::LA); i += S::THREADS_A) tws[i] = twt[i];
     const int cc = threadIdx.x % S::COLS, tau = threadIdx.x / S::COLS;
     const int c = blockIdx.x * S::COLS + cc;
@@ -55,6 +57,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
 template <class S, bool CANON, int AR>
 __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, LimbMaps ms)
 {
+    pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lz = blockIdx.y + blockIdx.z * gridDim.y;
@@ -74,6 +77,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, L
     const u64 *gin = L.src + ((size_t)h << S::LB);
     u64 *gout = L.dst + ((size_t)h << S::LB);
     u64 x[S::REGB];
+    pdl_wait();
 #pragma unroll
     for (int k = 0; k < S::REGB; ++k) x[k] = gin[k * S::TB + tau];
     stage_row_round1<S>(tsh, twt, G, tau);
@@ -227,6 +231,7 @@ int ntt_error_flag(bool clear)
 template <class S, int AR>
 __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, LimbMaps ms)
 {
+    pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
@@ -242,11 +247,12 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
     const u64 *gin = L.src + ((size_t)h << S::LB);
     u64 *gout = L.dst + ((size_t)h << S::LB);
     u64 x[S::REGB];
-#pragma unroll
-    for (int k = 0; k < S::REGB; ++k) x[k] = gin[k * S::TB + tau];
     // the last round's twiddles (common to the row) staged beside the loads,
     // as in the forward row pass; the block barriers of the first round
     // order them before their use
+    pdl_wait();
+#pragma unroll
+    for (int k = 0; k < S::REGB; ++k) x[k] = gin[k * S::TB + tau];
     stage_row_round1<S>(tsh, itwt, G, tau);
     row_inv_core<S, AR>(x, TwStaged<S>{tsh, itwt, G}, sm + rr * S::ROWPAD, tau, md);
 #pragma unroll
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
 template <class S, bool SC, int AR>
 __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, LimbMaps ms)
 {
+    pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
@@ -271,15 +278,18 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const ulonglong2 *twt = T.itw + ((size_t)L.tf << S::LOGN);
-    for (int i = threadIdx.x; i < (1 << S::LA); i += S::THREADS_A) tws[i] = twt[i];
+    ColStage<S> stage;  // in flight across pdl_wait (2^17: 92 -> 87 us; the forward pass gained nothing)
+    stage.load(twt);
     const int cc = threadIdx.x % S::COLS, tau = threadIdx.x / S::COLS;
     const int c = blockIdx.x * S::COLS + cc;
     constexpr int M = S::TA, NG = S::REGA / S::TA;
     u64 x[S::REGA];
+    pdl_wait();
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = L.src[((size_t)((tau * NG + gg) * M + k2) << S::LB) + c];
+    stage.store(tws);
     __syncthreads();
     fold_all<S::REGA, AR>(x, md);
     inv_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
@@ -348,7 +358,7 @@ static void fwd_col_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (k_fwd_col<S, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))));
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))));
 }
 
 // Persistent grid of the staged row pass: resident CTAs per SM x SMs, at
@@ -401,9 +411,9 @@ static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, cudaSt
         return;
     }
     if (canonical)
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row<S, true, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, true, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
     else
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (k_fwd_row<S, false, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, false, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
 }
 
 template <class S>
@@ -411,7 +421,7 @@ static void inv_row_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
-    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row", (k_inv_row<S, AR><<<gb, S::THREADS_B, S::SMEM_BT, st>>>(T, m))))
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row", (launch_dep(st, k_inv_row<S, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
 }
 
 // scaled: multiply by the maps' per-entry scale, or by N^-1 where a map has none.
@@ -421,9 +431,9 @@ static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStrea
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
     if (scaled)
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (k_inv_col<S, true, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
     else
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (k_inv_col<S, false, AR><<<ga, S::THREADS_A, S::SMEM_A, st>>>(T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, false, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
 }
 
 #define KS_DISPATCH_LOGN(logN, FN, ...)                                                                   \
@@ -516,6 +526,7 @@ void add_bup(BUpJobs &b, const Tables &T, const BUpJob &j)
 // ModUp P2: grid (N/256, ceil(max targets/TT), digit blocks of all jobs).
 __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_up(Tables T, BUpJobs bj)
 {
+    pdl_start();
     __shared__ u64 cs[kMaxQ][BC_TT];
     __shared__ int s_t[BC_TT];
     __shared__ int s_tf[BC_TT];
@@ -551,6 +562,7 @@ __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_up(Tables T, BUpJobs bj
     BAcc acc[BC_TT];
 #pragma unroll
     for (int g = 0; g < BC_TT; ++g) bacc_zero(acc[g]);
+    pdl_wait();
     // sources in groups of four: the loads of a group are issued together
     int i = 0;
     for (; i + 4 <= a; i += 4) {
@@ -587,7 +599,7 @@ int launch_bconv_up(const Tables &T, const BUpJobs &b, cudaStream_t st)
     if (span <= 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
     dim3 g((unsigned)(N / BC_THREADS), (unsigned)((span + BC_TT - 1) / BC_TT), (unsigned)b.zpre[b.n]);
-    KS_LAUNCH(st, "bconv_up", k_bconv_up<<<g, BC_THREADS, 0, st>>>(T, b));
+    KS_LAUNCH(st, "bconv_up", launch_dep(st, k_bconv_up, g, BC_THREADS, 0, T, b));
     return launch_status("ModUp BConv launch");
 }
 
@@ -602,6 +614,7 @@ void add_bdn(BDnJobs &b, const BDnJob &j)
 // ModDown P2: grid (N/256, ceil(max nact/TT), polynomials of all jobs).
 __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_down(Tables T, BDnJobs bj)
 {
+    pdl_start();
     __shared__ u64 cs[kMaxP][BC_TT];
     const int jb = find_slot(bj.zpre, bj.n, blockIdx.z);
     const BDnJob &J = bj.job[jb];
@@ -622,6 +635,7 @@ __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_down(Tables T, BDnJobs 
     BAcc acc[BC_TT];
 #pragma unroll
     for (int g = 0; g < BC_TT; ++g) bacc_zero(acc[g]);
+    pdl_wait();
     int k = 0;
     for (; k + 4 <= K; k += 4) {
         u64 wv[4];
@@ -661,7 +675,7 @@ int launch_bconv_down(const Tables &T, const BDnJobs &b, cudaStream_t st)
     if (span <= 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
     dim3 g((unsigned)(N / BC_THREADS), (unsigned)((span + BC_TT - 1) / BC_TT), (unsigned)b.zpre[b.n]);
-    KS_LAUNCH(st, "bconv_down", k_bconv_down<<<g, BC_THREADS, 0, st>>>(T, b));
+    KS_LAUNCH(st, "bconv_down", launch_dep(st, k_bconv_down, g, BC_THREADS, 0, T, b));
     return launch_status("ModDown BConv launch");
 }
 
@@ -684,6 +698,8 @@ __device__ __forceinline__ size_t galois_slot(size_t n, u64 g, int logN)
 __global__ void __launch_bounds__(256) k_automorph(Tables T, int t0, const u64 *in, u64 *out, u64 galois,
                                                    int accumulate)
 {
+    pdl_start();
+    pdl_wait();
     const int t = blockIdx.y;
     const size_t N = (size_t)1 << T.logN;
     const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -697,6 +713,8 @@ template <bool CK>
 __global__ void __launch_bounds__(256) k_apply_key(Tables T, int nact, int j0, int j1, const u64 *d, const u64 *D,
                                                    size_t dstride, KeyView key, u64 *cp, int accumulate, u64 galois)
 {
+    pdl_start();
+    pdl_wait();
     const int t = blockIdx.y;
     const int nt = nact + T.kp;
     const int nfull = T.nq + T.kp;
@@ -732,8 +750,7 @@ int launch_automorph(const Tables &T, int t0, int ntowers, const u64 *in, u64 *o
     if (ntowers == 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
     KS_LAUNCH(st, "automorph",
-              k_automorph<<<dim3((unsigned)(N / 256), (unsigned)ntowers), 256, 0, st>>>(T, t0, in, out, galois,
-                                                                                       accumulate ? 1 : 0));
+              launch_dep(st, k_automorph, dim3((unsigned)(N / 256), (unsigned)ntowers), 256, 0, T, t0, in, out, galois, accumulate ? 1 : 0));
     return launch_status("automorphism launch");
 }
 
@@ -745,12 +762,10 @@ int launch_apply_key(const Tables &T, int nact, int j_begin, int j_end, const u6
     dim3 g((unsigned)(N / 256), (unsigned)(nact + T.kp));
     if (key.comp)
         KS_LAUNCH(st, "apply_key",
-                  k_apply_key<true><<<g, 256, 0, st>>>(T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp,
-                                                       accumulate ? 1 : 0, galois));
+                  launch_dep(st, k_apply_key<true>, g, 256, 0, T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp, accumulate ? 1 : 0, galois));
     else
         KS_LAUNCH(st, "apply_key",
-                  k_apply_key<false><<<g, 256, 0, st>>>(T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp,
-                                                        accumulate ? 1 : 0, galois));
+                  launch_dep(st, k_apply_key<false>, g, 256, 0, T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp, accumulate ? 1 : 0, galois));
     return launch_status("apply-key launch");
 }
 
@@ -762,6 +777,8 @@ struct OutPtrs {
 __global__ void __launch_bounds__(256) k_down_final(Tables T, const u64 *cp, size_t cp_stride, const u64 *v,
                                                     size_t v_stride, OutPtrs outs)
 {
+    pdl_start();
+    pdl_wait();
     const int i = blockIdx.y, x = blockIdx.z;
     const size_t N = (size_t)1 << T.logN;
     const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -778,7 +795,7 @@ int launch_down_final(const Tables &T, int nact, int npoly, const u64 *cp, size_
     o.p[0] = outs[0];
     o.p[1] = npoly > 1 ? outs[1] : outs[0];
     dim3 g((unsigned)(N / 256), (unsigned)nact, (unsigned)npoly);
-    KS_LAUNCH(st, "down_final", k_down_final<<<g, 256, 0, st>>>(T, cp, cp_stride, v, v_stride, o));
+    KS_LAUNCH(st, "down_final", launch_dep(st, k_down_final, g, 256, 0, T, cp, cp_stride, v, v_stride, o));
     return launch_status("ModDown final launch");
 }
 
@@ -786,6 +803,8 @@ int launch_down_final(const Tables &T, int nact, int npoly, const u64 *cp, size_
 // grid (N/256, limbs)
 __global__ void k_scale(Tables T, LimbMaps ms, const ulonglong2 *fac)
 {
+    pdl_start();
+    pdl_wait();
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
     if (lg >= ms.pre[ms.n]) return;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, T.logN);
@@ -800,13 +819,15 @@ int launch_scale(const Tables &T, const LimbMaps &m, const ulonglong2 *factors_f
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
-    KS_LAUNCH(st, "scale", k_scale<<<limb_grid((unsigned)(N / 256), m.pre[m.n]), 256, 0, st>>>(T, m, factors_full));
+    KS_LAUNCH(st, "scale", launch_dep(st, k_scale, limb_grid((unsigned)(N / 256), m.pre[m.n]), 256, 0, T, m, factors_full));
     return launch_status("scale launch");
 }
 
 // grid (N/256, nact, nd): D[j][t] = d[t] for t in digit j.
 __global__ void k_bypass_copy(Tables T, int nact, const u64 *d, u64 *D)
 {
+    pdl_start();
+    pdl_wait();
     const int t = blockIdx.y, j = blockIdx.z;
     if (t / T.alpha != j) return;
     const size_t N = (size_t)1 << T.logN;
@@ -819,7 +840,7 @@ int launch_bypass_copy(const Tables &T, int nact, const u64 *d, u64 *D, cudaStre
 {
     const size_t N = (size_t)1 << T.logN;
     const int nd = (nact + T.alpha - 1) / T.alpha;
-    KS_LAUNCH(st, "bypass_copy", k_bypass_copy<<<dim3((unsigned)(N / 256), nact, nd), 256, 0, st>>>(T, nact, d, D));
+    KS_LAUNCH(st, "bypass_copy", launch_dep(st, k_bypass_copy, dim3((unsigned)(N / 256), nact, nd), 256, 0, T, nact, d, D));
     return launch_status("bypass copy launch");
 }
 

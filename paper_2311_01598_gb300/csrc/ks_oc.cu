@@ -320,6 +320,8 @@ static bool any_compressed(const OcJobs &oj)
 // sum_j NTT(z_{j,p_k}) * evk_{j,x,p_k}, canonical.  grid (N/256, jobs*K).
 __global__ void __launch_bounds__(256) k_oc_comb_p(Tables T, OcJobs oj)
 {
+    pdl_start();
+    pdl_wait();
     const int K = T.kp;
     const OcJob &J = oj.job[blockIdx.y / K];
     const int k = blockIdx.y % K;
@@ -377,6 +379,8 @@ __device__ __forceinline__ const u64 *v_limb(const OcJob &J, int x, int t, int K
 template <bool CK, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_pg(Tables T, OcJobs oj, KeyGroups kg)
 {
+    pdl_start();
+    pdl_wait();
     const int K = T.kp;
     const int g = blockIdx.y / K, k = blockIdx.y % K;
     const int m0 = kg.first[g], cnt = kg.first[g + 1] - m0;
@@ -431,6 +435,8 @@ __global__ void __launch_bounds__(256) k_oc_comb_pg(Tables T, OcJobs oj, KeyGrou
 template <bool CK, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGroups kg)
 {
+    pdl_start();
+    pdl_wait();
     const int K = T.kp;
     const int g = find_slot(kg.pre, kg.n, blockIdx.y);
     const int t = blockIdx.y - kg.pre[g];
@@ -539,15 +545,15 @@ static void comb_grouped(const Tables &T, const OcJobs &oj, const KeyGroups &kg,
     if (p_section) {
         const dim3 g((unsigned)(N / (256 * V)), kg.n * T.kp);
         if (ck)
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<true, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pg<true, V>, g, 256, 0, T, oj, kg)));
         else
-            KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pg<false, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pg<false, V>, g, 256, 0, T, oj, kg)));
     } else {
         const dim3 g((unsigned)(N / (256 * V)), kg.pre[kg.n]);
         if (ck)
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<true, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qg<true, V>, g, 256, 0, T, oj, kg)));
         else
-            KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qg<false, V><<<g, 256, 0, st>>>(T, oj, kg)));
+            KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qg<false, V>, g, 256, 0, T, oj, kg)));
     }
 }
 
@@ -565,6 +571,8 @@ size_t oc_scratch_words(const Tables &T, int nact)
 template <bool CK, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
 {
+    pdl_start();
+    pdl_wait();
     const int K = T.kp;
     const OcJob &J = oj.job[blockIdx.y / K];
     const int k = blockIdx.y % K;
@@ -600,6 +608,8 @@ __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
 template <bool CK, int V>
 __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
 {
+    pdl_start();
+    pdl_wait();
     const int jb = find_slot(oj.pre, oj.n, blockIdx.y);
     const OcJob &J = oj.job[jb];
     const int t = blockIdx.y - oj.pre[jb];
@@ -673,18 +683,18 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     if (grouped)  // P4+P5, P towers
         comb_grouped(T, oj, kg, true, st);
     else if (ck)
-        KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pw<true, 1><<<gp, 256, 0, st>>>(T, oj)));
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, 1>, gp, 256, 0, T, oj)));
     else
-        KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_pw<false, 1><<<gp, 256, 0, st>>>(T, oj)));
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, 1>, gp, 256, 0, T, oj)));
     if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;    // ModDown P1
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;        // ModDown P2
     if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;    // ModDown P3
     if (grouped)  // P4+P5 Q, ModDown P4
         comb_grouped(T, oj, kg, false, st);
     else if (ck)
-        KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qw<true, 4><<<gq, 256, 0, st>>>(T, oj)));
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, 4>, gq, 256, 0, T, oj)));
     else
-        KS_LAUNCH(st, "oc_comb_q", (k_oc_comb_qw<false, 4><<<gq, 256, 0, st>>>(T, oj)));
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, 4>, gq, 256, 0, T, oj)));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC whole-basis launch: ") + cudaGetErrorString(e));
     return KS_OK;
@@ -725,7 +735,7 @@ static int launch_oc_sections(const Tables &T, int n, const OcJob *jobs, int var
     if ((rc = launch_bconv_up(T, bp, st)) != KS_OK) return rc;
     if (variant == KS_OC_TOWER) {
         if ((rc = launch_ntt_fwd(T, mp, false, st)) != KS_OK) return rc;
-        KS_LAUNCH(st, "oc_comb_p", (k_oc_comb_p<<<dim3((unsigned)(N / 256), n * K), 256, 0, st>>>(T, oj)));
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_p, dim3((unsigned)(N / 256), n * K), 256, 0, T, oj)));
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC combine launch: ") + cudaGetErrorString(e));
         if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;
