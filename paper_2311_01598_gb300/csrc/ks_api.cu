@@ -235,8 +235,8 @@ static int run_mp(const ks_params *P, const Tables &T, const ks_key *K, int nact
 
 // ------------------------------------------------------------------ hoisted rotations
 // One ModUp of d (as MP) shared by R rotations: rotation r's key product reads
-// the raised digits through X -> X^g_r, then the ModDowns of all rotations
-// run as batched launches (groups of kMaxBatch rotations).
+// the raised digits through X -> X^g_r; the key products and ModDowns of all
+// rotations run as batched launches (groups of kMaxBatch rotations).
 static int run_hoisted(ks_params *P, uint32_t R, const ks_key *const *keys, const uint64_t *gal, int nact,
                        const u64 *d, u64 *const *out0, u64 *const *out1, cudaStream_t st)
 {
@@ -244,7 +244,6 @@ static int run_hoisted(ks_params *P, uint32_t R, const ks_key *const *keys, cons
     const size_t N = P->N;
     const int nt = nact + P->kp;
     const int nd = active_digits(P, nact);
-    const int K = P->kp;
     Workspace *w = nullptr;
     int rc = get_ws(P, st, true, &w);
     if (rc) return rc;
@@ -276,36 +275,29 @@ static int run_hoisted(ks_params *P, uint32_t R, const ks_key *const *keys, cons
     for (uint32_t r0 = 0; r0 < R; r0 += G) {
         const uint32_t g = std::min(G, R - r0);
         u64 *cpr = w->rot, *vr = w->rot + (size_t)G * cp_words;
-        for (uint32_t i = 0; i < g; ++i)
-            if ((rc = launch_apply_key(T, nact, 0, nd, d, w->D, (size_t)nt * N, key_view(keys[r0 + i]),
-                                       cpr + i * cp_words, false, st, gal[r0 + i])) != KS_OK)
-                return rc;
-        // ModDown of the g rotations: P1 iNTT, P2 BConv, P3 NTT, P4.
-        LimbMaps mP, mV;
-        mP.n = mV.n = 0;
-        BDnJobs bd;
-        bd.n = 0;
+        OcJob jobs[kMaxBatch];
         for (uint32_t i = 0; i < g; ++i) {
-            u64 *c = cpr + i * cp_words, *v = vr + i * v_words;
-            add_map(mP, LimbMap{c, c, nullptr, K, nt, nact, nact, nact, -1}, 2 * K);
-            add_bdn(bd, BDnJob{c, (size_t)nt * N, v, (size_t)nact * N, nact, 2});
-            add_map(mV, LimbMap{v, v, nullptr, nact, nact, 0, 0, nact, -1}, 2 * nact);
+            OcJob &J = jobs[i];
+            J.d = d;
+            J.out0 = out0[r0 + i];
+            J.out1 = out1[r0 + i];
+            J.key = key_view(keys[r0 + i]);
+            J.y = nullptr;
+            J.tmp = w->D;
+            J.v = vr + i * v_words;
+            J.cp = cpr + i * cp_words;
+            J.gal = gal[r0 + i];
+            J.pre = nullptr;
+            J.nact = nact;
+            J.nd = nd;
         }
-        if ((rc = launch_ntt_inv(T, mP, false, st)) != KS_OK) return rc;
-        if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;
-        if ((rc = launch_ntt_fwd(T, mV, false, st)) != KS_OK) return rc;
-        for (uint32_t i = 0; i < g; ++i) {
-            u64 *outs[2] = {out0[r0 + i], out1[r0 + i]};
-            if ((rc = launch_down_final(T, nact, 2, cpr + i * cp_words, (size_t)nt * N, vr + i * v_words,
-                                        (size_t)nact * N, outs, st)) != KS_OK)
-                return rc;
-        }
+        if ((rc = launch_oc_hoisted(T, (int)g, jobs, st)) != KS_OK) return rc;
     }
     return KS_OK;
 }
 
 // ------------------------------------------------------------------ DC
-// Digit-Centric: ModUp P1..P5 for one digit at a time, partial sums of c'
+// Digit-Centric: ModUp P2..P5 for one digit at a time, partial sums of c'
 // accumulated in device memory, then ModDown.
 static int run_dc(const ks_params *P, const Tables &T, const ks_key *K, int nact, const u64 *d, u64 *out0, u64 *out1,
                   Workspace *w, cudaStream_t st)
@@ -313,11 +305,11 @@ static int run_dc(const ks_params *P, const Tables &T, const ks_key *K, int nact
     const int nt = nact + P->kp;
     const int nd = active_digits(P, nact);
     int rc;
+    // P1 of every digit's towers in one launch (a digit's few limbs alone leave
+    // most of the chip idle: 17 us of 75 a digit at N = 2^16, 6 towers a digit)
+    LimbMap m1{d, w->y, pre_level(P, nact), nact, 0, 0, 0, nact, -1};
+    if ((rc = launch_ntt_inv(T, one_map(m1, nact), false, st)) != KS_OK) return rc;
     for (int j = 0; j < nd; ++j) {
-        const int lo = j * P->alpha;
-        const int a = std::min(P->alpha, nact - lo);
-        LimbMap m1{d, w->y, pre_level(P, nact) + lo, a, 0, lo, lo, nact, -1};
-        if ((rc = launch_ntt_inv(T, one_map(m1, a), false, st)) != KS_OK) return rc;
         BUpJobs bu;
         bu.n = 0;
         add_bup(bu, T, BUpJob{w->y, w->D, 0, nact, 0, nt, 0, j});
@@ -341,7 +333,9 @@ OcJob oc_job(const ks_params *P, const ks_key *K, int nact, const u64 *d, u64 *o
     J.key = key_view(K);
     J.y = scratch;
     J.tmp = J.y + (size_t)nact * N;
-    J.cp = J.tmp + ((size_t)nd * (nact + P->kp) + 2 * (size_t)nact) * N;
+    J.v = J.tmp + (size_t)nd * (nact + P->kp) * N;
+    J.gal = 1;
+    J.cp = J.v + 2 * (size_t)nact * N;
     J.pre = pre_level(P, nact);
     J.nact = nact;
     J.nd = nd;

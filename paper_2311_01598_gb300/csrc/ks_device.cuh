@@ -367,6 +367,107 @@ __device__ __forceinline__ u64 key_a(const KeyView &K, int j, int t, size_t n, i
     return K.evk[(((size_t)(2 * j + 1) * nfull + t) << logN) + n];
 }
 
+// V consecutive words a thread (V = 2: 16-byte loads and stores; limb bases and
+// even indices keep them aligned).
+template <int V>
+__device__ __forceinline__ void ldv(const u64 *p, u64 (&o)[V])
+{
+    static_assert(V == 1 || V % 2 == 0, "one word or pairs");
+    if constexpr (V == 1) {
+        o[0] = *p;
+    } else {
+#pragma unroll
+        for (int c = 0; c < V; c += 2) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p + c);
+            o[c] = t.x;
+            o[c + 1] = t.y;
+        }
+    }
+}
+template <int V>
+__device__ __forceinline__ void stv(u64 *p, const u64 (&v)[V])
+{
+    static_assert(V == 1 || V % 2 == 0, "one word or pairs");
+    if constexpr (V == 1) {
+        *p = v[0];
+    } else {
+#pragma unroll
+        for (int c = 0; c < V; c += 2) *reinterpret_cast<ulonglong2 *>(p + c) = make_ulonglong2(v[c], v[c + 1]);
+    }
+}
+
+// key product of V coefficients: x * b_j and x * a_j added into sb, sa
+template <bool CK, int V>
+__device__ __forceinline__ void key_macv(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 q,
+                                         const u64 (&x)[V], U128 (&sb)[V], U128 (&sa)[V])
+{
+    const size_t N = (size_t)1 << logN;
+    u64 kb[V], ka[V];
+    if (CK && K.comp) {
+        ldv<V>(K.evk + ((size_t)j * nfull + t) * N + n, kb);
+        key_a_words<V>(K.a_seed, j, t, n, logN, nfull, q, ka);
+    } else {
+        ldv<V>(K.evk + ((size_t)(2 * j) * nfull + t) * N + n, kb);
+        ldv<V>(K.evk + ((size_t)(2 * j + 1) * nfull + t) * N + n, ka);
+    }
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+        mac128(sb[c], x[c], kb[c]);
+        mac128(sa[c], x[c], ka[c]);
+    }
+}
+
+// the key words of V coefficients (regenerated a half for a compressed key)
+template <bool CK, int V>
+__device__ __forceinline__ void key_words(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 q,
+                                          u64 (&kb)[V], u64 (&ka)[V])
+{
+    const size_t N = (size_t)1 << logN;
+    if (CK && K.comp) {
+        ldv<V>(K.evk + ((size_t)j * nfull + t) * N + n, kb);
+        key_a_words<V>(K.a_seed, j, t, n, logN, nfull, q, ka);
+    } else {
+        ldv<V>(K.evk + ((size_t)(2 * j) * nfull + t) * N + n, kb);
+        ldv<V>(K.evk + ((size_t)(2 * j + 1) * nfull + t) * N + n, ka);
+    }
+}
+
+// The automorphism X -> X^g of the evaluation domain: slot n takes slot n' with
+// 2brv(n')+1 = (2brv(n)+1)g mod 2N.
+__device__ __forceinline__ size_t galois_slot(size_t n, u64 g, int logN)
+{
+    const u64 two_n = 2ull << logN;
+    const u64 e = ((2ull * (__brev((unsigned)n) >> (32 - logN)) + 1) * g) & (two_n - 1);
+    return (size_t)(__brev((unsigned)((e - 1) >> 1)) >> (32 - logN));
+}
+// V words of a limb through the automorphism, slots n..n+V-1 (n even for V > 1).
+// The low bit of a slot is the top bit of brv, 2^logN in the exponent, and g is
+// odd: slots n and n+1 come from one aligned pair, in order or swapped, so a
+// pair is one 16-byte load.
+template <int V>
+struct GaloisSlots {
+    u32 s[(V + 1) / 2];
+    __device__ __forceinline__ GaloisSlots(size_t n, u64 g, int logN)
+    {
+#pragma unroll
+        for (int c = 0; c < (V + 1) / 2; ++c) s[c] = (u32)galois_slot(n + 2 * c, g, logN);
+    }
+    __device__ __forceinline__ void load(const u64 *limb, u64 (&o)[V]) const
+    {
+        if constexpr (V == 1) {
+            o[0] = limb[s[0]];
+        } else {
+#pragma unroll
+            for (int c = 0; c < V / 2; ++c) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(limb + (s[c] & ~1u));
+                const bool swap = s[c] & 1;
+                o[2 * c] = swap ? t.y : t.x;
+                o[2 * c + 1] = swap ? t.x : t.y;
+            }
+        }
+    }
+};
+
 // Base-conversion accumulator: sum of y*c with y, c < 2^56 split at 28 bits.
 struct BAcc {
     u64 a0, a1, a2;

@@ -680,39 +680,41 @@ int launch_bconv_down(const Tables &T, const BDnJobs &b, cudaStream_t st)
 }
 
 // ------------------------------------------------------------------ apply key
-// ModUp P4+P5 (single job): grid (N/256, nact+K).  The stored key carries the
-// folded factors and 2^64, so REDC of the 128-bit sum gives the folded c'.
-// With galois = g != 1 the raised digits are read through the automorphism
-// X -> X^g of the evaluation domain (slot n takes slot n' with
-// 2brv(n')+1 = (2brv(n)+1)g mod 2N): the key product of a hoisted rotation.
-__device__ __forceinline__ size_t galois_slot(size_t n, u64 g, int logN)
-{
-    const u64 two_n = 2ull << logN;
-    const u64 e = ((2ull * (__brev((unsigned)n) >> (32 - logN)) + 1) * g) & (two_n - 1);
-    return (size_t)(__brev((unsigned)((e - 1) >> 1)) >> (32 - logN));
-}
-
 // Evaluation-domain automorphism X -> X^g of n towers starting at full
 // tower t0: out[t][n] = in[t][galois_slot(n)] (+ out[t][n] mod q_t with
-// accumulate).  Inputs canonical; grid (N/256, towers).
+// accumulate).  Inputs canonical; grid (N/1024, towers), four slots a thread.
+// Buffers that are only 8-byte aligned take V = 1, grid (N/256, towers).
+template <int V>
 __global__ void __launch_bounds__(256) k_automorph(Tables T, int t0, const u64 *in, u64 *out, u64 galois,
                                                    int accumulate)
 {
     pdl_start();
-    pdl_wait();
     const int t = blockIdx.y;
     const size_t N = (size_t)1 << T.logN;
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const u64 q = T.modc[t0 + t].q;
-    const u64 v = in[(size_t)t * N + galois_slot(n, galois, T.logN)];
+    const GaloisSlots<V> gs(n, galois, T.logN);
+    pdl_wait();
+    u64 v[V];
+    gs.load(in + (size_t)t * N, v);
     u64 *o = out + (size_t)t * N + n;
-    *o = accumulate ? reduce2(*o + v, q) : v;
+    if (accumulate) {
+        u64 a[V];
+        ldv<V>(o, a);
+#pragma unroll
+        for (int c = 0; c < V; ++c) v[c] = reduce2(a[c] + v[c], q);
+    }
+    stv<V>(o, v);
 }
 
+// ModUp P4+P5 (single job): grid (N/512, nact+K), two coefficients a thread.
+// The stored key carries the folded factors and 2^64, so REDC of the 128-bit sum
+// gives the folded c'.
 template <bool CK>
 __global__ void __launch_bounds__(256) k_apply_key(Tables T, int nact, int j0, int j1, const u64 *d, const u64 *D,
-                                                   size_t dstride, KeyView key, u64 *cp, int accumulate, u64 galois)
+                                                   size_t dstride, KeyView key, u64 *cp, int accumulate)
 {
+    constexpr int V = 2;
     pdl_start();
     pdl_wait();
     const int t = blockIdx.y;
@@ -720,28 +722,35 @@ __global__ void __launch_bounds__(256) k_apply_key(Tables T, int nact, int j0, i
     const int nfull = T.nq + T.kp;
     const int tf = full_tower(t, nact, T.nq);
     const size_t N = (size_t)1 << T.logN;
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t ns = galois == 1 ? n : galois_slot(n, galois, T.logN);
+    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[tf];
-    U128 sb = {0, 0}, sa = {0, 0};
+    u64 *cb = cp + (size_t)t * N + n;
+    u64 *ca = cp + ((size_t)nt + t) * N + n;
+    u64 pb[V] = {0, 0}, pa[V] = {0, 0};
+    if (accumulate) {  // issued with the first digit's loads
+        ldv<V>(cb, pb);
+        ldv<V>(ca, pa);
+    }
+    U128 sb[V], sa[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
     for (int j = j0; j < j1; ++j) {
         const bool own = t < nact && t / T.alpha == j;
-        const u64 dv = own ? d[(size_t)t * N + ns] : D[(size_t)(j - j0) * dstride + (size_t)t * N + ns];
-        mac128(sb, dv, key_b<CK>(key, j, tf, n, nfull, T.logN));
-        mac128(sa, dv, key_a<CK>(key, j, tf, n, nfull, T.logN, mc.q));
+        u64 x[V];
+        ldv<V>(own ? d + (size_t)t * N + n : D + (size_t)(j - j0) * dstride + (size_t)t * N + n, x);
+        key_macv<CK, V>(key, j, tf, n, nfull, T.logN, mc.q, x, sb, sa);
     }
     // D any 64-bit words: each product is below 2^64 q, the sum of at most 64
     // below 2^126 and its REDC below 65 q, reduced fully.
-    u64 rb = reduce_any(redc(sb, mc.q, mc.mont), mc.q, mc.one_sh);
-    u64 ra = key_a_finish<CK>(key, sa, mc, T.key_sc, tf);
-    u64 *cb = cp + (size_t)t * N + n;
-    u64 *ca = cp + ((size_t)nt + t) * N + n;
-    if (accumulate) {
-        rb = reduce2(rb + *cb, mc.q);
-        ra = reduce2(ra + *ca, mc.q);
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+        const u64 rb = reduce_any(redc(sb[c], mc.q, mc.mont), mc.q, mc.one_sh);
+        const u64 ra = key_a_finish<CK>(key, sa[c], mc, T.key_sc, tf);
+        pb[c] = accumulate ? reduce2(rb + pb[c], mc.q) : rb;
+        pa[c] = accumulate ? reduce2(ra + pa[c], mc.q) : ra;
     }
-    *cb = rb;
-    *ca = ra;
+    stv<V>(cb, pb);
+    stv<V>(ca, pa);
 }
 
 int launch_automorph(const Tables &T, int t0, int ntowers, const u64 *in, u64 *out, uint64_t galois, bool accumulate,
@@ -749,23 +758,27 @@ int launch_automorph(const Tables &T, int t0, int ntowers, const u64 *in, u64 *o
 {
     if (ntowers == 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
-    KS_LAUNCH(st, "automorph",
-              launch_dep(st, k_automorph, dim3((unsigned)(N / 256), (unsigned)ntowers), 256, 0, T, t0, in, out, galois, accumulate ? 1 : 0));
+    const unsigned gy = (unsigned)ntowers;
+    if ((((uintptr_t)in | (uintptr_t)out) & 15) == 0)
+        KS_LAUNCH(st, "automorph", launch_dep(st, k_automorph<4>, dim3((unsigned)(N / 1024), gy), 256, 0, T, t0, in, out,
+                                              galois, accumulate ? 1 : 0));
+    else
+        KS_LAUNCH(st, "automorph", launch_dep(st, k_automorph<1>, dim3((unsigned)(N / 256), gy), 256, 0, T, t0, in, out,
+                                              galois, accumulate ? 1 : 0));
     return launch_status("automorphism launch");
 }
 
 int launch_apply_key(const Tables &T, int nact, int j_begin, int j_end, const u64 *d, const u64 *D,
-                     size_t D_digit_stride, const KeyView &key, u64 *cp, bool accumulate, cudaStream_t st,
-                     uint64_t galois)
+                     size_t D_digit_stride, const KeyView &key, u64 *cp, bool accumulate, cudaStream_t st)
 {
     const size_t N = (size_t)1 << T.logN;
-    dim3 g((unsigned)(N / 256), (unsigned)(nact + T.kp));
+    dim3 g((unsigned)(N / 512), (unsigned)(nact + T.kp));
     if (key.comp)
-        KS_LAUNCH(st, "apply_key",
-                  launch_dep(st, k_apply_key<true>, g, 256, 0, T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp, accumulate ? 1 : 0, galois));
+        KS_LAUNCH(st, "apply_key", launch_dep(st, k_apply_key<true>, g, 256, 0, T, nact, j_begin, j_end, d, D,
+                                              D_digit_stride, key, cp, accumulate ? 1 : 0));
     else
-        KS_LAUNCH(st, "apply_key",
-                  launch_dep(st, k_apply_key<false>, g, 256, 0, T, nact, j_begin, j_end, d, D, D_digit_stride, key, cp, accumulate ? 1 : 0, galois));
+        KS_LAUNCH(st, "apply_key", launch_dep(st, k_apply_key<false>, g, 256, 0, T, nact, j_begin, j_end, d, D,
+                                              D_digit_stride, key, cp, accumulate ? 1 : 0));
     return launch_status("apply-key launch");
 }
 
@@ -773,7 +786,9 @@ struct OutPtrs {
     u64 *p[2];
 };
 
-// ModDown P4: out = cp - v mod q (cp canonical, v lazy, at most flz).
+// ModDown P4: out = cp - v mod q (cp canonical, v lazy, at most flz).  V slots a
+// thread; the stage entry's output may be only 8-byte aligned (V = 1).
+template <int V>
 __global__ void __launch_bounds__(256) k_down_final(Tables T, const u64 *cp, size_t cp_stride, const u64 *v,
                                                     size_t v_stride, OutPtrs outs)
 {
@@ -781,10 +796,14 @@ __global__ void __launch_bounds__(256) k_down_final(Tables T, const u64 *cp, siz
     pdl_wait();
     const int i = blockIdx.y, x = blockIdx.z;
     const size_t N = (size_t)1 << T.logN;
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[i];
-    const u64 r = cp[x * cp_stride + (size_t)i * N + n] + mc.flz - v[x * v_stride + (size_t)i * N + n];
-    outs.p[x][(size_t)i * N + n] = reduce_any(r, mc.q, mc.one_sh);
+    u64 a[V], b[V];
+    ldv<V>(cp + x * cp_stride + (size_t)i * N + n, a);
+    ldv<V>(v + x * v_stride + (size_t)i * N + n, b);
+#pragma unroll
+    for (int c = 0; c < V; ++c) a[c] = reduce_any(a[c] + mc.flz - b[c], mc.q, mc.one_sh);
+    stv<V>(outs.p[x] + (size_t)i * N + n, a);
 }
 
 int launch_down_final(const Tables &T, int nact, int npoly, const u64 *cp, size_t cp_stride, const u64 *v,
@@ -794,8 +813,12 @@ int launch_down_final(const Tables &T, int nact, int npoly, const u64 *cp, size_
     OutPtrs o;
     o.p[0] = outs[0];
     o.p[1] = npoly > 1 ? outs[1] : outs[0];
-    dim3 g((unsigned)(N / 256), (unsigned)nact, (unsigned)npoly);
-    KS_LAUNCH(st, "down_final", launch_dep(st, k_down_final, g, 256, 0, T, cp, cp_stride, v, v_stride, o));
+    if ((((uintptr_t)o.p[0] | (uintptr_t)o.p[1]) & 15) == 0)
+        KS_LAUNCH(st, "down_final", launch_dep(st, k_down_final<4>, dim3((unsigned)(N / 1024), nact, npoly), 256, 0, T, cp,
+                                               cp_stride, v, v_stride, o));
+    else
+        KS_LAUNCH(st, "down_final", launch_dep(st, k_down_final<1>, dim3((unsigned)(N / 256), nact, npoly), 256, 0, T, cp,
+                                               cp_stride, v, v_stride, o));
     return launch_status("ModDown final launch");
 }
 

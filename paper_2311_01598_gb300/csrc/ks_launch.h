@@ -148,11 +148,9 @@ int tc_error_flag(bool clear);
 int ntt_error_flag(bool clear);
 
 // ModUp P4+P5 (single job): cp[x][t] = sum_j D_{j,t} * evk_{j,x,t}, D_{j,t} = d_t
-// inside digit j; D holds lazy NTT output.  accumulate: add to cp.  galois
-// g != 1: every D_{j,t} (and d_t) is read through X -> X^g (hoisted rotation).
+// inside digit j; D holds lazy NTT output.  accumulate: add to cp.
 int launch_apply_key(const Tables &T, int nact, int j_begin, int j_end, const u64 *d, const u64 *D,
-                     size_t D_digit_stride, const KeyView &key, u64 *cp, bool accumulate, cudaStream_t st,
-                     uint64_t galois = 1);
+                     size_t D_digit_stride, const KeyView &key, u64 *cp, bool accumulate, cudaStream_t st);
 // Automorphism X -> X^g of the evaluation slots of ntowers limbs (full
 // towers t0..t0+ntowers-1): out = phi_g(in), or out + phi_g(in) mod q with
 // accumulate.  in and out must not overlap.
@@ -182,7 +180,9 @@ struct OcJob {
     u64 *out0, *out1;
     KeyView key;  // the fused variant reads full keys only (launch_oc)
     u64 *y;    // [nact][N]
-    u64 *tmp;  // [nd*(nact+K) + 2*nact][N]
+    u64 *tmp;  // [nd*(nact+K) + 2*nact][N]; whole basis: D, then v
+    u64 *v;    // whole basis: ModDown limbs [2][nact][N]
+    u64 gal;   // hoisted rotation: Galois element the job reads D and d through
     u64 *cp;   // [2][nact+K][N]
     const ulonglong2 *pre;  // ModUp P1 factors of the level
     int nact, nd;
@@ -225,5 +225,7 @@ int launch_oc_tower(const Tables &T, const OcJobs &oj, cudaStream_t st);
 // combine kernels (each key word read once per group of jobs); otherwise
 // every job streams its own key limbs.
 int launch_oc(const Tables &T, int njobs, const OcJob *jobs, int variant, cudaStream_t st, bool share_keys = false);
+// Rotations (at most kMaxBatch, one level) sharing the raised digits.
+int launch_oc_hoisted(const Tables &T, int n, const OcJob *jobs, cudaStream_t st);
 
 }  // namespace ks

@@ -27,6 +27,7 @@ namespace {
 template <class S, int MUL, bool CANON, int AR>
 __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_cl(Tables T, LimbMaps ms)
 {
+    pdl_start();
     typedef Cl<S, MUL> G_;
     constexpr int COLS = G_::COLS, ROWS = G_::ROWS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
         const int cc = threadIdx.x % COLS, tau = threadIdx.x / COLS;
         const int c = r * COLS + cc;
         u64 x[S::REGA];
+        pdl_wait();
 #pragma unroll
         for (int k = 0; k < S::REGA; ++k) x[k] = L.src[((size_t)(k * S::TA + tau) << S::LB) + c];
         __syncthreads();
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
 template <class S, int MUL, bool SC, int AR>
 __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_cl(Tables T, LimbMaps ms)
 {
+    pdl_start();
     typedef Cl<S, MUL> G_;
     constexpr int COLS = G_::COLS, ROWS = G_::ROWS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -116,6 +119,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
         const TwRow<S> tw{itw, (1 << S::LA) + h};
         const u64 *gin = L.src + ((size_t)h << S::LB);
         u64 x[S::REGB];
+        pdl_wait();
 #pragma unroll
         for (int k = 0; k < S::REGB; ++k) x[k] = gin[k * S::TB + tau];
         row_inv_core<S, AR>(x, tw, buf + rr * S::ROWPAD, tau, md);  // ends with buf free
@@ -190,13 +194,15 @@ static cudaError_t launch_cluster(KERN kern, int C, int threads, int smem, int l
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, T, m);
 }
 

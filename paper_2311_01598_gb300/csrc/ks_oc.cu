@@ -245,70 +245,6 @@ static int oc_rows(const Tables &T, const OcJobs &oj, bool p_section, cudaStream
 // plain row passes: more resident warps per SM than the fused row kernels, at
 // the price of one more round trip of the limbs through L2/HBM.
 
-// V consecutive coefficients per thread (V = 2: 16-byte loads and stores;
-// limb bases and even coefficient indices keep them aligned).
-template <int V>
-__device__ __forceinline__ void ldv(const u64 *p, u64 (&o)[V])
-{
-    static_assert(V == 1 || V % 2 == 0, "one word or pairs");
-    if constexpr (V == 1) {
-        o[0] = *p;
-    } else {
-#pragma unroll
-        for (int c = 0; c < V; c += 2) {
-            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p + c);
-            o[c] = t.x;
-            o[c + 1] = t.y;
-        }
-    }
-}
-template <int V>
-__device__ __forceinline__ void stv(u64 *p, const u64 (&v)[V])
-{
-    static_assert(V == 1 || V % 2 == 0, "one word or pairs");
-    if constexpr (V == 1) {
-        *p = v[0];
-    } else {
-#pragma unroll
-        for (int c = 0; c < V; c += 2) *reinterpret_cast<ulonglong2 *>(p + c) = make_ulonglong2(v[c], v[c + 1]);
-    }
-}
-// key product of V coefficients: x * b_j and x * a_j added into sb, sa
-template <bool CK, int V>
-__device__ __forceinline__ void key_macv(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 q,
-                                         const u64 (&x)[V], U128 (&sb)[V], U128 (&sa)[V])
-{
-    const size_t N = (size_t)1 << logN;
-    u64 kb[V], ka[V];
-    if (CK && K.comp) {
-        ldv<V>(K.evk + ((size_t)j * nfull + t) * N + n, kb);
-        key_a_words<V>(K.a_seed, j, t, n, logN, nfull, q, ka);
-    } else {
-        ldv<V>(K.evk + ((size_t)(2 * j) * nfull + t) * N + n, kb);
-        ldv<V>(K.evk + ((size_t)(2 * j + 1) * nfull + t) * N + n, ka);
-    }
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        mac128(sb[c], x[c], kb[c]);
-        mac128(sa[c], x[c], ka[c]);
-    }
-}
-
-// the key words of V coefficients (regenerated a half for a compressed key)
-template <bool CK, int V>
-__device__ __forceinline__ void key_words(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 q,
-                                          u64 (&kb)[V], u64 (&ka)[V])
-{
-    const size_t N = (size_t)1 << logN;
-    if (CK && K.comp) {
-        ldv<V>(K.evk + ((size_t)j * nfull + t) * N + n, kb);
-        key_a_words<V>(K.a_seed, j, t, n, logN, nfull, q, ka);
-    } else {
-        ldv<V>(K.evk + ((size_t)(2 * j) * nfull + t) * N + n, kb);
-        ldv<V>(K.evk + ((size_t)(2 * j + 1) * nfull + t) * N + n, ka);
-    }
-}
-
 static bool any_compressed(const OcJobs &oj)
 {
     for (int i = 0; i < oj.n; ++i)
@@ -370,9 +306,9 @@ __device__ __forceinline__ const u64 *q_limb(const OcJob &J, int j, int t, int j
     if (j == j0) return J.d + (size_t)t * N;
     return J.tmp + ((size_t)j * (J.nact + K) + t) * N;
 }
-__device__ __forceinline__ const u64 *v_limb(const OcJob &J, int x, int t, int K, size_t N)
+__device__ __forceinline__ const u64 *v_limb(const OcJob &J, int x, int t, size_t N)
 {
-    return J.tmp + ((size_t)J.nd * (J.nact + K) + (size_t)x * J.nact + t) * N;
+    return J.v + ((size_t)x * J.nact + t) * N;
 }
 
 // P towers.  grid (N/(256V), groups*K).
@@ -482,8 +418,8 @@ __global__ void __launch_bounds__(256) k_oc_comb_qg(Tables T, OcJobs oj, KeyGrou
             const OcJob &J = oj.job[kg.mem[m0 + i]];
             if (J.nact > t) {
                 u64 vb[V], va[V], o0[V], o1[V];
-                ldv<V>(v_limb(J, 0, t, K, N) + n, vb);
-                ldv<V>(v_limb(J, 1, t, K, N) + n, va);
+                ldv<V>(v_limb(J, 0, t, N) + n, vb);
+                ldv<V>(v_limb(J, 1, t, N) + n, va);
 #pragma unroll
                 for (int c = 0; c < V; ++c) {
                     const u64 cb = reduce_any(redc(sb[i][c], mc.q, mc.mont), mc.q, mc.one_sh);
@@ -567,15 +503,18 @@ size_t oc_scratch_words(const Tables &T, int nact)
 
 // Whole-basis variant: tmp holds D [nd][nact+K] then v [2][nact].
 // P-tower combine of this layout: c'_{x,p_k} from D rows at tower nact+k.
-// grid (N/(256V), jobs*K).
-template <bool CK, int V>
+// grid (N/(256V), jobs*K).  GAL: hoisted rotations, jobs of one level that share
+// D and d and read them through their own automorphism; the jobs of a tower lie
+// next to each other in the grid, so that its rows of D come from L2 for all but
+// the first.
+template <bool CK, bool GAL, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
 {
     pdl_start();
     pdl_wait();
     const int K = T.kp;
-    const OcJob &J = oj.job[blockIdx.y / K];
-    const int k = blockIdx.y % K;
+    const OcJob &J = oj.job[GAL ? blockIdx.y % oj.n : blockIdx.y / K];
+    const int k = GAL ? blockIdx.y / oj.n : blockIdx.y % K;
     const int tf = T.nq + k;
     const int t = J.nact + k;
     const int nt = J.nact + K;
@@ -583,12 +522,17 @@ __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
     const size_t N = (size_t)1 << T.logN;
     const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[tf];
+    const GaloisSlots<V> gs(n, GAL ? J.gal : 1, T.logN);
     U128 sb[V], sa[V];
 #pragma unroll
     for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
     for (int j = 0; j < J.nd; ++j) {
         u64 x[V];
-        ldv<V>(J.tmp + ((size_t)j * nt + t) * N + n, x);
+        const u64 *D = J.tmp + ((size_t)j * nt + t) * N;
+        if constexpr (GAL)
+            gs.load(D, x);
+        else
+            ldv<V>(D + n, x);
         key_macv<CK, V>(J.key, j, tf, n, nfull, T.logN, mc.q, x, sb, sa);
     }
     u64 ob[V], oa[V];
@@ -605,14 +549,14 @@ __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
 // Four CTAs per SM (64 registers, a few spilled words): more loads in flight
 // than three CTAs at the compiler's 74 registers (0.92 -> 0.95 of the copy
 // bandwidth on the benchmark step).
-template <bool CK, int V>
+template <bool CK, bool GAL, int V>
 __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
 {
     pdl_start();
     pdl_wait();
-    const int jb = find_slot(oj.pre, oj.n, blockIdx.y);
+    const int jb = GAL ? blockIdx.y % oj.n : find_slot(oj.pre, oj.n, blockIdx.y);
     const OcJob &J = oj.job[jb];
-    const int t = blockIdx.y - oj.pre[jb];
+    const int t = GAL ? blockIdx.y / oj.n : blockIdx.y - oj.pre[jb];
     const int nact = J.nact;
     const int nt = nact + T.kp;
     const int j0 = t / T.alpha;
@@ -620,18 +564,22 @@ __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
     const size_t N = (size_t)1 << T.logN;
     const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[t];
+    const GaloisSlots<V> gs(n, GAL ? J.gal : 1, T.logN);
     U128 sb[V], sa[V];
 #pragma unroll
     for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
     for (int j = 0; j < J.nd; ++j) {
         u64 x[V];
-        ldv<V>(j == j0 ? J.d + (size_t)t * N + n : J.tmp + ((size_t)j * nt + t) * N + n, x);
+        const u64 *D = j == j0 ? J.d + (size_t)t * N : J.tmp + ((size_t)j * nt + t) * N;
+        if constexpr (GAL)
+            gs.load(D, x);
+        else
+            ldv<V>(D + n, x);
         key_macv<CK, V>(J.key, j, t, n, nfull, T.logN, mc.q, x, sb, sa);
     }
-    const u64 *v = J.tmp + (size_t)J.nd * nt * N;
     u64 vb[V], va[V], o0[V], o1[V];
-    ldv<V>(v + (size_t)t * N + n, vb);
-    ldv<V>(v + (size_t)(nact + t) * N + n, va);
+    ldv<V>(J.v + (size_t)t * N + n, vb);
+    ldv<V>(J.v + (size_t)(nact + t) * N + n, va);
     const u64 qlz = mc.flz;
 #pragma unroll
     for (int c = 0; c < V; ++c) {
@@ -665,9 +613,8 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
         add_bup(bu, T, BUpJob{J.y, J.tmp, (size_t)nt * N, J.nact, 0, nt, 0, -1});
         add_map(mD, LimbMap{J.tmp, J.tmp, nullptr, nt, nt, 0, 0, J.nact, 0}, J.nd * nt);
         add_map(mw, LimbMap{J.cp, J.cp, nullptr, K, nt, J.nact, J.nact, J.nact, -1}, 2 * K);
-        u64 *v = J.tmp + (size_t)J.nd * nt * N;
-        add_bdn(bd, BDnJob{J.cp, (size_t)nt * N, v, (size_t)J.nact * N, J.nact, 2});
-        add_map(mv, LimbMap{v, v, nullptr, J.nact, J.nact, 0, 0, J.nact, -1}, 2 * J.nact);
+        add_bdn(bd, BDnJob{J.cp, (size_t)nt * N, J.v, (size_t)J.nact * N, J.nact, 2});
+        add_map(mv, LimbMap{J.v, J.v, nullptr, J.nact, J.nact, 0, 0, J.nact, -1}, 2 * J.nact);
         oj.job[i] = J;
         oj.pre[i + 1] = oj.pre[i] + J.nact;
     }
@@ -683,20 +630,62 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     if (grouped)  // P4+P5, P towers
         comb_grouped(T, oj, kg, true, st);
     else if (ck)
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, 1>, gp, 256, 0, T, oj)));
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, false, 1>, gp, 256, 0, T, oj)));
     else
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, 1>, gp, 256, 0, T, oj)));
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, false, 1>, gp, 256, 0, T, oj)));
     if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;    // ModDown P1
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;        // ModDown P2
     if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;    // ModDown P3
     if (grouped)  // P4+P5 Q, ModDown P4
         comb_grouped(T, oj, kg, false, st);
     else if (ck)
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, 4>, gq, 256, 0, T, oj)));
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, false, 4>, gq, 256, 0, T, oj)));
     else
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, 4>, gq, 256, 0, T, oj)));
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, false, 4>, gq, 256, 0, T, oj)));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC whole-basis launch: ") + cudaGetErrorString(e));
+    return KS_OK;
+}
+
+// Key products and ModDowns of rotations that share their raised digits (J.tmp
+// holds D, J.v and J.cp are the job's own; one level): P-tower combine, ModDown
+// P1-P3, then the Q-tower combine with the subtraction, each one launch for all
+// rotations.  Per rotation the key is streamed once and c' of the Q towers never
+// written: 8 rotations at N = 2^16, 24 + 8 primes, 898 -> 713 us (a launch per
+// rotation before, two coefficients a thread now).
+int launch_oc_hoisted(const Tables &T, int n, const OcJob *jobs, cudaStream_t st)
+{
+    const size_t N = (size_t)1 << T.logN;
+    const int K = T.kp, nact = jobs[0].nact, nt = nact + K;
+    int rc;
+    LimbMaps mw, mv;
+    mw.n = mv.n = 0;
+    BDnJobs bd;
+    bd.n = 0;
+    OcJobs oj;
+    oj.n = n;
+    for (int i = 0; i < n; ++i) {
+        const OcJob &J = jobs[i];
+        add_map(mw, LimbMap{J.cp, J.cp, nullptr, K, nt, nact, nact, nact, -1}, 2 * K);
+        add_bdn(bd, BDnJob{J.cp, (size_t)nt * N, J.v, (size_t)nact * N, nact, 2});
+        add_map(mv, LimbMap{J.v, J.v, nullptr, nact, nact, 0, 0, nact, -1}, 2 * nact);
+        oj.job[i] = J;
+    }
+    const bool ck = any_compressed(oj);
+    const dim3 gp((unsigned)(N / 512), n * K), gq((unsigned)(N / 512), n * nact);
+    if (ck)
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, true, 2>, gp, 256, 0, T, oj)));
+    else
+        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, true, 2>, gp, 256, 0, T, oj)));
+    if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;
+    if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;
+    if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;
+    if (ck)
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, true, 2>, gq, 256, 0, T, oj)));
+    else
+        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, true, 2>, gq, 256, 0, T, oj)));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(KS_ECUDA, std::string("hoisted rotations launch: ") + cudaGetErrorString(e));
     return KS_OK;
 }
 
