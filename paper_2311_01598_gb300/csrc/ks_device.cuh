@@ -543,8 +543,8 @@ struct Shape {
     // threads, 4 rows at 2^16: each block barrier holds only two warps, and
     // the forward row pass ran 6% faster with 8-row and 2% faster again with
     // 4-row blocks than with 16-row ones; 8-column column-pass blocks were
-    // slower); the 32-value column pass of 2^17 stays at the compiler's
-    // default (it would spill).
+    // slower); the 32-value forward column pass of 2^17 stays at the
+    // compiler's default (it would spill).
     static constexpr int MINB_A = LA <= 8 ? 4 : 1;
     static constexpr int MINB_B = 16;
     // The forward row kernel stages its rows' first-round twiddles (REGB

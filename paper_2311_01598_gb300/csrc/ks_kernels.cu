@@ -278,18 +278,16 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const ulonglong2 *twt = T.itw + ((size_t)L.tf << S::LOGN);
-    ColStage<S> stage;  // in flight across pdl_wait (2^17: 92 -> 87 us; the forward pass gained nothing)
-    stage.load(twt);
+    pdl_wait();
+    for (int i = threadIdx.x; i < (1 << S::LA); i += S::THREADS_A) tws[i] = twt[i];
     const int cc = threadIdx.x % S::COLS, tau = threadIdx.x / S::COLS;
     const int c = blockIdx.x * S::COLS + cc;
     constexpr int M = S::TA, NG = S::REGA / S::TA;
     u64 x[S::REGA];
-    pdl_wait();
 #pragma unroll
     for (int gg = 0; gg < NG; ++gg)
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) x[gg * M + k2] = L.src[((size_t)((tau * NG + gg) * M + k2) << S::LB) + c];
-    stage.store(tws);
     __syncthreads();
     fold_all<S::REGA, AR>(x, md);
     inv_round2<S::LA, S::RA, AR>(x, tau, TwSmem{tws}, md);
@@ -309,12 +307,104 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
         L.dst[((size_t)(k * S::TA + tau) << S::LB) + c] = inv_finish<AR, SC>(x[k], f, mc);
 }
 
+// Inverse column pass of nine stages (N = 2^17) in three rounds of three: 512
+// threads hold 16 columns with 16 values each, two groups of eight a round,
+// regrouped twice through shared memory.  The two-round form (k_inv_col) needs 32
+// values and 184 registers a thread, one block of 8 warps an SM; this one fits
+// 64, two blocks of 16 warps: 75 limbs 88 -> 75 us.  The forward pass stays in two
+// rounds (128 registers; 225 limbs 147 us against 158 in three).
+struct Col9 {
+    static constexpr int COLS = 16, THREADS = 512, SMEM = 512 * COLS * 8 + 512 * 16;
+    // Row of value m of group gg in round R (stages 3R..3R+2): thread tau's group
+    // is pair p = gg*32 + tau, sub-transform p / L at offset p % L.
+    template <int R> __device__ static __forceinline__ int row(int tau, int gg, int m)
+    {
+        constexpr int L = 512 >> (3 * R + 3);
+        const int p = gg * 32 + tau;
+        return (p / L) * (8 * L) + m * L + p % L;
+    }
+    template <int R> __device__ static __forceinline__ void get(u64 (&x)[16], const u64 *sm, int tau, int cc)
+    {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = sm[row<R>(tau, i / 8, i % 8) * COLS + cc];
+    }
+    template <int R> __device__ static __forceinline__ void put(const u64 (&x)[16], u64 *sm, int tau, int cc)
+    {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sm[row<R>(tau, i / 8, i % 8) * COLS + cc] = x[i];
+    }
+    template <int R, int AR>
+    __device__ static __forceinline__ void inv(u64 (&x)[16], int tau, const ulonglong2 *tws, const ModR<AR> &md)
+    {
+        constexpr int L = 512 >> (3 * R + 3);
+        fold_all<16, AR>(x, md);
+#pragma unroll
+        for (int i = 2; i >= 0; --i) {
+            const int half = 4 >> i;
+#pragma unroll
+            for (int gg = 0; gg < 2; ++gg)
+#pragma unroll
+                for (int b = 0; b < (1 << i); ++b) {
+                    const ulonglong2 W = tws[(1 << (3 * R + i)) + (((gg * 32 + tau) / L) << i) + b];
+#pragma unroll
+                    for (int k = 0; k < half; ++k)
+                        inv_bfly<AR>(x[gg * 8 + b * 2 * half + k], x[gg * 8 + b * 2 * half + k + half], W, md,
+                                     inv_fold(k, half));
+                }
+        }
+    }
+};
+
+template <class S, bool SC, int AR>
+__global__ void __launch_bounds__(Col9::THREADS, 2) k_inv_col9(Tables T, LimbMaps ms)
+{
+    static_assert(S::LA == 9, "nine column stages");
+    pdl_start();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    u64 *sm = reinterpret_cast<u64 *>(smem_raw);
+    ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + 512 * Col9::COLS);
+    const int lz = blockIdx.y + blockIdx.z * gridDim.y;
+    if (lz >= ms.pre[ms.n]) return;
+    // limbs in reverse order: the row pass wrote the last ones most recently
+    const LimbRef L = limb_ref(ms, ms.pre[ms.n] - 1 - lz, T.nq, T.alpha, S::LOGN);
+    if (L.skip) return;
+    const ModC &mc = T.modc[L.tf];
+    const ModR<AR> md = mod_inv<AR>(mc);
+    tws[threadIdx.x] = T.itw[((size_t)L.tf << S::LOGN) + threadIdx.x];
+    const int cc = threadIdx.x % Col9::COLS, tau = threadIdx.x / Col9::COLS;
+    const int c = blockIdx.x * Col9::COLS + cc;
+    u64 x[16];
+    pdl_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = L.src[((size_t)Col9::row<2>(tau, i / 8, i % 8) << S::LB) + c];
+    __syncthreads();
+    Col9::inv<2, AR>(x, tau, tws, md);
+    Col9::put<2>(x, sm, tau, cc);
+    __syncthreads();
+    Col9::get<1>(x, sm, tau, cc);
+    Col9::inv<1, AR>(x, tau, tws, md);
+    Col9::put<1>(x, sm, tau, cc);  // the words this thread read
+    __syncthreads();
+    Col9::get<0>(x, sm, tau, cc);
+    Col9::inv<0, AR>(x, tau, tws, md);
+    ulonglong2 f = make_ulonglong2(0, 0);
+    if (SC) f = L.scale ? L.scale[L.b] : make_ulonglong2(mc.ninv, mc.ninv_sh);
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+        L.dst[((size_t)Col9::row<0>(tau, i / 8, i % 8) << S::LB) + c] = inv_finish<AR, SC>(x[i], f, mc);
+}
+
 template <class S, int AR>
 static void set_smem_attrs_ar()
 {
     cudaFuncSetAttribute(k_fwd_col<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_inv_col<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
-    cudaFuncSetAttribute(k_inv_col<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+    if constexpr (S::LA == 9) {
+        cudaFuncSetAttribute(k_inv_col9<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Col9::SMEM);
+        cudaFuncSetAttribute(k_inv_col9<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Col9::SMEM);
+    } else {
+        cudaFuncSetAttribute(k_inv_col<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+        cudaFuncSetAttribute(k_inv_col<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_A);
+    }
     cudaFuncSetAttribute(k_fwd_row<S, true, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
     cudaFuncSetAttribute(k_fwd_row<S, false, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
     cudaFuncSetAttribute(k_inv_row<S, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BT);
@@ -358,7 +448,7 @@ static void fwd_col_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))));
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
 }
 
 // Persistent grid of the staged row pass: resident CTAs per SM x SMs, at
@@ -430,10 +520,20 @@ static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStrea
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    if (scaled)
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
-    else
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, false, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
+    if constexpr (S::LA == 9) {
+        const dim3 g9 = limb_grid((1 << S::LB) / Col9::COLS, m.pre[m.n]);
+        constexpr int TH = Col9::THREADS, SM = Col9::SMEM;
+        if (scaled)
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, true, AR>, g9, TH, SM, T, m))))
+        else
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, false, AR>, g9, TH, SM, T, m))))
+    } else {
+        constexpr int TH = S::THREADS_A, SM = S::SMEM_A;
+        if (scaled)
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, TH, SM, T, m))))
+        else
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, false, AR>, ga, TH, SM, T, m))))
+    }
 }
 
 #define KS_DISPATCH_LOGN(logN, FN, ...)                                                                   \

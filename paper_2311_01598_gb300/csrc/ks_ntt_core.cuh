@@ -56,30 +56,6 @@ __device__ __forceinline__ void stage_row_round1(ulonglong2 *sh, const ulonglong
         sh[f] = __ldg(t + (G << st) + f + 1 - (1 << st));
     }
 }
-// The column pass's twiddles (the first 2^LA of the tower's table) on their way
-// to shared memory, the loads and the stores apart.
-template <class S>
-struct ColStage {
-    static constexpr int N = ((1 << S::LA) + S::THREADS_A - 1) / S::THREADS_A;
-    ulonglong2 v[N];
-    __device__ __forceinline__ void load(const ulonglong2 *t)
-    {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const int f = threadIdx.x + i * S::THREADS_A;
-            v[i] = f < (1 << S::LA) ? __ldg(t + f) : make_ulonglong2(0, 0);
-        }
-    }
-    __device__ __forceinline__ void store(ulonglong2 *sh) const
-    {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const int f = threadIdx.x + i * S::THREADS_A;
-            if (f < (1 << S::LA)) sh[f] = v[i];
-        }
-    }
-};
-
 // Twiddle fetcher of the forward row pass: first round from the staged row
 // block, second round from the tower table.
 template <class S>
