@@ -89,6 +89,8 @@ def lib_path() -> str:
 def lib():
     """Load the CUDA library (raises if it was not built)."""
     global _lib
+    if _lib is not None:  # loaded: no lock on the calls' path
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -226,10 +228,20 @@ def check(rc: int) -> None:
         raise KSError(rc, lib().ks_last_error().decode())
 
 
+_torch_cuda = None
+
+
 def _stream_handle(stream) -> ctypes.c_void_p:
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
+        # torch's current stream as its raw handle: building a torch Stream
+        # object for it costs 3 us a call, a fifth of a small transform
+        global _torch_cuda
+        if _torch_cuda is None:
+            import torch
+            torch.cuda.current_stream()  # initialises CUDA in torch, as before
+            _torch_cuda = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        raw, device = _torch_cuda
+        return ctypes.c_void_p(raw(device()))
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
