@@ -595,8 +595,10 @@ __device__ __forceinline__ void fwd_round1(u64 (&x)[1 << RR], const TW &tw, cons
 // tau is group tau*NG + gg of the sub-transform (the high RR bits of the
 // index).  tw.r2(s, s2, tau, gg, g2) is the twiddle of stage s = RR + s2 and
 // sub-group g2 of that group.
-template <int L, int RR, int AR, class TW>
-__device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m)
+// The first NPRE twiddles, in the order stage, sub-group, group, come from pre.
+template <int L, int RR, int AR, int NPRE = 0, class TW>
+__device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m,
+                                           const ulonglong2 *pre = nullptr)
 {
     constexpr int M = 1 << (L - RR);
     constexpr int NG = (1 << RR) / M;
@@ -607,7 +609,8 @@ __device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int tau, const TW 
         for (int gg = 0; gg < NG; ++gg) {
 #pragma unroll
             for (int g2 = 0; g2 < (1 << s2); ++g2) {
-                const ulonglong2 W = tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
+                const int e = ((1 << s2) - 1 + g2) * NG + gg;
+                const ulonglong2 W = e < NPRE ? pre[e] : tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
 #pragma unroll
                 for (int k = 0; k < half; ++k)
                     fwd_bfly<AR>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W, m);
@@ -616,9 +619,11 @@ __device__ __forceinline__ void fwd_round2(u64 (&x)[1 << RR], int tau, const TW 
     }
 }
 
-// Inverse of fwd_round2: local stages L-1 .. RR on the low bits.
-template <int L, int RR, int AR, class TW>
-__device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m)
+// Inverse of fwd_round2: local stages L-1 .. RR on the low bits.  The first
+// stage's first NPRE twiddles, in the order sub-group, group, come from pre.
+template <int L, int RR, int AR, int NPRE = 0, class TW>
+__device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int tau, const TW &tw, const ModR<AR> &m,
+                                           const ulonglong2 *pre = nullptr)
 {
     constexpr int M = 1 << (L - RR);
     constexpr int NG = (1 << RR) / M;
@@ -629,7 +634,8 @@ __device__ __forceinline__ void inv_round2(u64 (&x)[1 << RR], int tau, const TW 
         for (int gg = 0; gg < NG; ++gg) {
 #pragma unroll
             for (int g2 = 0; g2 < (1 << s2); ++g2) {
-                const ulonglong2 W = tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
+                const int e = s2 == L - RR - 1 ? g2 * NG + gg : NPRE;
+                const ulonglong2 W = e < NPRE ? pre[e] : tw.template r2<NG>(RR + s2, s2, tau, gg, g2);
 #pragma unroll
                 for (int k = 0; k < half; ++k)
                     inv_bfly<AR>(x[gg * M + g2 * 2 * half + k], x[gg * M + g2 * 2 * half + k + half], W, m,
@@ -666,6 +672,13 @@ __device__ __forceinline__ void inv_round1(u64 (&x)[1 << RR], const TW &tw, cons
 // made each load touch lines 2^s2 * 16 bytes apart, and the L1 pipeline, 90%
 // busy, bounded the row passes (1920 forward limbs of 2^16: 569 -> 494 us; 640
 // inverse ones: 250 -> 205 us).
+// A table load issued where it stands (a plain one is moved to its use).
+__device__ __forceinline__ ulonglong2 ldg_now(const ulonglong2 *p)
+{
+    ulonglong2 r;
+    asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(r.x), "=l"(r.y) : "l"(p));
+    return r;
+}
 struct TwSmem {
     const ulonglong2 *t;
     __device__ __forceinline__ ulonglong2 operator()(int s, int i) const { return t[(1 << s) + i]; }
@@ -682,6 +695,10 @@ struct TwRow {
     template <int NG> __device__ __forceinline__ ulonglong2 r2(int s, int, int tau, int gg, int g2) const
     {
         return __ldg(t + (G << s) + (g2 * NG + gg) * S::TB + tau);
+    }
+    template <int NG> __device__ __forceinline__ ulonglong2 r2v(int s, int tau, int gg, int g2) const
+    {
+        return ldg_now(t + (G << s) + (g2 * NG + gg) * S::TB + tau);
     }
 };
 
