@@ -188,10 +188,11 @@ struct OcJob {
     int nact, nd;
 };
 // The jobs of one Output-Centric launch group, with prefix counts of their Q
-// towers: job j owns Q-section items [pre[j], pre[j+1]).
+// towers: job j owns Q-section items [pre[j], pre[j+1]); whole-basis groups
+// whose jobs share keys count them by tower instead (oc_shared_keys, ks_oc.cu).
 struct OcJobs {
     int n;
-    int pre[kMaxBatch + 1];
+    int pre[(kMaxBatch > kMaxQ ? kMaxBatch : kMaxQ) + 1];
     OcJob job[kMaxBatch];
 };
 // Scratch words one job needs at level nact.

@@ -502,34 +502,55 @@ size_t oc_scratch_words(const Tables &T, int nact)
 }
 
 // Whole-basis variant: tmp holds D [nd][nact+K] then v [2][nact].
-// P-tower combine of this layout: c'_{x,p_k} from D rows at tower nact+k.
-// grid (N/(256V), jobs*K).  GAL: hoisted rotations, jobs of one level that share
-// D and d and read them through their own automorphism; the jobs of a tower lie
-// next to each other in the grid, so that its rows of D come from L2 for all but
-// the first.
-template <bool CK, bool GAL, int V>
+// The order of its combine kernels' blocks:
+//   COMB_PLAIN   job by job, tower by tower; grid (N/(256V), rows);
+//   COMB_SHARED  full keys, and some jobs share one (a busy evaluator has more
+//                ciphertexts than keys; half a compressed key is regenerated, and
+//                6 jobs of 3 such keys at N = 2^14 lost 2 us of 121 this way): tower by tower, block of coefficients by block of
+//                coefficients, the jobs next to each other, so that a key's
+//                words are in L2 for all but the first of its jobs; grid
+//                (rows * N/(256V)), oj by falling level with oj.pre[t] the
+//                (tower, job) pairs below tower t.  64 jobs of 16 keys: Q combine
+//                855 -> 752 us, P combine 398 -> 380; without shared keys the
+//                plain order is the faster one (16 jobs: 2117 us a step, 2126);
+//   COMB_GAL     hoisted rotations, jobs of one level that share D and d and read
+//                them through their own automorphism: the jobs of a tower next
+//                to each other, so that its rows of D come from L2 for all but
+//                the first; grid (N/(256V), rows).
+enum { COMB_PLAIN = 0, COMB_SHARED = 1, COMB_GAL = 2 };
+// P-tower combine: c'_{x,p_k} from D rows at tower nact+k; jobs*K rows.
+template <bool CK, int ORDER, int V>
 __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
 {
     pdl_start();
     pdl_wait();
     const int K = T.kp;
-    const OcJob &J = oj.job[GAL ? blockIdx.y % oj.n : blockIdx.y / K];
-    const int k = GAL ? blockIdx.y / oj.n : blockIdx.y % K;
+    const size_t N = (size_t)1 << T.logN;
+    unsigned jb, k, cb = blockIdx.x;
+    if constexpr (ORDER == COMB_SHARED) {
+        const unsigned nb = (unsigned)(N / (256 * V)), r = blockIdx.x / oj.n;
+        jb = blockIdx.x % oj.n;
+        k = r / nb;
+        cb = r % nb;
+    } else {
+        jb = ORDER == COMB_GAL ? blockIdx.y % oj.n : blockIdx.y / K;
+        k = ORDER == COMB_GAL ? blockIdx.y / oj.n : blockIdx.y % K;
+    }
+    const OcJob &J = oj.job[jb];
     const int tf = T.nq + k;
     const int t = J.nact + k;
     const int nt = J.nact + K;
     const int nfull = T.nq + K;
-    const size_t N = (size_t)1 << T.logN;
-    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const size_t n = ((size_t)cb * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[tf];
-    const GaloisSlots<V> gs(n, GAL ? J.gal : 1, T.logN);
+    const GaloisSlots<V> gs(n, ORDER == COMB_GAL ? J.gal : 1, T.logN);
     U128 sb[V], sa[V];
 #pragma unroll
     for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
     for (int j = 0; j < J.nd; ++j) {
         u64 x[V];
         const u64 *D = J.tmp + ((size_t)j * nt + t) * N;
-        if constexpr (GAL)
+        if constexpr (ORDER == COMB_GAL)
             gs.load(D, x);
         else
             ldv<V>(D + n, x);
@@ -545,33 +566,43 @@ __global__ void __launch_bounds__(256) k_oc_comb_pw(Tables T, OcJobs oj)
     stv<V>(J.cp + (size_t)(nt + t) * N + n, oa);
 }
 
-// Q-tower combine of the whole-basis layout.  grid (N/(256V), sum of nact).
+// Q-tower combine; sum of nact rows.
 // Four CTAs per SM (64 registers, a few spilled words): more loads in flight
 // than three CTAs at the compiler's 74 registers (0.92 -> 0.95 of the copy
 // bandwidth on the benchmark step).
-template <bool CK, bool GAL, int V>
+template <bool CK, int ORDER, int V>
 __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
 {
     pdl_start();
     pdl_wait();
-    const int jb = GAL ? blockIdx.y % oj.n : find_slot(oj.pre, oj.n, blockIdx.y);
+    const size_t N = (size_t)1 << T.logN;
+    unsigned jb, cb = blockIdx.x;
+    int t;
+    if constexpr (ORDER == COMB_SHARED) {
+        const unsigned nb = (unsigned)(N / (256 * V));
+        t = find_slot(oj.pre, oj.job[0].nact, blockIdx.x / nb);
+        const unsigned jobs = oj.pre[t + 1] - oj.pre[t], r = blockIdx.x - (unsigned)oj.pre[t] * nb;
+        jb = r % jobs;
+        cb = r / jobs;
+    } else {
+        jb = ORDER == COMB_GAL ? blockIdx.y % oj.n : find_slot(oj.pre, oj.n, blockIdx.y);
+        t = ORDER == COMB_GAL ? blockIdx.y / oj.n : blockIdx.y - oj.pre[jb];
+    }
     const OcJob &J = oj.job[jb];
-    const int t = GAL ? blockIdx.y / oj.n : blockIdx.y - oj.pre[jb];
     const int nact = J.nact;
     const int nt = nact + T.kp;
     const int j0 = t / T.alpha;
     const int nfull = T.nq + T.kp;
-    const size_t N = (size_t)1 << T.logN;
-    const size_t n = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const size_t n = ((size_t)cb * blockDim.x + threadIdx.x) * V;
     const ModC &mc = T.modc[t];
-    const GaloisSlots<V> gs(n, GAL ? J.gal : 1, T.logN);
+    const GaloisSlots<V> gs(n, ORDER == COMB_GAL ? J.gal : 1, T.logN);
     U128 sb[V], sa[V];
 #pragma unroll
     for (int c = 0; c < V; ++c) sb[c] = sa[c] = U128{0, 0};
     for (int j = 0; j < J.nd; ++j) {
         u64 x[V];
         const u64 *D = j == j0 ? J.d + (size_t)t * N : J.tmp + ((size_t)j * nt + t) * N;
-        if constexpr (GAL)
+        if constexpr (ORDER == COMB_GAL)
             gs.load(D, x);
         else
             ldv<V>(D + n, x);
@@ -590,6 +621,46 @@ __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
     }
     stv<V>(J.out0 + (size_t)t * N + n, o0);
     stv<V>(J.out1 + (size_t)t * N + n, o1);
+}
+
+// When two jobs share a key: the jobs by falling level and the towers' prefix
+// counts, for COMB_SHARED.
+static bool oc_shared_keys(OcJobs &oj)
+{
+    const u64 *keys[kMaxBatch];
+    for (int i = 0; i < oj.n; ++i) keys[i] = oj.job[i].key.evk;
+    std::sort(keys, keys + oj.n);
+    if (std::adjacent_find(keys, keys + oj.n) == keys + oj.n) return false;
+    std::stable_sort(oj.job, oj.job + oj.n, [](const OcJob &a, const OcJob &b) { return a.nact > b.nact; });
+    oj.pre[0] = 0;
+    for (int t = 0, jobs = oj.n; t < oj.job[0].nact; ++t) {
+        while (oj.job[jobs - 1].nact <= t) --jobs;
+        oj.pre[t + 1] = oj.pre[t] + jobs;
+    }
+    return true;
+}
+
+// Both combines of a whole-basis launch group.
+template <int ORDER>
+static void comb_whole(const Tables &T, const OcJobs &oj, bool p_section, bool ck, int rows, cudaStream_t st)
+{
+    // Q towers four coefficients a thread (two 16-byte accesses per stream), P
+    // towers, which have few rows, one (two measured slower); rotations two
+    constexpr int VP = ORDER == COMB_GAL ? 2 : 1, VQ = ORDER == COMB_GAL ? 2 : 4;
+    const unsigned nb = (unsigned)(((size_t)1 << T.logN) / (256 * (p_section ? VP : VQ)));
+    const dim3 g = ORDER == COMB_SHARED ? dim3(nb * (unsigned)rows) : dim3(nb, (unsigned)rows);
+    constexpr int CORDER = ORDER == COMB_SHARED ? COMB_PLAIN : ORDER;  // compressed keys: never COMB_SHARED
+    if (p_section) {
+        if (ck)
+            KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, CORDER, VP>, g, 256, 0, T, oj)));
+        else
+            KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, ORDER, VP>, g, 256, 0, T, oj)));
+    } else {
+        if (ck)
+            KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, CORDER, VQ>, g, 256, 0, T, oj)));
+        else
+            KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, ORDER, VQ>, g, 256, 0, T, oj)));
+    }
 }
 
 static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share_keys, cudaStream_t st)
@@ -624,24 +695,21 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     const bool ck = any_compressed(oj);
     KeyGroups kg;
     const bool grouped = share_keys && key_groups(oj, kg);
-    // Q towers four coefficients a thread (two 16-byte accesses per stream); the
-    // P-tower combine has few rows and keeps one (two measured slower)
-    const dim3 gp((unsigned)(N / 256), n * K), gq((unsigned)(N / 1024), oj.pre[n]);
-    if (grouped)  // P4+P5, P towers
-        comb_grouped(T, oj, kg, true, st);
-    else if (ck)
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, false, 1>, gp, 256, 0, T, oj)));
-    else
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, false, 1>, gp, 256, 0, T, oj)));
+    const int q_rows = oj.pre[n];  // before oc_shared_keys counts by tower
+    const bool shared = !grouped && !ck && oc_shared_keys(oj);
+    auto combine = [&](bool p_section) {
+        if (grouped)
+            comb_grouped(T, oj, kg, p_section, st);
+        else if (shared)
+            comb_whole<COMB_SHARED>(T, oj, p_section, ck, p_section ? n * K : q_rows, st);
+        else
+            comb_whole<COMB_PLAIN>(T, oj, p_section, ck, p_section ? n * K : q_rows, st);
+    };
+    combine(true);  // P4+P5, P towers
     if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;    // ModDown P1
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;        // ModDown P2
     if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;    // ModDown P3
-    if (grouped)  // P4+P5 Q, ModDown P4
-        comb_grouped(T, oj, kg, false, st);
-    else if (ck)
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, false, 4>, gq, 256, 0, T, oj)));
-    else
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, false, 4>, gq, 256, 0, T, oj)));
+    combine(false);  // P4+P5 Q, ModDown P4
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(KS_ECUDA, std::string("OC whole-basis launch: ") + cudaGetErrorString(e));
     return KS_OK;
@@ -672,18 +740,11 @@ int launch_oc_hoisted(const Tables &T, int n, const OcJob *jobs, cudaStream_t st
         oj.job[i] = J;
     }
     const bool ck = any_compressed(oj);
-    const dim3 gp((unsigned)(N / 512), n * K), gq((unsigned)(N / 512), n * nact);
-    if (ck)
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<true, true, 2>, gp, 256, 0, T, oj)));
-    else
-        KS_LAUNCH(st, "oc_comb_p", (launch_dep(st, k_oc_comb_pw<false, true, 2>, gp, 256, 0, T, oj)));
+    comb_whole<COMB_GAL>(T, oj, true, ck, n * K, st);
     if ((rc = launch_ntt_inv(T, mw, false, st)) != KS_OK) return rc;
     if ((rc = launch_bconv_down(T, bd, st)) != KS_OK) return rc;
     if ((rc = launch_ntt_fwd(T, mv, false, st)) != KS_OK) return rc;
-    if (ck)
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<true, true, 2>, gq, 256, 0, T, oj)));
-    else
-        KS_LAUNCH(st, "oc_comb_q", (launch_dep(st, k_oc_comb_qw<false, true, 2>, gq, 256, 0, T, oj)));
+    comb_whole<COMB_GAL>(T, oj, false, ck, n * nact, st);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(KS_ECUDA, std::string("hoisted rotations launch: ") + cudaGetErrorString(e));
     return KS_OK;

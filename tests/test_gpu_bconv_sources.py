@@ -54,3 +54,24 @@ def test_uneven_runs():
         for (_, _, _, o0, o1), (w0, w1) in zip(jobs, want):
             assert np.array_equal(ks.to_host(o0), w0) and np.array_equal(ks.to_host(o1), w1)
             o0.zero_(), o1.zero_()
+
+
+@pytest.mark.parametrize("njobs,nkeys", [(2, 1), (7, 3), (64, 5), (9, 9)])
+def test_shared_keys(njobs, nkeys):
+    """Batches whose jobs share keys at uneven levels (the combines' job-next-to-job
+    order), equal levels and the smallest ones among them."""
+    need_gpu()
+    ks = built_lib()
+    P, C = pair(10, 7, 2, 3)
+    evks = [np.stack([np.stack([inputs.uniform_towers(C.q + C.p, C.N, seed=1000 * k + 10 * j + x) for x in range(2)])
+                      for j in range(P.ndig)]) for k in range(nkeys)]
+    keys = [P.upload_key(e) for e in evks]
+    jobs, want = [], []
+    for i in range(njobs):
+        lv = 1 + (5 * i + i // 4) % 7
+        d = inputs.uniform_towers(C.q[:lv], C.N, seed=300 + i)
+        want.append(C.keyswitch(lv, d, evks[i % nkeys]))
+        jobs.append((keys[i % nkeys], lv, ks.to_device(d), ks.empty((lv, C.N)), ks.empty((lv, C.N))))
+    P.switch_batch(jobs, "OC")
+    for (_, _, _, o0, o1), (w0, w1) in zip(jobs, want):
+        assert np.array_equal(ks.to_host(o0), w0) and np.array_equal(ks.to_host(o1), w1)
