@@ -103,11 +103,13 @@ int ks_params_info(const ks_params *params, uint64_t *h_q, uint64_t *h_p,
                    uint32_t *alpha, uint32_t *n_digits);
 
 /* Implementation options of a parameter set (none changes any result).
- *   KS_OPT_BCONV_TENSOR (default 1): run the fast base conversions (ModUp P2,
+ *   KS_OPT_BCONV_TENSOR: 1 runs the fast base conversions (ModUp P2,
  *     ModDown P2) on the tensor cores (tcgen05, exact f16 slices)
  *     wherever at most 18 source towers meet (36 for primes just below a power
  *     of two, as the default rule gives); 0 selects the CUDA-core kernels
- *     everywhere.
+ *     everywhere.  As long as it is not set, conversions of at most 2^17
+ *     multiply-adds a digit (sources x targets x N at the top level) take the
+ *     CUDA cores and the others run as with 1.
  *   KS_OPT_BATCH_LANES (default 2, 1..4): an Output-Centric batch of at least
  *     4 jobs per lane is split over that many library streams, forked from
  *     and joined back to the caller's stream (the memory-bound combine

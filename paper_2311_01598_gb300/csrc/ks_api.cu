@@ -724,8 +724,8 @@ int ks_params_set_option(ks_params *P, int option, int value)
     std::lock_guard<std::mutex> g(P->mu);
     if (option == KS_OPT_BCONV_TENSOR && (value == 0 || value == 1)) {
         P->bconv_tensor = value;
-        P->tables.up_tc = value ? P->d_up_tc : nullptr;
-        P->tables.dn_tc = value ? P->d_dn_tc : nullptr;
+        P->tables.up_tc = up_tc_chosen(P) ? P->d_up_tc : nullptr;
+        P->tables.dn_tc = dn_tc_chosen(P) ? P->d_dn_tc : nullptr;
         return KS_OK;
     }
     if (option == KS_OPT_NTT_CLUSTER && value >= 0 && value <= 2) {

@@ -472,9 +472,9 @@ int build_tables(ks_params *P)
     T.key_sc = P->d_key_sc;
     T.plain_sc = P->d_plain_sc;
     T.up_mat_lvl = P->d_up_mat_lvl;
-    T.up_tc = P->bconv_tensor ? P->d_up_tc : nullptr;
+    T.up_tc = up_tc_chosen(P) ? P->d_up_tc : nullptr;
     T.up_tc_lvl = P->d_up_tc_lvl;
-    T.dn_tc = P->bconv_tensor ? P->d_dn_tc : nullptr;
+    T.dn_tc = dn_tc_chosen(P) ? P->d_dn_tc : nullptr;
     T.ntt_cluster = P->ntt_cluster;
     T.row_stage = P->row_stage;
     T.tc_below54 = below54;

@@ -127,7 +127,7 @@ struct ks_params {
     int *d_up_mat_lvl = nullptr;         // [nq levels][ndig]: ModUp matrix offsets per level
     uint4 *d_up_tc = nullptr, *d_dn_tc = nullptr;  // tensor-core BConv slabs
     int *d_up_tc_lvl = nullptr;
-    int bconv_tensor = 1;                // use the tensor-core BConv where supported
+    int bconv_tensor = -1;               // tensor-core BConv: -1 by size, 0 never, 1 wherever supported
     int ntt_cluster = 0;                 // NTTs as one cluster launch where supported
     int row_stage = 0;                   // forward row passes staged by bulk copies
     int batch_lanes = 2;                 // internal streams a large Output-Centric batch is split over
@@ -173,6 +173,28 @@ struct ks_key {
 };
 
 namespace ks {
+// Whether the base conversions of nsrc sources to ntgt targets use the tensor
+// cores.  By size: the tensor-core kernel has one CTA an SM, which allocates
+// tensor memory, stages its targets and then runs producers, MMA and epilogue one
+// after the other, 1.5 to 8 us a launch before its rate counts, and an output
+// costs it the same at one source as at nine; the CUDA-core kernel starts at once
+// and pays by the source.  One key switch (OC) and 24, us, tensor / CUDA cores:
+//   L+1, K, dnum     N = 2^12                  2^13                      2^14                      2^15
+//   3, 1, 3     35.3/31.1  84.7/72.5     50.3/42.6  122/94         60.9/57.4  178/140        69.3/72.1  306/251
+//   6, 2, 3     36.6/33.6  92.1/72.0     57.9/49.7  149/126        64.6/69.8  253/230        76.8/89.8  481/457
+//   9, 3, 3     41.5/38.1  109/102       59.3/62.7  186/190        68.6/86.2  341/371        92.3/101   667/755
+//   12, 2, 6    44.8/44.5  170/163       66.4/66.9  306/317        85.1/93.6  595/642        108/114    1178/1299
+//   24, 8, 3    52.5/57.3                74.7/80.4                 93.0/110                  124/140
+// so the line is drawn at 2^17 multiply-adds a digit (9 targets at three sources
+// and 2^12, 6 at two and 2^13, 8 at one and 2^14).
+inline bool bconv_tc_chosen(const ks_params *P, int nsrc, int ntgt)
+{
+    if (P->bconv_tensor >= 0) return P->bconv_tensor != 0;
+    return ((size_t)nsrc * ntgt << P->logN) > (size_t)1 << 17;
+}
+inline bool up_tc_chosen(const ks_params *P) { return bconv_tc_chosen(P, P->alpha, P->nq + P->kp - P->alpha); }
+inline bool dn_tc_chosen(const ks_params *P) { return bconv_tc_chosen(P, P->kp, P->nq); }
+
 inline KeyView key_view(const ks_key *K) { return KeyView{K->d_evk, K->a_seed, K->compressed}; }
 }  // namespace ks
 

@@ -356,8 +356,8 @@ class Params:
                               _stream_handle(stream)))
 
     def set_bconv_tensor(self, on: bool) -> None:
-        """KS_OPT_BCONV_TENSOR: base conversions on the tensor cores (default)
-        or on the CUDA cores."""
+        """KS_OPT_BCONV_TENSOR: base conversions on the tensor cores or on
+        the CUDA cores (until it is called: by the conversion's size)."""
         check(lib().ks_params_set_option(self.handle, 1, 1 if on else 0))
 
     def set_batch_lanes(self, lanes: int) -> None:

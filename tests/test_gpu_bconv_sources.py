@@ -75,3 +75,30 @@ def test_shared_keys(njobs, nkeys):
     P.switch_batch(jobs, "OC")
     for (_, _, _, o0, o1), (w0, w1) in zip(jobs, want):
         assert np.array_equal(ks.to_host(o0), w0) and np.array_equal(ks.to_host(o1), w1)
+
+
+@pytest.mark.parametrize("logN,nq,kp,dnum", [(12, 3, 1, 3), (12, 9, 3, 3), (13, 7, 2, 4), (13, 9, 2, 5), (14, 8, 1, 8),
+                                             (14, 9, 1, 9), (10, 12, 8, 2), (11, 5, 28, 1)])
+def test_engine_by_size(logN, nq, kp, dnum):
+    """Conversions on both sides of 2^17 multiply-adds: the size's engine, either
+    one asked for by the schedule or the option, and the oracle agree."""
+    need_gpu()
+    ks = built_lib()
+    P, C = pair(logN, nq, kp, dnum)
+    evk = np.stack([np.stack([inputs.uniform_towers(C.q + C.p, C.N, seed=10 * j + x) for x in range(2)])
+                    for j in range(P.ndig)])
+    key = P.upload_key(evk)
+    for nact in (nq, 1):
+        d = inputs.uniform_towers(C.q[:nact], C.N, seed=nact)
+        want = C.keyswitch(nact, d, evk)
+        dd = ks.to_device(d)
+        for option in (None, True, False):
+            if option is not None:
+                P.set_bconv_tensor(option)
+            for df in (0, 1, 2):
+                for engine in (-1, 0, 1):
+                    o = ks.empty((nact, C.N)), ks.empty((nact, C.N))
+                    P.switch_batch_sched([(key, nact, dd, *o)], ks.Schedule(df, 2, 64, 0, -1, engine))
+                    for x in (0, 1):
+                        assert np.array_equal(ks.to_host(o[x]), want[x]), (option, df, engine, nact)
+    assert P.device_status() == 0
