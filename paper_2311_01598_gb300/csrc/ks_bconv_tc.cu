@@ -12,8 +12,8 @@
 //   z_t == sum_b 2^(Wb) P_{t,b}  (mod r_t),
 //   P_{t,b} = sum_i sum_a y_{i,a} c'_{i,a,t,b},
 // and every P_{t,b} (at most 18 sources x 7 bytes x 255^2, or 9 x 7 x 255 x
-// 511 with W = 9, below 2^23) is an exact integer in the fp32 accumulator.  One MMA of M=128 coefficients,
-// K = 7*(sources) padded to 64 (up to 9 sources) or 128 (up to 18: two K
+// 511 with W = 9, below 2^23) is an exact integer in the fp32 accumulator.
+// One MMA of M=128 coefficients, K = 7*(sources) padded to 64 (up to 9 sources) or 128 (up to 18: two K
 // blocks), N = 8 per target (7 byte rows used) computes
 // all P_{t,b} of up to 32 targets.  19 to 36 sources take two such A tiles with
 // an accumulator each, added in the epilogue (16 targets at a time).  The A
@@ -181,7 +181,7 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t phase)
 // targets of one (job, digit) (ModUp) or (job, polynomial) (ModDown).
 struct TcItem {
     const u64 *src;     // source tower 0 at the tile's first coefficient; tower i at + i*N
-    int nsrc;           // source towers (<= 18)
+    int nsrc;           // source towers (<= 36)
     int G;              // targets (0: nothing to do)
     int key;            // (job block, target block): the B slabs and targets change with it
     int sbase;          // slab index base (ModUp: of the digit at this level)

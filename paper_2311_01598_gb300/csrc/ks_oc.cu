@@ -17,6 +17,11 @@
 //                 pass of the ModDown limbs (ModDown P3) and the subtraction
 //                 (ModDown P4) written to the output.
 // The key is read once, inside the fused row kernels, while they compute.
+//
+// The whole-basis form (the default's launches, launch_oc_whole) keeps the order
+// of special towers before Q towers but converts and transforms the digits to
+// every tower at once, and forms the key products in streaming combine kernels:
+// larger launches than the two sections', faster in every batch measured.
 #include <algorithm>
 
 #include "ks_ntt_core.cuh"

@@ -181,19 +181,7 @@ static void scheduler(ks_server *S)
                 Req &r = S->reqs[take[i]];
                 r.state = 1;
                 r.t_admit = t;
-                const int nact = (int)r.nact;
-                const int nd = (nact + P0->alpha - 1) / P0->alpha;
-                OcJob &J = jobs[i];
-                J.d = r.d;
-                J.out0 = r.o0;
-                J.out1 = r.o1;
-                J.key = key_view(r.K);
-                J.y = (u64 *)(S->pool_mem + r.off);
-                J.tmp = J.y + (size_t)nact * P0->N;
-                J.cp = J.tmp + ((size_t)nd * (nact + P0->kp) + 2 * (size_t)nact) * P0->N;
-                J.pre = P0->d_up_pre_lvl + (size_t)(nact - 1) * P0->nq;
-                J.nact = nact;
-                J.nd = nd;
+                jobs[i] = oc_job(P0, r.K, (int)r.nact, r.d, r.o0, r.o1, (u64 *)(S->pool_mem + r.off));
             }
             S->inflight_jobs += (uint32_t)take.size();
             cudaStream_t lane = S->lanes[li];
