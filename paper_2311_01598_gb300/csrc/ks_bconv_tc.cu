@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(TC_PIPE_THREADS, 1) k_bconv_tc(Tables T, BUpJo
     __shared__ int s_G[2], s_off[2];  // of the item in each buffer: targets, coefficients past the stretch's first
     pdl_start();
     const int i0 = tc_run_start(split, blockIdx.x, gridDim.x), i1 = tc_run_start(split, blockIdx.x + 1, gridDim.x);
-    if (i0 >= i1) return;
+    if (i0 >= i1) return pdl_wait();
     const size_t N = (size_t)1 << T.logN;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     if (tid == 0) {
@@ -652,16 +652,7 @@ static int launch_tc_for(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, 
 
 int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, const int *, cudaStream_t st)
 {
-    int span = 0;  // most targets of any (job, digit): the range minus the digit's own towers
-    for (int i = 0; i < b.n; ++i) {
-        const BUpJob &J = b.job[i];
-        const int nd = (J.nact + T.alpha - 1) / T.alpha;
-        for (int j = (J.jsel >= 0 ? J.jsel : 0); j < (J.jsel >= 0 ? J.jsel + 1 : nd); ++j) {
-            const int lo = j * T.alpha, hi = std::min(lo + T.alpha, J.nact);
-            const int olo = std::max(lo, J.t_begin), ohi = std::min(hi, J.t_end);
-            span = std::max(span, (J.t_end - J.t_begin) - std::max(0, ohi - olo));
-        }
-    }
+    const int span = bup_span(T, b);
     if (span <= 0) return KS_OK;
     BDnJobs none;
     none.n = 0;

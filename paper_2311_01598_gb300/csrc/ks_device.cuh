@@ -43,8 +43,11 @@ namespace ks {
 // Kernels launched with launch_dep: pdl_start lets the next kernel of the stream
 // begin its own prologue once every block of this one has started; pdl_wait
 // holds a block until the stream's previous kernel is complete.  Before pdl_wait
-// a kernel reads only its parameters and the parameter set's tables.  Blocks
-// with nothing to do may leave without waiting: every launch has others.
+// a kernel reads only its parameters and the parameter set's tables.  Every
+// path out of a kernel passes pdl_wait, also that of a block with nothing to do:
+// a launch of such blocks alone (one digit's own towers, all of them bypassed)
+// would else be complete before its predecessor, and the kernel after it start
+// on data still being written.
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

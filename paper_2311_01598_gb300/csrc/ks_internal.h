@@ -220,8 +220,9 @@ class LaunchScope {
         __VA_ARGS__;                          \
     } while (0)
 
-// Launch of a kernel that begins with pdl_start and calls pdl_wait before it
-// touches anything earlier work may write (ks_device.cuh): the launch may start
+// Launch of a kernel that begins with pdl_start and whose every block calls
+// pdl_wait, before it touches anything earlier work may write and before it
+// leaves (ks_device.cuh): the launch may start
 // while the stream's previous kernel drains (programmatic dependent launch), so
 // its dispatch, its descriptors and the constants it stages overlap that
 // kernel's last wave.  Ordering is the stream's: pdl_wait returns when the

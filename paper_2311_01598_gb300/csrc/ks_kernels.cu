@@ -19,9 +19,9 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lg >= ms.pre[ms.n]) return;
+    if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModR<AR> md = mod_fwd<AR>(T.modc[L.tf]);
     const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
     pdl_wait();
@@ -61,12 +61,12 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, L
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lz = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lz >= ms.pre[ms.n]) return;
+    if (lz >= ms.pre[ms.n]) return pdl_wait();
     // limbs in reverse order: the column pass wrote the last ones most
     // recently, so the first blocks find their rows in L2
     const int lg = ms.pre[ms.n] - 1 - lz;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_fwd<AR>(mc);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
@@ -235,9 +235,9 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lg >= ms.pre[ms.n]) return;
+    if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModR<AR> md = mod_inv<AR>(T.modc[L.tf]);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
@@ -270,11 +270,11 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
     const int lz = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lz >= ms.pre[ms.n]) return;
+    if (lz >= ms.pre[ms.n]) return pdl_wait();
     // limbs in reverse order: the row pass wrote the last ones most recently
     const int lg = ms.pre[ms.n] - 1 - lz;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const ulonglong2 *twt = T.itw + ((size_t)L.tf << S::LOGN);
@@ -364,10 +364,10 @@ __global__ void __launch_bounds__(Col9::THREADS, 2) k_inv_col9(Tables T, LimbMap
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + 512 * Col9::COLS);
     const int lz = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lz >= ms.pre[ms.n]) return;
+    if (lz >= ms.pre[ms.n]) return pdl_wait();
     // limbs in reverse order: the row pass wrote the last ones most recently
     const LimbRef L = limb_ref(ms, ms.pre[ms.n] - 1 - lz, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     tws[threadIdx.x] = T.itw[((size_t)L.tf << S::LOGN) + threadIdx.x];
@@ -623,6 +623,21 @@ void add_bup(BUpJobs &b, const Tables &T, const BUpJob &j)
     b.n += 1;
 }
 
+int bup_span(const Tables &T, const BUpJobs &b)
+{
+    int span = 0;
+    for (int i = 0; i < b.n; ++i) {
+        const BUpJob &J = b.job[i];
+        const int nd = (J.nact + T.alpha - 1) / T.alpha;
+        for (int j = (J.jsel >= 0 ? J.jsel : 0); j < (J.jsel >= 0 ? J.jsel + 1 : nd); ++j) {
+            const int lo = j * T.alpha, hi = std::min(lo + T.alpha, J.nact);
+            const int olo = std::max(lo, J.t_begin), ohi = std::min(hi, J.t_end);
+            span = std::max(span, (J.t_end - J.t_begin) - std::max(0, ohi - olo));
+        }
+    }
+    return span;
+}
+
 // ModUp P2: grid (N/256, ceil(max targets/TT), digit blocks of all jobs).
 __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_up(Tables T, BUpJobs bj)
 {
@@ -641,7 +656,7 @@ __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_up(Tables T, BUpJobs bj
     const int ov = ohi > olo ? ohi - olo : 0;
     const int nb = (J.t_end - J.t_begin) - ov;
     const int u0 = blockIdx.y * BC_TT;
-    if (u0 >= nb) return;
+    if (u0 >= nb) return pdl_wait();
     const int nfull = T.nq + T.kp;
     const u64 *mat = T.up_mat + T.up_mat_lvl[(size_t)(nact - 1) * T.ndig + j];
     if (threadIdx.x < BC_TT) {
@@ -694,8 +709,7 @@ int launch_bconv_up(const Tables &T, const BUpJobs &b, cudaStream_t st)
 {
     if (b.n == 0) return KS_OK;
     if (T.up_tc && bconv_tc_supported(T, T.alpha)) return launch_bconv_up_tc(T, b, T.up_tc, T.up_tc_lvl, st);
-    int span = 0;
-    for (int i = 0; i < b.n; ++i) span = std::max(span, b.job[i].t_end - b.job[i].t_begin);
+    const int span = bup_span(T, b);
     if (span <= 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
     dim3 g((unsigned)(N / BC_THREADS), (unsigned)((span + BC_TT - 1) / BC_TT), (unsigned)b.zpre[b.n]);
@@ -722,7 +736,7 @@ __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_down(Tables T, BDnJobs 
     const int nact = J.nact;
     const int ib = J.i_begin, ie = J.i_end < 0 ? nact : J.i_end;
     const int i0 = ib + blockIdx.y * BC_TT;  // first target tower of the block
-    if (i0 >= ie) return;
+    if (i0 >= ie) return pdl_wait();
     const int K = T.kp;
     for (int idx = threadIdx.x; idx < K * BC_TT; idx += blockDim.x) {
         const int k = idx / BC_TT, g = idx % BC_TT;

@@ -95,6 +95,9 @@ struct BUpJobs {
     BUpJob job[kMaxBatch];
 };
 void add_bup(BUpJobs &b, const Tables &T, const BUpJob &j);
+// Most targets of any (job, digit): the range minus the digit's own towers (0:
+// there is nothing to convert, and nothing is launched).
+int bup_span(const Tables &T, const BUpJobs &b);
 int launch_bconv_up(const Tables &T, const BUpJobs &b, cudaStream_t st);
 
 // ModDown P2: w = cp rows [nact, nact+K) of each polynomial (canonical,

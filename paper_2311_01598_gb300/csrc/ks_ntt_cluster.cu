@@ -35,9 +35,9 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(buf + G_::BUFW);
     ulonglong2 *tsh_all = tws + (1 << S::LA);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lg >= ms.pre[ms.n]) return;
+    if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_fwd<AR>(mc);
     const int r = cluster_rank();
@@ -103,9 +103,9 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
     u64 *buf = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(buf + G_::BUFW);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
-    if (lg >= ms.pre[ms.n]) return;
+    if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return;
+    if (L.skip) return pdl_wait();
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const int r = cluster_rank();
