@@ -1182,8 +1182,8 @@ int ks_ntt(const ks_params *P, uint32_t first_tower, uint32_t n_towers, uint64_t
     if ((uint64_t)first_tower + n_towers > (uint64_t)(P->nq + P->kp)) return fail(KS_EINVAL, "tower range outside the basis");
     if ((rc = set_device(P)) != KS_OK) return rc;
     LimbMap m{d_data, d_data, nullptr, (int)n_towers, 0, 0, (int)first_tower, P->nq, -1};
-    if (inverse) return launch_ntt_inv(P->tables, one_map(m, (int)n_towers), true, (cudaStream_t)stream);
-    return launch_ntt_fwd(P->tables, one_map(m, (int)n_towers), true, (cudaStream_t)stream);
+    if (inverse) return launch_ntt_inv(P->tables, one_map(m, (int)n_towers), true, (cudaStream_t)stream, true);
+    return launch_ntt_fwd(P->tables, one_map(m, (int)n_towers), true, (cudaStream_t)stream, true);
 }
 
 int ks_modup(const ks_params *P, uint32_t level_towers, const uint64_t *d_in, uint64_t *d_ext, ks_stream_t stream)

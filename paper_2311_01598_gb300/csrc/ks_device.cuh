@@ -41,7 +41,8 @@ namespace ks {
 
 // ------------------------------------------------------------------ dependent launches
 // Kernels launched with launch_dep: pdl_start lets the next kernel of the stream
-// begin its own prologue once every block of this one has started; pdl_wait
+// begin its own prologue once every block of this one has started (without it,
+// once every block has ended); pdl_wait
 // holds a block until the stream's previous kernel is complete.  Before pdl_wait
 // a kernel reads only its parameters and the parameter set's tables.  Every
 // path out of a kernel passes pdl_wait, also that of a block with nothing to do:

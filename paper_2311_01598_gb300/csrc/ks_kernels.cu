@@ -10,11 +10,12 @@ namespace ks {
 
 // ------------------------------------------------------------------ NTT passes
 // Forward column pass (stages 0..LA-1).  grid (2^LB/COLS, limbs).  AR: the
-// butterfly form the set's primes allow (ks_device.cuh).
+// butterfly form the set's primes allow (ks_device.cuh).  early: the next kernel
+// may start with this one, else as its blocks end (early_start).
 template <class S, int AR>
-__global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
@@ -55,9 +56,9 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
 // layout; measured faster than storing each thread's consecutive values
 // with strided vector stores).
 template <class S, bool CANON, int AR>
-__global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lz = blockIdx.y + blockIdx.z * gridDim.y;
@@ -229,9 +230,9 @@ int ntt_error_flag(bool clear)
 // Inverse row pass (stages logN-1..LA), first half of the iNTT.  Input below
 // 4q; output below 4q (AR_PM: any 64-bit value, folded by the column pass).
 template <class S, int AR>
-__global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
@@ -263,9 +264,9 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
 // scale (SC: the job's per-entry scale where its map has one, else N^-1);
 // output canonical.
 template <class S, bool SC, int AR>
-__global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + (1 << S::LA) * S::COLS);
@@ -356,10 +357,10 @@ struct Col9 {
 };
 
 template <class S, bool SC, int AR>
-__global__ void __launch_bounds__(Col9::THREADS, 2) k_inv_col9(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(Col9::THREADS, 2) k_inv_col9(Tables T, LimbMaps ms, int early)
 {
     static_assert(S::LA == 9, "nine column stages");
-    pdl_start();
+    if (early) pdl_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     u64 *sm = reinterpret_cast<u64 *>(smem_raw);
     ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + 512 * Col9::COLS);
@@ -443,12 +444,40 @@ static bool any_scale(const LimbMaps &ms)
     return false;
 }
 
+// When the kernel behind an NTT pass may start: with the pass, or as its blocks
+// end.  Inside a key switch always with it, so that its dispatch and prologue
+// overlap the pass.  A transform called alone (ks_ntt) is followed by a pass as
+// wide as itself, whose blocks, dispatched while this pass still holds some SMs
+// more than others, crowd on what is free and keep that placement for their whole
+// run: a loss once the grid is wide enough to crowd, nothing where one wave follows
+// another.  So alone: with the pass up to 2^16 words (where the overlap is worth
+// 0.3 to 0.6 us of 8) and from a wave of blocks on (half a wave for the forward
+// row pass), as its blocks end between.  us, forward / inverse, calls back to back,
+// always with the pass -> this rule (plain launches before dependent ones):
+//   N = 2^13, 16 limbs  7.2 / 13.4 -> 7.0 / 7.8    (11.4 / 12.3)
+//   N = 2^14, 32        19.0 / 21.5 -> 9.9 / 10.5  (16.7 / 16.7)
+//   N = 2^15, 16        19.6 / 22.0 -> 10.2 / 10.8 (17.4 / 16.8)
+//   N = 2^16, 8         19.4 / 21.5 -> 10.0 / 10.6 (15.6 / 16.8)
+//   N = 2^17, 4         23.2 / 23.9 -> 13.7 / 14.2 (19.2 / 22.9)
+//   N = 2^16, 64        40.4 / 44.9 -> 40.4 / 44.9 (53.6 / 65.1)
+// In the chains the rule gained 2.9% on a digit-centric switch and lost 2.5% on
+// batches of small rings, whose other lane keeps the SMs busy.
 template <class S>
-static void fwd_col_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
+static int early_start(const LimbMaps &m, const dim3 &g, unsigned blocks_per_sm, bool alone)
+{
+    constexpr unsigned kSMs = 152;
+    return !alone || ((size_t)m.pre[m.n] << S::LOGN) <= ((size_t)1 << 16) ||
+           (size_t)g.x * g.y * g.z >= (size_t)blocks_per_sm * kSMs;
+}
+
+template <class S>
+static void fwd_col_S(const Tables &T, const LimbMaps &m, bool alone, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col", (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m))))
+    const int early = early_start<S>(m, ga, S::LA == 9 ? 2 : S::MINB_A, alone);
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col",
+                                (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m, early))))
 }
 
 // Persistent grid of the staged row pass: resident CTAs per SM x SMs, at
@@ -481,7 +510,7 @@ static int staged_grid(int items)
 }
 
 template <class S>
-static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st)
+static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, bool alone, cudaStream_t st)
 {
     set_smem_attrs<S>();
     // the bulk copies need 16-byte aligned sources (row blocks of an aligned
@@ -500,39 +529,45 @@ static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, cudaSt
                                                                                          TH, SM, st>>>(T, m))))
         return;
     }
+    const int early = early_start<S>(m, gb, S::MINB_B / 2, alone);
+    constexpr int TH = S::THREADS_B, SM = S::SMEM_BT;
     if (canonical)
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, true, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, true, AR>, gb, TH, SM, T, m, early))))
     else
-        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, false, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
+        KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, false, AR>, gb, TH, SM, T, m, early))))
 }
 
 template <class S>
-static void inv_row_S(const Tables &T, const LimbMaps &m, cudaStream_t st)
+static void inv_row_S(const Tables &T, const LimbMaps &m, bool alone, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
-    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row", (launch_dep(st, k_inv_row<S, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m))))
+    const int early = early_start<S>(m, gb, S::MINB_B, alone);
+    KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row",
+                                (launch_dep(st, k_inv_row<S, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m, early))))
 }
 
 // scaled: multiply by the maps' per-entry scale, or by N^-1 where a map has none.
 template <class S>
-static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
+static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, bool alone, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
     if constexpr (S::LA == 9) {
         const dim3 g9 = limb_grid((1 << S::LB) / Col9::COLS, m.pre[m.n]);
         constexpr int TH = Col9::THREADS, SM = Col9::SMEM;
+        const int early = early_start<S>(m, g9, 2, alone);
         if (scaled)
-            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, true, AR>, g9, TH, SM, T, m))))
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, true, AR>, g9, TH, SM, T, m, early))))
         else
-            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, false, AR>, g9, TH, SM, T, m))))
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, false, AR>, g9, TH, SM, T, m, early))))
     } else {
         constexpr int TH = S::THREADS_A, SM = S::SMEM_A;
+        const int early = early_start<S>(m, ga, S::MINB_A, alone);
         if (scaled)
-            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, TH, SM, T, m))))
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, TH, SM, T, m, early))))
         else
-            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, false, AR>, ga, TH, SM, T, m))))
+            KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, false, AR>, ga, TH, SM, T, m, early))))
     }
 }
 
@@ -569,42 +604,42 @@ void add_map(LimbMaps &ms, const LimbMap &m, int nlimbs)
 int launch_fwd_col(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
-    KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, st);
+    KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, false, st);
     return launch_status("forward column pass launch");
 }
 
 int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st)
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
-    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m, scale_by_ninv || any_scale(m), st);
+    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m, scale_by_ninv || any_scale(m), false, st);
     return launch_status("inverse column pass launch");
 }
 
-int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st)
+int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone)
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     if (T.ntt_cluster) {
         const int rc = launch_ntt_fwd_cluster(T, m, canonical, st);
         if (rc != KS_EUNSUPPORTED) return rc;
     }
-    KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, st);
+    KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, alone, st);
     LimbMaps m2 = m;
     for (int j = 0; j < m2.n; ++j) m2.m[j].src = m2.m[j].dst;
-    KS_DISPATCH_LOGN(T.logN, fwd_row_S, T, m2, canonical, st);
+    KS_DISPATCH_LOGN(T.logN, fwd_row_S, T, m2, canonical, alone, st);
     return launch_status("forward NTT launch");
 }
 
-int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st)
+int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st, bool alone)
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     if (T.ntt_cluster) {
         const int rc = launch_ntt_inv_cluster(T, m, scale_by_ninv || any_scale(m), st);
         if (rc != KS_EUNSUPPORTED) return rc;
     }
-    KS_DISPATCH_LOGN(T.logN, inv_row_S, T, m, st);
+    KS_DISPATCH_LOGN(T.logN, inv_row_S, T, m, alone, st);
     LimbMaps m2 = m;
     for (int j = 0; j < m2.n; ++j) m2.m[j].src = m2.m[j].dst;
-    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m2, scale_by_ninv || any_scale(m), st);
+    KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m2, scale_by_ninv || any_scale(m), alone, st);
     return launch_status("inverse NTT launch");
 }
 

@@ -61,12 +61,13 @@ void add_map(LimbMaps &ms, const LimbMap &m, int nlimbs);
 
 // Forward NTT (column pass src->dst, row pass in place on dst).  Input below
 // 4q.  canonical: output in [0, q); otherwise lazy, at most ModC::flz (every
-// consumer of lazy output reduces it).
-int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st);
+// consumer of lazy output reduces it).  alone: not part of a key switch's chain
+// (when the next kernel may start: early_start, ks_kernels.cu).
+int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone = false);
 // Inverse NTT without the N^-1 factor (row pass src->dst, column pass in
 // place); the column pass multiplies by the per-entry scale when the job's
 // map has one, or by N^-1 when scale_by_ninv; output canonical.  Input below 4q.
-int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st);
+int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st, bool alone = false);
 // One-launch forms over thread-block clusters (ks_ntt_cluster.cu): the same
 // contracts and bit-identical outputs; scaled (inverse): by the maps'
 // per-entry scale, or by N^-1 where a map has none.  They return KS_EUNSUPPORTED, launching

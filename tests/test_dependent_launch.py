@@ -111,3 +111,39 @@ def test_shard_inside_one_digit(logN, nq, dnum, nact):
     for x in range(2):
         got = np.concatenate([ks.to_host(o[x]) for o in outs if o[x].shape[0] > 0])
         assert np.array_equal(got, want[x])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("logN,nq,kp", [(10, 48, 17), (13, 7, 2), (14, 60, 32), (16, 34, 4), (17, 3, 2)])
+def test_transforms_alone(logN, nq, kp):
+    """Transforms called one after the other on the same limbs, below, at and past
+    the sizes where the next kernel may start with a pass (2^16 words; a wave, half
+    a wave of blocks): inverse of forward, and forward three times, against the
+    oracle on the first and the last limb."""
+    need_gpu()
+    ks = built_lib()
+    from oracle import oracle as orc
+    P, C = pair(logN, nq, kp, 1)
+    primes = P.q + P.p
+    nt = len(primes)
+    a = inputs.uniform_towers(primes, C.N, seed=logN)
+    words = 1 << 16 >> logN
+    counts = {1, words, words + 1, nt - 1, nt}
+    for waves in (8 * 152, 16 * 152):  # row blocks of half a wave and of one
+        rows = 4 if logN >= 16 else 8
+        limbs = waves // ((1 << logN - logN // 2) // rows)
+        counts |= {limbs, limbs + 1}
+    for n in sorted(c for c in counts if 1 <= c <= nt):
+        x = ks.to_device(a[:n])
+        for _ in range(2):
+            P.ntt(0, x, inverse=False)
+            P.ntt(0, x, inverse=True)
+        assert np.array_equal(ks.to_host(x), a[:n]), n
+        for _ in range(3):
+            P.ntt(0, x, inverse=False)
+        got = ks.to_host(x)
+        for t in {0, n - 1}:
+            want = a[t]
+            for _ in range(3):
+                want = orc.ntt(want, logN, primes[t], orc.find_psi(primes[t], logN))
+            assert np.array_equal(got[t], want), (n, t)
