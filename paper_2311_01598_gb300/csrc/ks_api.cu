@@ -860,10 +860,6 @@ int run_batch(ks_params *P, uint32_t n, const ks_job *jobs, const ks_schedule &s
     // passes of another.
     const int lanes = std::min<int>(P->batch_lanes, (int)(n / kLaneJobs));
     if (lanes > 1) {
-        // jobs of one key on one lane, where the combine kernels run them side by
-        // side (64 jobs of 16 keys: 5004 -> 4968 us)
-        if (sc.order == 0)
-            std::stable_sort(idx.begin(), idx.end(), [&](uint32_t a, uint32_t b) { return jobs[a].key < jobs[b].key; });
         std::vector<ks_job> sorted(n);
         for (uint32_t i = 0; i < n; ++i) sorted[i] = jobs[idx[i]];
         if ((rc = lane_streams(P)) != KS_OK) return rc;
