@@ -228,20 +228,28 @@ def check(rc: int) -> None:
         raise KSError(rc, lib().ks_last_error().decode())
 
 
-_torch_cuda = None
+_current_stream = None
+
+
+def _torch_stream():
+    """A function returning torch's current stream as its raw handle: building
+    a torch Stream object for it costs 3 us a call, a fifth of a small transform,
+    so torch's own raw lookups are used where this torch has them."""
+    import torch
+    torch.cuda.current_stream()  # initialises CUDA in torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
 def _stream_handle(stream) -> ctypes.c_void_p:
     if stream is None:
-        # torch's current stream as its raw handle: building a torch Stream
-        # object for it costs 3 us a call, a fifth of a small transform
-        global _torch_cuda
-        if _torch_cuda is None:
-            import torch
-            torch.cuda.current_stream()  # initialises CUDA in torch, as before
-            _torch_cuda = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
-        raw, device = _torch_cuda
-        return ctypes.c_void_p(raw(device()))
+        global _current_stream
+        if _current_stream is None:
+            _current_stream = _torch_stream()
+        return ctypes.c_void_p(_current_stream())
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
