@@ -509,15 +509,17 @@ size_t oc_scratch_words(const Tables &T, int nact)
 // Whole-basis variant: tmp holds D [nd][nact+K] then v [2][nact].
 // The order of its combine kernels' blocks:
 //   COMB_PLAIN   job by job, tower by tower; grid (N/(256V), rows);
-//   COMB_SHARED  full keys, and some jobs share one (a busy evaluator has more
+//   COMB_SHARED  full keys, some jobs share one (a busy evaluator has more
 //                ciphertexts than keys; half a compressed key is regenerated, and
-//                6 jobs of 3 such keys at N = 2^14 lost 2 us of 121 this way): tower by tower, block of coefficients by block of
-//                coefficients, the jobs next to each other, so that a key's
-//                words are in L2 for all but the first of its jobs; grid
-//                (rows * N/(256V)), oj by falling level with oj.pre[t] the
-//                (tower, job) pairs below tower t.  64 jobs of 16 keys: Q combine
-//                855 -> 752 us, P combine 398 -> 380; without shared keys the
-//                plain order is the faster one (16 jobs: 2117 us a step, 2126);
+//                6 jobs of 3 such keys at N = 2^14 lost 2 us of 121 this way), and
+//                the launch reads more than L2 holds (kSharedWords): tower by
+//                tower, block of coefficients by block of coefficients, the jobs
+//                next to each other, so that a key's words are in L2 for all but
+//                the first of its jobs; grid (rows * N/(256V)), oj by falling
+//                level with oj.pre[t] the (tower, job) pairs below tower t.  64
+//                jobs of 16 keys: Q combine 855 -> 752 us, P combine 398 -> 380;
+//                without shared keys the plain order is the faster one (16 jobs:
+//                2117 us a step, 2126);
 //   COMB_GAL     hoisted rotations, jobs of one level that share D and d and read
 //                them through their own automorphism: the jobs of a tower next
 //                to each other, so that its rows of D come from L2 for all but
@@ -628,10 +630,30 @@ __global__ void __launch_bounds__(256, 4) k_oc_comb_qw(Tables T, OcJobs oj)
     stv<V>(J.out1 + (size_t)t * N + n, o1);
 }
 
+// Digit and key words of a launch group from which COMB_SHARED is taken: 192 MB,
+// half as much again as L2.  Below, the plain order finds the keys in L2 as well
+// and the shared one only costs its index arithmetic and uneven blocks.  A whole
+// batch, us, plain / shared order:
+//   MB a launch  jobs, keys                         plain   shared
+//    75          2, 1  N = 2^16, levels 4 and 11     145.4   148.3
+//    77          7, 3  N = 2^14, levels 5 to 10      126.9   132.5
+//   113          7, 3  N = 2^14, level 10            155.9   157.0
+//   129          16, 4 (two lanes), the same         270.1   270.9
+//   192          3, 1  N = 2^16, levels 4 to 18      252.2   253.5
+//   258          32, 8 (two lanes) N = 2^14          519.8   512.3
+//   264          7, 3  N = 2^15, level 12            298.0   292.5
+//   302          2, 1  N = 2^16, level 24            318.8   313.2
+//  1057          7, 6  the same (one pair)           975.8   972.1
+// One pair among 16 jobs of two lanes makes no difference (2125 us, both).
+constexpr size_t kSharedWords = (size_t)24 << 20;
+
 // When two jobs share a key: the jobs by falling level and the towers' prefix
 // counts, for COMB_SHARED.
-static bool oc_shared_keys(OcJobs &oj)
+static bool oc_shared_keys(const Tables &T, OcJobs &oj)
 {
+    size_t words = 0;
+    for (int i = 0; i < oj.n; ++i) words += (size_t)oj.job[i].nd * (oj.job[i].nact + T.kp) * 3 << T.logN;
+    if (words <= kSharedWords) return false;
     const u64 *keys[kMaxBatch];
     for (int i = 0; i < oj.n; ++i) keys[i] = oj.job[i].key.evk;
     std::sort(keys, keys + oj.n);
@@ -701,7 +723,7 @@ static int launch_oc_whole(const Tables &T, int n, const OcJob *jobs, bool share
     KeyGroups kg;
     const bool grouped = share_keys && key_groups(oj, kg);
     const int q_rows = oj.pre[n];  // before oc_shared_keys counts by tower
-    const bool shared = !grouped && !ck && oc_shared_keys(oj);
+    const bool shared = !grouped && !ck && oc_shared_keys(T, oj);
     auto combine = [&](bool p_section) {
         if (grouped)
             comb_grouped(T, oj, kg, p_section, st);
