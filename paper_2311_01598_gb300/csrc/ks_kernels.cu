@@ -437,6 +437,8 @@ static dim3 limb_grid(unsigned gx, int limbs)
     return dim3(gx, gy, (unsigned)((limbs + gy - 1) / gy));
 }
 
+static size_t grid_blocks(const dim3 &g) { return (size_t)g.x * g.y * g.z; }
+
 static bool any_scale(const LimbMaps &ms)
 {
     for (int j = 0; j < ms.n; ++j)
@@ -444,38 +446,12 @@ static bool any_scale(const LimbMaps &ms)
     return false;
 }
 
-// When the kernel behind an NTT pass may start: with the pass, or as its blocks
-// end.  Inside a key switch always with it, so that its dispatch and prologue
-// overlap the pass.  A transform called alone (ks_ntt) is followed by a pass as
-// wide as itself, whose blocks, dispatched while this pass still holds some SMs
-// more than others, crowd on what is free and keep that placement for their whole
-// run: a loss once the grid is wide enough to crowd, nothing where one wave follows
-// another.  So alone: with the pass up to 2^16 words (where the overlap is worth
-// 0.3 to 0.6 us of 8) and from a wave of blocks on (half a wave for the forward
-// row pass), as its blocks end between.  us, forward / inverse, calls back to back,
-// always with the pass -> this rule (plain launches before dependent ones):
-//   N = 2^13, 16 limbs  7.2 / 13.4 -> 7.0 / 7.8    (11.4 / 12.3)
-//   N = 2^14, 32        19.0 / 21.5 -> 9.9 / 10.5  (16.7 / 16.7)
-//   N = 2^15, 16        19.6 / 22.0 -> 10.2 / 10.8 (17.4 / 16.8)
-//   N = 2^16, 8         19.4 / 21.5 -> 10.0 / 10.6 (15.6 / 16.8)
-//   N = 2^17, 4         23.2 / 23.9 -> 13.7 / 14.2 (19.2 / 22.9)
-//   N = 2^16, 64        40.4 / 44.9 -> 40.4 / 44.9 (53.6 / 65.1)
-// In the chains the rule gained 2.9% on a digit-centric switch and lost 2.5% on
-// batches of small rings, whose other lane keeps the SMs busy.
-template <class S>
-static int early_start(const LimbMaps &m, const dim3 &g, unsigned blocks_per_sm, bool alone)
-{
-    constexpr unsigned kSMs = 152;
-    return !alone || ((size_t)m.pre[m.n] << S::LOGN) <= ((size_t)1 << 16) ||
-           (size_t)g.x * g.y * g.z >= (size_t)blocks_per_sm * kSMs;
-}
-
 template <class S>
 static void fwd_col_S(const Tables &T, const LimbMaps &m, bool alone, cudaStream_t st)
 {
     set_smem_attrs<S>();
     const dim3 ga = limb_grid((1 << S::LB) / S::COLS, m.pre[m.n]);
-    const int early = early_start<S>(m, ga, S::LA == 9 ? 2 : S::MINB_A, alone);
+    const int early = early_start(T, m.pre[m.n], grid_blocks(ga), S::LA == 9 ? 2 : S::MINB_A, alone);
     KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_col",
                                 (launch_dep(st, k_fwd_col<S, AR>, ga, S::THREADS_A, S::SMEM_A, T, m, early))))
 }
@@ -529,7 +505,7 @@ static void fwd_row_S(const Tables &T, const LimbMaps &m, bool canonical, bool a
                                                                                          TH, SM, st>>>(T, m))))
         return;
     }
-    const int early = early_start<S>(m, gb, S::MINB_B / 2, alone);
+    const int early = early_start(T, m.pre[m.n], grid_blocks(gb), S::MINB_B / 2, alone);
     constexpr int TH = S::THREADS_B, SM = S::SMEM_BT;
     if (canonical)
         KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_fwd_row", (launch_dep(st, k_fwd_row<S, true, AR>, gb, TH, SM, T, m, early))))
@@ -542,7 +518,7 @@ static void inv_row_S(const Tables &T, const LimbMaps &m, bool alone, cudaStream
 {
     set_smem_attrs<S>();
     const dim3 gb = limb_grid((1 << S::LA) / S::ROWS, m.pre[m.n]);
-    const int early = early_start<S>(m, gb, S::MINB_B, alone);
+    const int early = early_start(T, m.pre[m.n], grid_blocks(gb), S::MINB_B, alone);
     KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_row",
                                 (launch_dep(st, k_inv_row<S, AR>, gb, S::THREADS_B, S::SMEM_BT, T, m, early))))
 }
@@ -556,14 +532,14 @@ static void inv_col_S(const Tables &T, const LimbMaps &m, bool scaled, bool alon
     if constexpr (S::LA == 9) {
         const dim3 g9 = limb_grid((1 << S::LB) / Col9::COLS, m.pre[m.n]);
         constexpr int TH = Col9::THREADS, SM = Col9::SMEM;
-        const int early = early_start<S>(m, g9, 2, alone);
+        const int early = early_start(T, m.pre[m.n], grid_blocks(g9), 2, alone);
         if (scaled)
             KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, true, AR>, g9, TH, SM, T, m, early))))
         else
             KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col9<S, false, AR>, g9, TH, SM, T, m, early))))
     } else {
         constexpr int TH = S::THREADS_A, SM = S::SMEM_A;
-        const int early = early_start<S>(m, ga, S::MINB_A, alone);
+        const int early = early_start(T, m.pre[m.n], grid_blocks(ga), S::MINB_A, alone);
         if (scaled)
             KS_DISPATCH_AR(T, KS_LAUNCH(st, "ntt_inv_col", (launch_dep(st, k_inv_col<S, true, AR>, ga, TH, SM, T, m, early))))
         else
@@ -619,7 +595,7 @@ int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStrea
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     if (T.ntt_cluster) {
-        const int rc = launch_ntt_fwd_cluster(T, m, canonical, st);
+        const int rc = launch_ntt_fwd_cluster(T, m, canonical, st, alone);
         if (rc != KS_EUNSUPPORTED) return rc;
     }
     KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, alone, st);
@@ -633,7 +609,7 @@ int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaS
 {
     if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
     if (T.ntt_cluster) {
-        const int rc = launch_ntt_inv_cluster(T, m, scale_by_ninv || any_scale(m), st);
+        const int rc = launch_ntt_inv_cluster(T, m, scale_by_ninv || any_scale(m), st, alone);
         if (rc != KS_EUNSUPPORTED) return rc;
     }
     KS_DISPATCH_LOGN(T.logN, inv_row_S, T, m, alone, st);

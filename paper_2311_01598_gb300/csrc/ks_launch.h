@@ -59,10 +59,36 @@ __host__ __device__ inline int find_slot(const int *pre, int n, int x)
 LimbMaps one_map(const LimbMap &m, int nlimbs);
 void add_map(LimbMaps &ms, const LimbMap &m, int nlimbs);
 
+// When the kernel behind an NTT pass may start: with the pass, or as its blocks
+// end.  Inside a key switch always with it, so that its dispatch and prologue
+// overlap the pass.  A transform called alone (ks_ntt) is followed by a pass as
+// wide as itself, whose blocks, dispatched while this pass still holds some SMs
+// more than others, crowd on what is free and keep that placement for their whole
+// run: a loss once the grid is wide enough to crowd, nothing where one wave follows
+// another.  So alone: with the pass up to 2^16 words (where the overlap is worth
+// 0.3 to 0.6 us of 8) and from a wave of blocks on (half a wave for the forward
+// row pass), as its blocks end between.  us, forward / inverse, calls back to back,
+// always with the pass -> this rule (plain launches before dependent ones):
+//   N = 2^13, 16 limbs  7.2 / 13.4 -> 7.0 / 7.8    (11.4 / 12.3)
+//   N = 2^14, 32        19.0 / 21.5 -> 9.9 / 10.5  (16.7 / 16.7)
+//   N = 2^15, 16        19.6 / 22.0 -> 10.2 / 10.8 (17.4 / 16.8)
+//   N = 2^16, 8         19.4 / 21.5 -> 10.0 / 10.6 (15.6 / 16.8)
+//   N = 2^17, 4         23.2 / 23.9 -> 13.7 / 14.2 (19.2 / 22.9)
+//   N = 2^16, 64        40.4 / 44.9 -> 40.4 / 44.9 (53.6 / 65.1)
+// The one-launch cluster form likewise: N = 2^14, 64 limbs 20.2 / 22.2 -> 14.3 / 15.4
+// (20.9 / 21.2), N = 2^16, 12 limbs 21.4 / 25.0 -> 14.1 / 15.9 (19.2 / 21.1).
+// In the chains the rule gained 2.9% on a digit-centric switch and lost 2.5% on
+// batches of small rings, whose other lane keeps the SMs busy.
+inline int early_start(const Tables &T, int limbs, size_t blocks, int blocks_per_sm, bool alone)
+{
+    constexpr int kSMs = 152;
+    return !alone || ((size_t)limbs << T.logN) <= ((size_t)1 << 16) || blocks >= (size_t)blocks_per_sm * kSMs;
+}
+
 // Forward NTT (column pass src->dst, row pass in place on dst).  Input below
 // 4q.  canonical: output in [0, q); otherwise lazy, at most ModC::flz (every
 // consumer of lazy output reduces it).  alone: not part of a key switch's chain
-// (when the next kernel may start: early_start, ks_kernels.cu).
+// (early_start).
 int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone = false);
 // Inverse NTT without the N^-1 factor (row pass src->dst, column pass in
 // place); the column pass multiplies by the per-entry scale when the job's
@@ -74,8 +100,8 @@ int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaS
 // nothing, when the ring degree's shape or the device has no cluster form;
 // launch_ntt_fwd/inv use them when T.ntt_cluster is set and fall back.
 bool ntt_cluster_shape(int logN);
-int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st);
-int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st);
+int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone);
+int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st, bool alone);
 // Single passes.
 int launch_fwd_col(const Tables &T, const LimbMaps &m, cudaStream_t st);
 int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st);

@@ -23,11 +23,12 @@ namespace {
 
 // Forward NTT (input below 4q; output canonical with CANON, else lazy, at most flz).
 // grid (C, limbs), cluster (C, 1, 1): every CTA of a cluster has the same
-// limb, so the early exits below are uniform over the cluster.
+// limb, so the early exits below are uniform over the cluster.  early: the next
+// kernel may start with this one, else as its blocks end (early_start).
 template <class S, int MUL, bool CANON, int AR>
-__global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_cl(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_cl(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     typedef Cl<S, MUL> G_;
     constexpr int COLS = G_::COLS, ROWS = G_::ROWS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -94,9 +95,9 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
 // Inverse NTT (input below 4q), then the scale (SC: the job's per-entry scale
 // where its map has one, else N^-1); output canonical.
 template <class S, int MUL, bool SC, int AR>
-__global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_cl(Tables T, LimbMaps ms)
+__global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_cl(Tables T, LimbMaps ms, int early)
 {
-    pdl_start();
+    if (early) pdl_start();
     typedef Cl<S, MUL> G_;
     constexpr int COLS = G_::COLS, ROWS = G_::ROWS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -186,7 +187,7 @@ struct ClKernels {
 
 template <class KERN>
 static cudaError_t launch_cluster(KERN kern, int C, int threads, int smem, int limbs, const Tables &T,
-                                  const LimbMaps &m, cudaStream_t st)
+                                  const LimbMaps &m, int early, cudaStream_t st)
 {
     const unsigned gy = (unsigned)std::min(limbs, 32768);
     cudaLaunchConfig_t cfg = {};
@@ -203,13 +204,13 @@ static cudaError_t launch_cluster(KERN kern, int C, int threads, int smem, int l
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, T, m);
+    return cudaLaunchKernelEx(&cfg, kern, T, m, early);
 }
 
 // Returns KS_EUNSUPPORTED (nothing launched) when the shape or the device
 // cannot run the cluster form.
 template <class S, int MUL>
-static int fwd_cl_SM(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st)
+static int fwd_cl_SM(const Tables &T, const LimbMaps &m, bool canonical, bool alone, cudaStream_t st)
 {
     typedef Cl<S, MUL> G;
     if constexpr (!G::OK) {
@@ -219,19 +220,20 @@ static int fwd_cl_SM(const Tables &T, const LimbMaps &m, bool canonical, cudaStr
         cudaError_t e;
         const int limbs = m.pre[m.n];
         constexpr int C = G::C, TH = G::THREADS, SM = G::SMEM;
+        const int early = early_start(T, limbs, (size_t)limbs * C, G::MINB, alone);
         if (canonical)
             KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_cl", (e = launch_cluster(k_fwd_cl<S, MUL, true, AR>, C, TH, SM, limbs,
-                                                                               T, m, st))))
+                                                                               T, m, early, st))))
         else
             KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_fwd_cl", (e = launch_cluster(k_fwd_cl<S, MUL, false, AR>, C, TH, SM, limbs,
-                                                                               T, m, st))))
+                                                                               T, m, early, st))))
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("cluster NTT launch: ") + cudaGetErrorString(e));
         return KS_OK;
     }
 }
 
 template <class S, int MUL>
-static int inv_cl_SM(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
+static int inv_cl_SM(const Tables &T, const LimbMaps &m, bool scaled, bool alone, cudaStream_t st)
 {
     typedef Cl<S, MUL> G;
     if constexpr (!G::OK) {
@@ -241,12 +243,13 @@ static int inv_cl_SM(const Tables &T, const LimbMaps &m, bool scaled, cudaStream
         cudaError_t e;
         const int limbs = m.pre[m.n];
         constexpr int C = G::C, TH = G::THREADS, SM = G::SMEM;
+        const int early = early_start(T, limbs, (size_t)limbs * C, G::MINB, alone);
         if (scaled)
             KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_inv_cl", (e = launch_cluster(k_inv_cl<S, MUL, true, AR>, C, TH, SM, limbs,
-                                                                               T, m, st))))
+                                                                               T, m, early, st))))
         else
             KS_DISPATCH_AR2(T, KS_LAUNCH(st, "ntt_inv_cl", (e = launch_cluster(k_inv_cl<S, MUL, false, AR>, C, TH, SM, limbs,
-                                                                               T, m, st))))
+                                                                               T, m, early, st))))
         if (e != cudaSuccess) return fail(KS_ECUDA, std::string("cluster NTT launch: ") + cudaGetErrorString(e));
         return KS_OK;
     }
@@ -254,14 +257,14 @@ static int inv_cl_SM(const Tables &T, const LimbMaps &m, bool scaled, cudaStream
 
 // T.ntt_cluster: 1 = CTAs of the two-pass size, 2 = CTAs twice as wide
 template <class S>
-static int fwd_cl_S(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st)
+static int fwd_cl_S(const Tables &T, const LimbMaps &m, bool canonical, bool alone, cudaStream_t st)
 {
-    return T.ntt_cluster == 2 ? fwd_cl_SM<S, 2>(T, m, canonical, st) : fwd_cl_SM<S, 1>(T, m, canonical, st);
+    return T.ntt_cluster == 2 ? fwd_cl_SM<S, 2>(T, m, canonical, alone, st) : fwd_cl_SM<S, 1>(T, m, canonical, alone, st);
 }
 template <class S>
-static int inv_cl_S(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
+static int inv_cl_S(const Tables &T, const LimbMaps &m, bool scaled, bool alone, cudaStream_t st)
 {
-    return T.ntt_cluster == 2 ? inv_cl_SM<S, 2>(T, m, scaled, st) : inv_cl_SM<S, 1>(T, m, scaled, st);
+    return T.ntt_cluster == 2 ? inv_cl_SM<S, 2>(T, m, scaled, alone, st) : inv_cl_SM<S, 1>(T, m, scaled, alone, st);
 }
 
 #define KS_CL_DISPATCH(logN, FN, ...)                         \
@@ -294,14 +297,14 @@ bool ntt_cluster_shape(int logN)
     }
 }
 
-int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st)
+int launch_ntt_fwd_cluster(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone)
 {
-    KS_CL_DISPATCH(T.logN, fwd_cl_S, T, m, canonical, st);
+    KS_CL_DISPATCH(T.logN, fwd_cl_S, T, m, canonical, alone, st);
 }
 
-int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st)
+int launch_ntt_inv_cluster(const Tables &T, const LimbMaps &m, bool scaled, cudaStream_t st, bool alone)
 {
-    KS_CL_DISPATCH(T.logN, inv_cl_S, T, m, scaled, st);
+    KS_CL_DISPATCH(T.logN, inv_cl_S, T, m, scaled, alone, st);
 }
 
 }  // namespace ks

@@ -147,3 +147,30 @@ def test_transforms_alone(logN, nq, kp):
             for _ in range(3):
                 want = orc.ntt(want, logN, primes[t], orc.find_psi(primes[t], logN))
             assert np.array_equal(got[t], want), (n, t)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cluster", [1, 2])
+@pytest.mark.parametrize("logN,nq,kp", [(10, 48, 17), (14, 60, 32), (16, 40, 4)])
+def test_cluster_transforms_alone(logN, nq, kp, cluster):
+    """The same for the one-launch cluster form, below and past 2^16 words and a
+    wave of blocks (16 CTAs a limb at 2^16, 4 or 8 at 2^14, 1 or 2 at 2^10)."""
+    need_gpu()
+    ks = built_lib()
+    from oracle import oracle as orc
+    P, C = pair(logN, nq, kp, 1)
+    P.set_ntt_cluster(cluster)
+    primes = P.q + P.p
+    a = inputs.uniform_towers(primes, C.N, seed=logN)
+    for n in sorted({1, 2, min(64, len(primes)), 19, 38, len(primes)}):
+        x = ks.to_device(a[:n])
+        for _ in range(2):
+            P.ntt(0, x, inverse=False)
+            P.ntt(0, x, inverse=True)
+        assert np.array_equal(ks.to_host(x), a[:n]), n
+        for _ in range(2):
+            P.ntt(0, x, inverse=False)
+        got = ks.to_host(x)
+        for t in {0, n - 1}:
+            psi = orc.find_psi(primes[t], logN)
+            assert np.array_equal(got[t], orc.ntt(orc.ntt(a[t], logN, primes[t], psi), logN, primes[t], psi)), (n, t)
