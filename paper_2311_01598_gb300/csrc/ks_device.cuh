@@ -48,7 +48,10 @@ namespace ks {
 // path out of a kernel passes pdl_wait, also that of a block with nothing to do:
 // a launch of such blocks alone (one digit's own towers, all of them bypassed)
 // would else be complete before its predecessor, and the kernel after it start
-// on data still being written.
+// on data still being written.  The one exception are the transforms' blocks of
+// bypassed limbs (L.skip), which leave at once: their launchers make sure that a
+// limb is transformed (any_limb).  Waiting, they held places that the transformed
+// limbs' blocks of small switches want (N = 2^15, 4 + 2 towers, MP: 69.6 -> 75.6 us).
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

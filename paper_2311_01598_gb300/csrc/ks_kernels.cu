@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_fwd_col(Tables T, L
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
     if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModR<AR> md = mod_fwd<AR>(T.modc[L.tf]);
     const ulonglong2 *twt = T.tw + ((size_t)L.tf << S::LOGN);
     pdl_wait();
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_fwd_row(Tables T, L
     // recently, so the first blocks find their rows in L2
     const int lg = ms.pre[ms.n] - 1 - lz;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_fwd<AR>(mc);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(S::THREADS_B, S::MINB_B) k_inv_row(Tables T, L
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
     if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModR<AR> md = mod_inv<AR>(T.modc[L.tf]);
     const int rr = threadIdx.x / S::TB, tau = threadIdx.x % S::TB;
     const int h = blockIdx.x * S::ROWS + rr;
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(S::THREADS_A, S::MINB_A) k_inv_col(Tables T, L
     // limbs in reverse order: the row pass wrote the last ones most recently
     const int lg = ms.pre[ms.n] - 1 - lz;
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const ulonglong2 *twt = T.itw + ((size_t)L.tf << S::LOGN);
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(Col9::THREADS, 2) k_inv_col9(Tables T, LimbMap
     if (lz >= ms.pre[ms.n]) return pdl_wait();
     // limbs in reverse order: the row pass wrote the last ones most recently
     const LimbRef L = limb_ref(ms, ms.pre[ms.n] - 1 - lz, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     tws[threadIdx.x] = T.itw[((size_t)L.tf << S::LOGN) + threadIdx.x];
@@ -438,6 +438,23 @@ static dim3 limb_grid(unsigned gx, int limbs)
 }
 
 static size_t grid_blocks(const dim3 &g) { return (size_t)g.x * g.y * g.z; }
+
+// Whether the maps have a limb to transform.  Blocks of bypassed limbs leave
+// without waiting for the stream's previous kernel (pdl_wait), so a set of
+// bypassed limbs alone (a tower shard inside the active digit) is not launched.
+static bool any_limb(const Tables &T, const LimbMaps &ms)
+{
+    for (int j = 0; j < ms.n; ++j) {
+        const LimbMap &M = ms.m[j];
+        const int limbs = ms.pre[j + 1] - ms.pre[j];
+        if (M.skip_base < 0 && limbs > 0) return true;
+        for (int l = 0; l < limbs; ++l) {
+            const int t = M.toff + l % M.per;
+            if (t >= M.nact || t / T.alpha != l / M.per + M.skip_base) return true;
+        }
+    }
+    return false;
+}
 
 static bool any_scale(const LimbMaps &ms)
 {
@@ -579,21 +596,21 @@ void add_map(LimbMaps &ms, const LimbMap &m, int nlimbs)
 
 int launch_fwd_col(const Tables &T, const LimbMaps &m, cudaStream_t st)
 {
-    if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
+    if (!any_limb(T, m)) return KS_OK;
     KS_DISPATCH_LOGN(T.logN, fwd_col_S, T, m, false, st);
     return launch_status("forward column pass launch");
 }
 
 int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st)
 {
-    if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
+    if (!any_limb(T, m)) return KS_OK;
     KS_DISPATCH_LOGN(T.logN, inv_col_S, T, m, scale_by_ninv || any_scale(m), false, st);
     return launch_status("inverse column pass launch");
 }
 
 int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStream_t st, bool alone)
 {
-    if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
+    if (!any_limb(T, m)) return KS_OK;
     if (T.ntt_cluster) {
         const int rc = launch_ntt_fwd_cluster(T, m, canonical, st, alone);
         if (rc != KS_EUNSUPPORTED) return rc;
@@ -607,7 +624,7 @@ int launch_ntt_fwd(const Tables &T, const LimbMaps &m, bool canonical, cudaStrea
 
 int launch_ntt_inv(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaStream_t st, bool alone)
 {
-    if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
+    if (!any_limb(T, m)) return KS_OK;
     if (T.ntt_cluster) {
         const int rc = launch_ntt_inv_cluster(T, m, scale_by_ninv || any_scale(m), st, alone);
         if (rc != KS_EUNSUPPORTED) return rc;
@@ -965,7 +982,7 @@ __global__ void k_scale(Tables T, LimbMaps ms, const ulonglong2 *fac)
 
 int launch_scale(const Tables &T, const LimbMaps &m, const ulonglong2 *factors_full, cudaStream_t st)
 {
-    if (m.n == 0 || m.pre[m.n] == 0) return KS_OK;
+    if (!any_limb(T, m)) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
     KS_LAUNCH(st, "scale", launch_dep(st, k_scale, limb_grid((unsigned)(N / 256), m.pre[m.n]), 256, 0, T, m, factors_full));
     return launch_status("scale launch");

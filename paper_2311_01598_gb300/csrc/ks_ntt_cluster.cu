@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_fwd_c
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
     if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_fwd<AR>(mc);
     const int r = cluster_rank();
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(Cl<S, MUL>::THREADS, Cl<S, MUL>::MINB) k_inv_c
     const int lg = blockIdx.y + blockIdx.z * gridDim.y;
     if (lg >= ms.pre[ms.n]) return pdl_wait();
     const LimbRef L = limb_ref(ms, lg, T.nq, T.alpha, S::LOGN);
-    if (L.skip) return pdl_wait();
+    if (L.skip) return;
     const ModC &mc = T.modc[L.tf];
     const ModR<AR> md = mod_inv<AR>(mc);
     const int r = cluster_rank();
