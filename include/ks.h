@@ -315,9 +315,9 @@ typedef struct {
                             full keys, else run as 2)                          */
     int32_t chunk;       /* KS_OC: jobs per batched launch group, 1..64           */
     int32_t order;       /* 0 = jobs in the given order, 1 = grouped by level
-                            (descending), 2 = grouped by key (KS_OC: jobs of a
-                            launch sharing a key also share each read of its
-                            limbs in the combine kernels)                        */
+                            (descending), 2 = grouped by key (KS_OC, one lane:
+                            jobs of a launch sharing a key also share each read
+                            of its limbs in the combine kernels)                 */
     int32_t ntt;         /* NTT form: 0 = two launches (column pass, row pass),
                             1 = one cluster launch per NTT (KS_OPT_NTT_CLUSTER),
                             2 = the same with CTAs twice as wide; -1 = the

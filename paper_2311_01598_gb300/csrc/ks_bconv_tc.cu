@@ -177,13 +177,12 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t phase)
     return done != 0;
 }
 
-// One unit of work: a tile of 128 coefficients for one block of <= 16
-// targets of one (job, digit) (ModUp) or (job, polynomial) (ModDown).
+// One unit of work: a tile of 128 coefficients for one block of at most 32
+// targets (16 with two A tiles) of one (job, digit) (ModUp) or (job, polynomial) (ModDown).
 struct TcItem {
     const u64 *src;     // source tower 0 at the tile's first coefficient; tower i at + i*N
     int nsrc;           // source towers (<= 36)
     int G;              // targets (0: nothing to do)
-    int key;            // (job block, target block): the B slabs and targets change with it
     int sbase;          // slab index base (ModUp: of the digit at this level)
     int t_first, ov_at, ov, nact, t_base;  // target numbering (ModUp)
     u64 *dst0;          // output base: target t at dst0 + (t - t_base)*N
@@ -196,7 +195,6 @@ __device__ __forceinline__ TcItem tc_item(const Tables &T, const BUpJobs &bu, co
     const size_t N = (size_t)1 << T.logN;
     const int xt = item % XT, r = item / XT, tb = r % TBN, z = r / TBN;
     TcItem it;
-    it.key = r;
     if (MODE == 0) {
         const int jb = find_slot(bu.zpre, bu.n, z);
         const BUpJob &J = bu.job[jb];
@@ -650,25 +648,23 @@ static int launch_tc_for(const Tables &T, const BUpJobs &bu, const BDnJobs &bd, 
                      : launch_tc<MODE, 1, 1, 8, false>(T, bu, bd, span, slabs, st, name);
 }
 
-int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, const int *, cudaStream_t st)
+int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, cudaStream_t st)
 {
     const int span = bup_span(T, b);
     if (span <= 0) return KS_OK;
     BDnJobs none;
     none.n = 0;
-    Tables Tt = T;
-    Tt.up_tc = slabs;
-    return launch_tc_for<0>(Tt, b, none, T.alpha, span, slabs, st, "bconv_up");
+    return launch_tc_for<0>(T, b, none, T.alpha, span, T.up_tc, st, "bconv_up");
 }
 
-int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, const uint4 *slabs, cudaStream_t st)
+int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, cudaStream_t st)
 {
     int span = 0;
     for (int i = 0; i < b.n; ++i) span = std::max(span, b.job[i].nact);
     if (span <= 0) return KS_OK;
     BUpJobs none;
     none.n = 0;
-    return launch_tc_for<1>(T, none, b, T.kp, span, slabs, st, "bconv_down");
+    return launch_tc_for<1>(T, none, b, T.kp, span, T.dn_tc, st, "bconv_down");
 }
 
 int tc_error_flag(bool clear)

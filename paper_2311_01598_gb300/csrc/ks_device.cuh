@@ -293,7 +293,7 @@ __device__ __forceinline__ u64 redc(U128 T, u64 q, u64 mont)
     u64 m = T.lo * mont;
     return T.hi + __umul64hi(m, q) + (T.lo != 0 ? 1 : 0);
 }
-// Canonical key product of the a half from its 128-bit sum (see key_a).
+// Canonical key product of the a half from its 128-bit sum (see key_macv).
 template <bool CK>
 __device__ __forceinline__ u64 key_a_finish(const KeyView &K, U128 sa, const ModC &mc, const ulonglong2 *fold, int t)
 {
@@ -356,24 +356,6 @@ __device__ __forceinline__ void key_a_words(u64 seed, int j, int t, size_t n, in
         st += 64 * kGamma;
     }
 }
-// Key words of digit j, full tower t, slot n.  Full keys hold both halves
-// times the tower's fold factor and 2^64; a compressed key's a-word is
-// canonical, so its sum of products is multiplied by that factor once per
-// output (key_a_finish).
-// CK: the launch may contain compressed keys (otherwise every key is full
-// and the regeneration code is left out of the kernel).
-template <bool CK>
-__device__ __forceinline__ u64 key_b(const KeyView &K, int j, int t, size_t n, int nfull, int logN)
-{
-    return K.evk[(((size_t)((CK && K.comp) ? j : 2 * j) * nfull + t) << logN) + n];
-}
-template <bool CK>
-__device__ __forceinline__ u64 key_a(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 r)
-{
-    if (CK && K.comp) return key_a_word(K.a_seed, j, t, n, logN, nfull, r);
-    return K.evk[(((size_t)(2 * j + 1) * nfull + t) << logN) + n];
-}
-
 // V consecutive words a thread (V = 2: 16-byte loads and stores; limb bases and
 // even indices keep them aligned).
 template <int V>
@@ -403,7 +385,11 @@ __device__ __forceinline__ void stv(u64 *p, const u64 (&v)[V])
     }
 }
 
-// key product of V coefficients: x * b_j and x * a_j added into sb, sa
+// key product of V coefficients: x * b_j and x * a_j added into sb, sa.  Full keys
+// hold both halves times the tower's fold factor and 2^64; a compressed key's
+// a-word is canonical, so its sum of products is multiplied by that factor once
+// per output (key_a_finish).  CK: the launch may contain compressed keys
+// (otherwise every key is full and the regeneration code is left out).
 template <bool CK, int V>
 __device__ __forceinline__ void key_macv(const KeyView &K, int j, int t, size_t n, int nfull, int logN, u64 q,
                                          const u64 (&x)[V], U128 (&sb)[V], U128 (&sa)[V])

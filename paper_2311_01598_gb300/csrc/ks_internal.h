@@ -54,7 +54,7 @@ struct ModC {
     u64 one_sh;  // floor(2^64 / q): Shoup companion of 1
     u64 r28, r28_sh;  // 2^28 mod q and its Shoup companion
     u64 r56, r56_sh;  // 2^56 mod q and its Shoup companion
-    u64 ninv, ninv_sh;  // N^-1 mod q and its Shoup companion
+    u64 ninv, ninv_sh;  // N^-1 mod q as a pair of the set's form (Shoup, or AR_PM)
     u64 r2;             // 2^128 mod q (into Montgomery form)
     u64 flz;            // multiple of q no forward NTT output (lazy) exceeds; flz + q < 2^64
     // q = 2^b - c just below a power of two (arith AR_PM, ks_device.cuh)
@@ -186,7 +186,13 @@ namespace ks {
 //   12, 2, 6    44.8/44.5  170/163       66.4/66.9  306/317        85.1/93.6  595/642        108/114    1178/1299
 //   24, 8, 3    52.5/57.3                74.7/80.4                 93.0/110                  124/140
 // so the line is drawn at 2^17 multiply-adds a digit (9 targets at three sources
-// and 2^12, 6 at two and 2^13, 8 at one and 2^14).
+// and 2^12, 6 at two and 2^13, 8 at one and 2^14).  The smallest sets of the larger
+// rings fall below it too.  For a lone switch of theirs the sign changes from set
+// to set, as the places of the small launches' blocks do; from four jobs on the
+// CUDA cores win in all of them (1, 4 and 24 jobs):
+//   3, 1, 3     2^15: 71.8/73.9  111/97    309/253
+//   2, 1, 2     2^15: 66.2/76.3  97.3/79.8 225/174     2^16: 73.5/65.6  123/112   396/308
+//   1, 1, 1     2^16: 66.6/75.1  97.0/87.2 265/190     2^17: 93.8/79.2  142/124   487/364
 inline bool bconv_tc_chosen(const ks_params *P, int nsrc, int ntgt)
 {
     if (P->bconv_tensor >= 0) return P->bconv_tensor != 0;

@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(BC_THREADS, 4) k_bconv_up(Tables T, BUpJobs bj
 int launch_bconv_up(const Tables &T, const BUpJobs &b, cudaStream_t st)
 {
     if (b.n == 0) return KS_OK;
-    if (T.up_tc && bconv_tc_supported(T, T.alpha)) return launch_bconv_up_tc(T, b, T.up_tc, T.up_tc_lvl, st);
+    if (T.up_tc && bconv_tc_supported(T, T.alpha)) return launch_bconv_up_tc(T, b, st);
     const int span = bup_span(T, b);
     if (span <= 0) return KS_OK;
     const size_t N = (size_t)1 << T.logN;
@@ -810,7 +810,7 @@ int launch_bconv_down(const Tables &T, const BDnJobs &b, cudaStream_t st)
     for (int i = 0; i < b.n; ++i)
         ranged = ranged || b.job[i].i_begin != 0 || (b.job[i].i_end >= 0 && b.job[i].i_end != b.job[i].nact) ||
                  b.job[i].w != nullptr;
-    if (!ranged && T.dn_tc && bconv_tc_supported(T, T.kp)) return launch_bconv_down_tc(T, b, T.dn_tc, st);
+    if (!ranged && T.dn_tc && bconv_tc_supported(T, T.kp)) return launch_bconv_down_tc(T, b, st);
     int span = 0;
     for (int i = 0; i < b.n; ++i)
         span = std::max(span, (b.job[i].i_end < 0 ? b.job[i].nact : b.job[i].i_end) - b.job[i].i_begin);

@@ -108,8 +108,8 @@ int launch_inv_col(const Tables &T, const LimbMaps &m, bool scale_by_ninv, cudaS
 
 // ModUp P2.  Job: digit j (all active digits, or only jsel >= 0) converts its
 // canonical coefficient-form towers y[lo..hi) to the towers of D_l with
-// compact index in [t_begin, t_end) outside the digit; output lazy in
-// [0, 2r) at D + j'*dstride + (t - t_base)*N, j' = j (or 0 with jsel).
+// compact index in [t_begin, t_end) outside the digit; output lazy,
+// below 4r, at D + j'*dstride + (t - t_base)*N, j' = j (or 0 with jsel).
 struct BUpJob {
     const u64 *y;
     u64 *D;
@@ -128,7 +128,7 @@ int bup_span(const Tables &T, const BUpJobs &b);
 int launch_bconv_up(const Tables &T, const BUpJobs &b, cudaStream_t st);
 
 // ModDown P2: w = cp rows [nact, nact+K) of each polynomial (canonical,
-// coefficient form) -> v[x][i] = sum_k w_k * p_k^-1 mod q_i, lazy [0, 2q).
+// coefficient form) -> v[x][i] = sum_k w_k * p_k^-1 mod q_i, lazy, below 4q.
 struct BDnJob {
     const u64 *cp;
     size_t cp_stride;
@@ -155,8 +155,8 @@ int launch_bconv_down(const Tables &T, const BDnJobs &b, cudaStream_t st);
 // CUDA-core kernels; used by launch_bconv_up/down when the tables are present
 // and the shape is supported (at most 18 or 36 sources, N a multiple of 128).
 bool bconv_tc_supported(const Tables &T, int nsrc);
-int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, const uint4 *slabs, const int *slab_lvl, cudaStream_t st);
-int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, const uint4 *slabs, cudaStream_t st);
+int launch_bconv_up_tc(const Tables &T, const BUpJobs &b, cudaStream_t st);
+int launch_bconv_down_tc(const Tables &T, const BDnJobs &b, cudaStream_t st);
 // K blocks of 64 slice columns for nsrc sources: one up to 9, two up to 18, two
 // tiles of two blocks up to 36 (with the folding epilogue only: tc_pm_b != 0).
 inline int tc_kblocks(int nsrc) { return nsrc <= 9 ? 1 : nsrc <= 18 ? 2 : 4; }
