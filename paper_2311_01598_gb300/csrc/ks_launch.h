@@ -256,6 +256,8 @@ int launch_oc_tower(const Tables &T, const OcJobs &oj, cudaStream_t st);
 // combine kernels (each key word read once per group of jobs); otherwise
 // every job streams its own key limbs.
 int launch_oc(const Tables &T, int njobs, const OcJob *jobs, int variant, cudaStream_t st, bool share_keys = false);
+// The variant whose launches a group runs (full_keys: none of its keys is compressed).
+int oc_variant_run(const Tables &T, bool full_keys, int variant);
 // Rotations (at most kMaxBatch, one level) sharing the raised digits.
 int launch_oc_hoisted(const Tables &T, int n, const OcJob *jobs, cudaStream_t st);
 

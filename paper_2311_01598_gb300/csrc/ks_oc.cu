@@ -842,18 +842,24 @@ static int launch_oc_sections(const Tables &T, int n, const OcJob *jobs, int var
     return oc_rows(T, oj, false, st);
 }
 
+// The tower kernel needs a ring degree with a cluster geometry, and it and the
+// fused row kernels read the key's a half from memory; other launch groups, and
+// the split variant, run the whole-basis launches (same result).  The split
+// variant's own form converted and transformed the digits for each section
+// apart: one launch more, the source tiles built twice; slower in all 16 measured
+// shapes (N = 2^11..2^17, 1 to 64 jobs), by 0.4% (N = 2^17, 4 jobs) to 17% (N =
+// 2^13, 16 jobs).
+int oc_variant_run(const Tables &T, bool full_keys, int variant)
+{
+    if (variant == KS_OC_SPLIT || !full_keys || (variant == KS_OC_TOWER && !oc_tower_supported(T))) return KS_OC_WHOLE;
+    return variant;
+}
+
 int launch_oc(const Tables &T, int njobs, const OcJob *jobs, int variant, cudaStream_t st, bool share_keys)
 {
-    // The tower kernel needs a ring degree with a cluster geometry, and it and
-    // the fused row kernels read the key's a half from memory; other launch
-    // groups, and the split variant, run the whole-basis launches (same
-    // result).  The split variant's own form converted and transformed the
-    // digits for each section apart: one launch more, the source tiles built
-    // twice; slower in all 16 measured shapes (N = 2^11..2^17, 1 to 64 jobs), by
-    // 0.4% (N = 2^17, 4 jobs) to 17% (N = 2^13, 16 jobs).
     bool full = true;
     for (int i = 0; i < njobs; ++i) full = full && !jobs[i].key.comp;
-    if (variant == KS_OC_SPLIT || !full || (variant == KS_OC_TOWER && !oc_tower_supported(T))) variant = KS_OC_WHOLE;
+    variant = oc_variant_run(T, full, variant);
     for (int i0 = 0; i0 < njobs; i0 += kMaxBatch) {
         const int n = std::min(kMaxBatch, njobs - i0);
         const int rc = variant == KS_OC_WHOLE ? launch_oc_whole(T, n, jobs + i0, share_keys, st)

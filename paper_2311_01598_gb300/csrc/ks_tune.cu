@@ -32,6 +32,28 @@ static std::vector<ks_schedule> candidates()
     return c;
 }
 
+// For each candidate the one whose launches it runs for these jobs (-1: its own).
+// Such twins are not timed apart: the pick between them would be noise, and the
+// cache hands it on to batches of the same signature for which they differ (a
+// batch of compressed keys cached the fused variant, which it runs as whole
+// basis; host batches of 8 full keys then ran fused: 1241 -> 1461 us a call).
+static std::vector<int> twins(const ks_params *P, uint32_t n, const ks_job *jobs, const std::vector<ks_schedule> &c)
+{
+    bool any_full = false;  // a batch of both kinds runs each launch group by its own keys
+    for (uint32_t i = 0; i < n; ++i) any_full = any_full || !jobs[i].key->compressed;
+    std::vector<int> t(c.size(), -1);
+    for (size_t i = 0; i < c.size(); ++i) {
+        if (c[i].dataflow != KS_OC) continue;
+        ks_schedule s = c[i];
+        s.oc_variant = oc_variant_run(P->tables, any_full, s.oc_variant);
+        if (s.oc_variant == c[i].oc_variant) continue;
+        for (size_t k = 0; k < c.size(); ++k)
+            if (c[k].dataflow == KS_OC && c[k].oc_variant == s.oc_variant && c[k].chunk == s.chunk && c[k].order == s.order)
+                t[i] = (int)k;
+    }
+    return t;
+}
+
 // Relative timing difference below which stage 1 treats schedules as tied.
 constexpr float kTieFrac = 0.003f;
 
@@ -229,19 +251,23 @@ int ks_autotune(ks_params *P, uint32_t n, const ks_job *jobs, uint32_t reps, ks_
     // stage 1: structure
     std::vector<ks_schedule> c = candidates();
     std::vector<float> ms(c.size(), 1e30f);
+    const std::vector<int> twin = twins(P, n, jobs, c);
     float best_ms = 1e30f;
     for (size_t i = 0; i < c.size() && rc == KS_OK; ++i) {
+        if (twin[i] >= 0) continue;
         rc = time_schedule(P, n, jobs, c[i], reps, st, e0, e1, &ms[i]);
-        if (rc != KS_OK) break;
-        if (i < max && ms_out) ms_out[i] = ms[i];
         best_ms = std::min(best_ms, ms[i]);
+    }
+    for (size_t i = 0; i < c.size() && rc == KS_OK; ++i) {
+        if (twin[i] >= 0) ms[i] = ms[twin[i]];
+        if (i < max && ms_out) ms_out[i] = ms[i];
     }
     // Among the schedules within kTieFrac of the fastest (timing noise),
     // the one with the largest launch groups: the same time in fewer launches.
     ks_schedule base = c[0];
     int base_chunk = -1;
     for (size_t i = 0; i < c.size(); ++i)
-        if (ms[i] <= best_ms * (1.0f + kTieFrac) && c[i].chunk > base_chunk) {
+        if (twin[i] < 0 && ms[i] <= best_ms * (1.0f + kTieFrac) && c[i].chunk > base_chunk) {
             base = c[i];
             base_chunk = c[i].chunk;
         }
