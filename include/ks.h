@@ -351,7 +351,10 @@ int ks_tune_candidates(const ks_params *params, uint32_t max, ks_schedule *out, 
  * are overwritten -- every schedule writes the same values):
  *   1. every structural candidate (ks_tune_candidates); ms_out[i] gets
  *      candidate i's time in ms (max entries); of the candidates within
- *      0.3% of the fastest, the one with the largest launch group wins;
+ *      0.3% of the fastest, the one with the largest launch group wins.  A
+ *      candidate that runs another's launches for these jobs (oc_variant 1;
+ *      0 and 3 for compressed keys; 3 without a cluster geometry) gets that
+ *      one's time and is not picked;
  *   2. the fastest structure under each implementation pair (ntt, bconv) in
  *      {(0,1), (1,1), (0,0), (1,0)} (ks_autotune_impl); when max leaves room
  *      for them, ms_out[n_candidates + k] gets pair k's time.
@@ -566,11 +569,12 @@ int ks_server_run_trace(ks_server *server, uint32_t n, const ks_request *reqs, c
 
 /* Arithmetic ceilings of the current GPU for the two inner loops of key
  * switching, measured with register-only loops of the same device code:
- * forward NTT butterflies per second and base-conversion multiply-
- * accumulates per second.  iters: loop trips per thread (e.g. 4096). */
+ * forward NTT butterflies per second (of primes just below a power of two, as
+ * the default rule gives) and base-conversion multiply-accumulates per
+ * second.  iters: loop trips per thread (e.g. 4096). */
 int ks_probe_alu(int iters, double *bfly_per_s, double *mac_per_s);
 
-/* The same ceiling for the inverse (Harvey) NTT butterfly, inverse
+/* The same ceiling for the inverse NTT butterfly of those primes, inverse
  * butterflies per second (the ceiling of the inverse NTT passes). */
 int ks_probe_inv_bfly(int iters, double *inv_bfly_per_s);
 
